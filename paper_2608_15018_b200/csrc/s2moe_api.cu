@@ -15,6 +15,7 @@
 #include "ffn_stream.cuh"
 #include "expand.cuh"
 #include "ffn_tc.cuh"
+#include "ffn_rows.cuh"
 #include "route.cuh"
 #include "layer_tc.cuh"
 
@@ -49,6 +50,10 @@ struct s2moe_ctx {
     int bf16_kg2_from = 2;                // batches of this many tokens and more: two k-tiles per ring stage (bf16)
     float *pre = nullptr;                 // plan 3: fp32 pre-activations [gate|up][slot][f]
     std::vector<TcMaps> tc_maps;          // plan 3: per layer, weight maps filled at create
+    std::vector<RwMaps> rw_maps;          // plan 3 with bf16 weights: the same for ffn_rows_kernel
+    std::vector<int> rw_mode;             // per layer: RwArgs::mode
+    RwMaps rw_act{};                      // its maps 11..18 (the workspace's activations) for batches of rw_act_B tokens
+    int rw_act_B = 0;
     void *encode_tiled = nullptr;         // cuTensorMapEncodeTiled, looked up through the runtime
     int last_cuda = 0;
     int64_t launches = 0;
@@ -388,14 +393,14 @@ bool make_map_plain(const s2moe_ctx *ctx, CUtensorMap *out, const void *base, ui
 }
 
 // 3-D bf16 tensor {cols, rows, 2}: the hi array and, `plane_bytes` further, the lo array of the
-// activations; box = 64 columns x 8 rows x both planes
+// activations; box = 64 columns x box_rows rows x both planes
 bool make_map_hilo(const s2moe_ctx *ctx, CUtensorMap *out, const void *base, uint64_t rows, uint64_t cols,
-                   uint64_t plane_bytes)
+                   uint64_t plane_bytes, uint32_t box_rows = 8)
 {
     if (!ctx->encode_tiled || !base || rows == 0) return false;
     const cuuint64_t dims[3] = {cols, rows, 2};
     const cuuint64_t strides[2] = {cols * 2, plane_bytes};
-    const cuuint32_t box[3] = {64, 8, 2};
+    const cuuint32_t box[3] = {64, box_rows, 2};
     const cuuint32_t estr[3] = {1, 1, 1};
     return ((EncodeTiledFn)ctx->encode_tiled)(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(base), dims,
                                               strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -450,6 +455,51 @@ bool make_map_hilo_ktiles(const s2moe_ctx *ctx, CUtensorMap *out, const void *ba
                                               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Maps of bf16 W_gate and W_up (same shape) for ffn_rows_kernel.  As one 5-D tensor {64 columns, 8 rows,
+// k-tiles, matrix, groups of 8 rows}, boxes of 1, 2 and 4 groups and two k-tiles land as
+// [group][matrix][k-tile][8 rows][128 bytes]; the matrix of lower address comes first (*swap: W_up).
+// Matrices that a 40-bit stride does not join, or that are one and the same, get a map each (*apart).
+bool make_gateup_maps(const s2moe_ctx *ctx, CUtensorMap *out, const void *gate, const void *up, uint64_t rows, uint64_t cols,
+                      bool *swap, bool *apart)
+{
+    if (!ctx->encode_tiled || !gate || !up || rows == 0 || rows % 8 || cols % 64) return false;
+    const uintptr_t a = (uintptr_t)gate, b = (uintptr_t)up;
+    const uintptr_t diff = a < b ? b - a : a - b;
+    *apart = diff == 0 || diff >= (1ull << 40);
+    *swap = !*apart && b < a;
+    if (*apart)
+        return make_map_ktiles(ctx, &out[0], gate, rows, cols, 8, 2) && make_map_ktiles(ctx, &out[1], up, rows, cols, 8, 2);
+    const cuuint64_t dims[5] = {64, 8, cols / 64, 2, rows / 8};
+    const cuuint64_t strides[4] = {cols * 2, 128, diff, cols * 16};
+    const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+    for (int i = 0; i < 3; ++i) {
+        const cuuint32_t box[5] = {64, 8, 2, 2, 1u << i};
+        if (((EncodeTiledFn)ctx->encode_tiled)(&out[i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, (void *)(a < b ? a : b), dims, strides, box,
+                                               estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                                               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return false;
+    }
+    return true;
+}
+
+// the maps of ffn_rows_kernel that only depend on the layer's weights, and RwArgs::mode
+bool make_rows_maps(const s2moe_ctx *ctx, const LayerPtrs &lp, uint64_t n_w_experts, RwMaps *m, int *mode)
+{
+    const Shape &sh = ctx->shape;
+    bool swap = false, apart = false;
+    if (!make_gateup_maps(ctx, &m->m[0], lp.w_gate, lp.w_up, n_w_experts * sh.f, (uint64_t)sh.d, &swap, &apart)) return false;
+    *mode = (swap ? 1 : 0) | (apart ? 4 : 0);
+    if (sh.n_sh) {
+        if (!make_gateup_maps(ctx, &m->m[3], lp.sh_gate, lp.sh_up, (uint64_t)sh.n_sh * sh.f_sh, (uint64_t)sh.d, &swap, &apart)) return false;
+        *mode |= (swap ? 2 : 0) | (apart ? 8 : 0);
+    }
+    for (int h = 0; h < 2; ++h) {
+        if (!make_map(ctx, &m->m[6 + 2 * h], lp.w_down, n_w_experts * sh.d, (uint64_t)sh.f, h ? 64 : 128)) return false;
+        if (sh.n_sh && !make_map(ctx, &m->m[7 + 2 * h], lp.sh_down, (uint64_t)sh.n_sh * sh.d, (uint64_t)sh.f_sh, h ? 64 : 128)) return false;
+    }
+    return true;
+}
+
 // The plan a batch of B tokens runs with: the streaming kernel when it is allowed and its
 // shared-memory layout fits, else the CUDA-core kernels; 0 when plan 2 was demanded and does not fit.
 int plan_for(const s2moe_ctx *ctx, int B, StPlan *out)
@@ -466,7 +516,10 @@ int plan_for(const s2moe_ctx *ctx, int B, StPlan *out)
         const fused::TcPlan tp = fused::tc_make_plan(s0, B, ctx->n_sm, B * s0.k + s0.n_sh * B);
         return tp.feasible ? 4 : 0;
     }
-    if (want == 0 || want == 3) {
+    if ((want == 0 || want == 3) && s0.weight_dtype == DT_BF16) {
+        if (!ctx->rw_maps.empty() && rw_make_plan(s0, B, ctx->n_sm, false).feasible) return 3;
+        if (want == 3) return 0;
+    } else if (want == 0 || want == 3) {
         const TcPlan tp = tc_make_plan(s0, B, ctx->n_sm, B * s0.k + s0.n_sh * B, B >= ctx->bf16_kg2_from ? 2 : 1);
         if (tp.feasible && !ctx->tc_maps.empty()) return 3;
         if (want == 3) return 0;
@@ -537,8 +590,9 @@ int verify_one(s2moe_ctx *ctx, int layer, int B, const void *hidden, const float
     // experts the routing kernel announces before it (not with offloaded experts: their weights are
     // fetched between the two kernels)
     const bool want_early = plan == 3 && ctx->early_start && ctx->use_pdl && !ctx->offload && sh.weight_dtype == DT_BF16;
-    TcPlan tp3 = tc_make_plan(sh, B, ctx->n_sm, B * sh.k + sh.n_sh * B, B >= ctx->bf16_kg2_from ? 2 : 1, want_early);
-    if (sh.weight_dtype == DT_BF16 && ctx->wave_split[0] > 0) { tp3.split[0] = ctx->wave_split[0]; tp3.split[1] = ctx->wave_split[1]; }
+    const bool rows3 = plan == 3 && sh.weight_dtype == DT_BF16;
+    const RwPlan rp = rows3 ? rw_make_plan(sh, B, ctx->n_sm, want_early) : RwPlan{};
+    const TcPlan tp3 = plan == 3 && !rows3 ? tc_make_plan(sh, B, ctx->n_sm, B * sh.k + sh.n_sh * B) : TcPlan{};
     // what the FFN kernels accumulate into is cleared by the routing kernel's blocks
     ZeroList zl{};
     zl.ptr[0] = out;
@@ -546,7 +600,7 @@ int verify_one(s2moe_ctx *ctx, int layer, int B, const void *hidden, const float
     if (plan == 3 || plan == 4) {
         const size_t used = (size_t)B * sh.k * sh.f + (size_t)sh.n_sh * B * sh.f_sh;
         zl.ptr[1] = ctx->pre;
-        zl.n16[1] = used * 2 * sizeof(float) / 16;
+        zl.n16[1] = rows3 ? 0 : used * 2 * sizeof(float) / 16;
         zl.ptr[2] = ctx->ws.sync + (kTcReady - 8);      // the hand-over counters of the two waves
         zl.n16[2] = 8 * sizeof(int32_t) / 16;
         if (sh.weight_dtype == DT_Q4B32) {
@@ -555,7 +609,7 @@ int verify_one(s2moe_ctx *ctx, int layer, int B, const void *hidden, const float
             zl.perm_n16 = (size_t)B * sh.d * 2 / 16;
         }
     }
-    if (plan == 3 && tp3.early) {
+    if (rows3 && rp.early) {
         // a token's first expert by original logit stays selected for alpha < 1 (see gating_block);
         // otherwise only the shared experts start early
         const bool bias_on = sh.alpha > 0.0 && sh.cap < sh.E && sh.k < sh.E;
@@ -566,7 +620,30 @@ int verify_one(s2moe_ctx *ctx, int layer, int B, const void *hidden, const float
         const int rc = fetch_experts(ctx, layer, st);
         if (rc != S2MOE_OK) return rc;
     }
-    if (plan == 3 || plan == 4) {
+    if (rows3) {
+        RwMaps maps = ctx->rw_maps[layer];
+        const size_t n_routed = (size_t)B * sh.k;
+        if (ctx->rw_act_B != B) {
+            const uint64_t plane = (uint64_t)((const uint8_t *)ctx->act_lo - (const uint8_t *)ctx->act_hi);
+            ctx->rw_act_B = 0;
+            for (int i = 0; i < 4; ++i) {
+                if (!make_map_hilo(ctx, &ctx->rw_act.m[11 + i], ctx->act_hi, n_routed, (uint64_t)sh.f, plane, 8u << i)) return S2MOE_ECUDA;
+                if (sh.n_sh && !make_map_hilo(ctx, &ctx->rw_act.m[15 + i], ctx->act_hi + n_routed * sh.f, (uint64_t)sh.n_sh * B,
+                                              (uint64_t)sh.f_sh, plane, 8u << i))
+                    return S2MOE_ECUDA;
+            }
+            ctx->rw_act_B = B;
+        }
+        for (int i = 11; i < 19; ++i) maps.m[i] = ctx->rw_act.m[i];
+        if (!make_map_ktiles(ctx, &maps.m[10], hidden, (uint64_t)B, (uint64_t)sh.d, (uint32_t)(rp.x_bytes ? rp.xr : rp.n1), rp.x_bytes ? 8 : 2))
+            return S2MOE_ECUDA;
+        RwArgs a;
+        a.sh = sh; a.ws = ctx->ws; a.plan = rp; a.y = out; a.act_hi = ctx->act_hi; a.act_lo = ctx->act_lo; a.B = B;
+        a.mode = ctx->rw_mode[layer];
+        LaunchScope scope(ctx, KC_TC, st);
+        cudaLaunchConfig_t lc = pdl_config(ctx, rp.n_cta, kRwThreads, rp.smem_bytes, st, rp.early != 0);
+        cudaLaunchKernelEx(&lc, ffn_rows_kernel, maps, a);
+    } else if (plan == 3 || plan == 4) {
 
         const fused::TcPlan tp4 = plan == 4 ? fused::tc_make_plan(sh, B, ctx->n_sm, B * sh.k + sh.n_sh * B) : fused::TcPlan{};
         const bool q4 = plan == 4 ? tp4.q4 != 0 : tp3.q4 != 0;
@@ -775,7 +852,8 @@ int create_impl(const s2moe_config *config, const s2moe_layer_weights *layers, i
             ctx->encode_tiled = fn;
             ctx->tc_maps.resize(config->n_layers);
             const bool q4 = sh.weight_dtype == DT_Q4B32;
-            bool ok = cudaFuncSetAttribute(ffn_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcMaxSmem) == cudaSuccess &&
+            bool ok = cudaFuncSetAttribute(ffn_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kRwMaxSmem) == cudaSuccess &&
+                      cudaFuncSetAttribute(ffn_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcMaxSmem) == cudaSuccess &&
                       cudaFuncSetAttribute(ffn_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcMaxSmem) == cudaSuccess &&
                       cudaFuncSetAttribute(fused::layer_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcMaxSmem) == cudaSuccess &&
                       cudaFuncSetAttribute(fused::layer_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcMaxSmem) == cudaSuccess;
@@ -838,6 +916,16 @@ int create_impl(const s2moe_config *config, const s2moe_layer_weights *layers, i
                 }
             }
             if (!ok) ctx->tc_maps.clear();
+            if (ok && !q4) {
+                ctx->rw_maps.resize(config->n_layers);
+                ctx->rw_mode.resize(config->n_layers);
+                bool rok = true;
+                for (int l = 0; l < config->n_layers && rok; ++l) {
+                    std::memset(&ctx->rw_maps[l], 0, sizeof(RwMaps));
+                    rok = make_rows_maps(ctx, ctx->layers[l], (uint64_t)n_w_experts, &ctx->rw_maps[l], &ctx->rw_mode[l]);
+                }
+                if (!rok) ctx->rw_maps.clear();
+            }
         }
     }
     ctx->act_hi = (__nv_bfloat16 *)(base + o_ahi); ctx->act_lo = (__nv_bfloat16 *)(base + o_alo);

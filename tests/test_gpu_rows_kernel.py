@@ -1,0 +1,53 @@
+"""The bf16 expert kernel that cuts the first projection by rows (kernel plan 3) at the sizes where it can
+go wrong: widths that are no multiple of a task, row block or k-tile, one k-tile, a last row block of 64
+rows, token counts around the padding steps, few and many experts, and the layouts of W_gate and W_up in
+memory (ascending, descending, the same matrix twice).  Tolerance: the library's own for bf16 weights."""
+import pytest
+import torch
+
+from gpu_util import check_outputs, run_case
+from paper_2608_15018_b200 import binding, workloads
+from paper_2608_15018_b200.workloads import CONFIGS
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("d,f,f_sh", [(64, 32, 32), (128, 96, 160), (192, 1056, 0), (576, 224, 2080), (1152, 544, 64)])
+@pytest.mark.parametrize("B", [1, 8, 9, 17, 33, 64])
+def test_ragged_sizes(d, f, f_sh, B):
+    wl = CONFIGS["cfg3"].with_(d_model=d, d_ff=f, d_ff_shared=f_sh, n_shared=2 if f_sh else 0, shared_gate=bool(f_sh),
+                               n_experts=24, top_k=3, cap=6, seed=B)
+    rep, _ = run_case(wl, n_tokens=B, plan=3)
+    assert rep.plan == 3 and rep.tokens_checked == B
+
+
+@pytest.mark.parametrize("E,k,B", [(1, 1, 1), (2, 1, 64), (256, 16, 5), (200, 2, 40)])
+def test_few_and_many_experts(E, k, B):
+    wl = CONFIGS["cfg2"].with_(d_model=256, d_ff=320, n_experts=E, top_k=k, cap=min(E, 2 * k), sigma=1.0, seed=E)
+    rep, _ = run_case(wl, n_tokens=B, plan=3)
+    assert rep.plan == 3 and rep.tokens_checked == B
+
+
+@pytest.mark.parametrize("layout", ["up_first", "tied"])
+def test_layouts_of_gate_and_up(layout):
+    wl = CONFIGS["cfg3"].with_(d_model=320, d_ff=352, d_ff_shared=416, n_experts=10, top_k=2, cap=4, n_layers=1)
+    T = workloads.layer_weights(wl, 0, "cuda")
+    for g, u in (("w_gate", "w_up"), ("sh_gate", "sh_up")):
+        if layout == "tied":
+            T[u] = T[g]
+        else:
+            both = torch.stack([T[u], T[g]])
+            T[u], T[g] = both[0], both[1]
+            assert T[u].data_ptr() < T[g].data_ptr()
+    H = workloads.hidden_states(wl, 0, 11, device="cuda")
+    with binding.S2MoE(binding.Config.from_workload(wl, n_layers=1, kernel_plan=3), [T]) as m:
+        o = m.verify_layer(0, H)
+        assert m.device_status() == 0
+    check_outputs(wl, T, H, None, o)
+
+
+def test_large_expert_count_and_width_still_run():
+    """256 experts of a wide layer: the task table of a CTA is at its largest."""
+    wl = CONFIGS["cfg2"].with_(d_model=64, d_ff=14336, n_experts=256, top_k=16, cap=256, sigma=1.0, n_layers=1)
+    rep, _ = run_case(wl, n_tokens=64, plan=3, tok_list=list(range(0, 64, 9)))
+    assert rep.plan == 3
