@@ -1453,10 +1453,25 @@ int s2moe_adaptive_expand(int32_t n_cand, int32_t n_layers, int32_t n_experts, c
     if (!parent || !p_tok || !masks || !admitted || !order || !n_admitted) return S2MOE_EINVAL;
     const int lw = n_layers * ((n_experts + 63) / 64);
     if (n_cand > kExpandMaxCand || lw > kExpandMaxWords) return S2MOE_ERANGE;
-    const int threads = ((n_cand + 31) / 32) * 32;
-    adaptive_expand_kernel<<<1, threads, 0, (cudaStream_t)cuda_stream>>>(
-        n_cand, lw, parent, p_tok, reinterpret_cast<const unsigned long long *>(masks), c_draft, t_ar, t_exp,
-        admitted, order, n_admitted, reinterpret_cast<unsigned long long *>(union_out));
+    // as many threads per candidate as it has words, within the block's limit
+    const int np = (n_cand + 31) / 32 * 32;
+    int parts = kExpandThreads / np;
+    if (parts > lw) parts = lw;
+    const int threads = np * parts;
+    const size_t rows = sizeof(uint64_t) * (size_t)(n_cand | 1) * lw;
+    const unsigned long long *mk = reinterpret_cast<const unsigned long long *>(masks);
+    unsigned long long *un = reinterpret_cast<unsigned long long *>(union_out);
+    cudaStream_t st = (cudaStream_t)cuda_stream;
+    if (rows <= (size_t)kExpandMaxSmem) {
+        if (rows > 32 * 1024 && cudaFuncSetAttribute(adaptive_expand_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                     kExpandMaxSmem) != cudaSuccess)
+            return S2MOE_ECUDA;
+        adaptive_expand_kernel<true><<<1, threads, rows, st>>>(n_cand, lw, parent, p_tok, mk, c_draft, t_ar, t_exp, admitted,
+                                                               order, n_admitted, un);
+    } else {
+        adaptive_expand_kernel<false><<<1, threads, 0, st>>>(n_cand, lw, parent, p_tok, mk, c_draft, t_ar, t_exp, admitted,
+                                                             order, n_admitted, un);
+    }
     return cudaGetLastError() == cudaSuccess ? S2MOE_OK : S2MOE_ECUDA;
 }
 
