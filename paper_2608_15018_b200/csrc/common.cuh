@@ -14,6 +14,7 @@ constexpr int kMaxTokens = 64;
 constexpr int kMaxExperts = 256;
 constexpr int kMaxTopK = 16;
 constexpr int kMaxShared = 4;
+constexpr int kEarlyWords = kMaxExperts / 32;   // words of one list of Workspace::early
 
 enum : int { DT_F32 = 0, DT_BF16 = 1, DT_Q4B32 = 2 };
 
@@ -61,9 +62,11 @@ struct Workspace {
     unsigned long long *tokmask;   // [E + n_sh] bit b set: token b is bucketed to the group
     uint4 *gtab;           // [n_active][2] {group, tokens, first slot, 0}, {mask lo, mask hi, 0, 0}: the
                            // active groups in their final form, or NULL when nobody reads it
-    int32_t *early;        // 8 words of 64 bits, {tag << 32 | bits of 32 experts}: the experts whose first projection
-                           // may start before the gating has ended, published by the routing kernel (see
-                           // gating_block), or NULL
+    unsigned long long *early;   // kEarlyWords + 1 words, or NULL.  {1 << 32 | bits of 32 experts}: the selected experts, as soon as
+                           // they are known; the last word: {1 << 32 | value of the arrival counter when all routing
+                           // blocks of the launch have arrived}, once the launch's inputs may be read
+    float *gsum;           // [E] sum over the tokens of w_b * l_{b,e} in float (the order in which experts are most likely to
+                           // be selected), zero between the layers
     const int32_t *slot_of;  // [E] device slot that holds each routed expert's weights (expert offloading), or
                              // NULL: every expert is resident at its own index
 };

@@ -26,14 +26,20 @@
 // a CTA arrive (release) when their activations of the wave are stored, a watcher warp polls it and
 // opens the wave's token tiles to the producer.
 //
-// Early start: see route.cuh.  The kernel is resident while the gating still runs.  It streams the
-// first projection of the shared experts at once, that of the experts the routing kernel announces
-// as soon as the list is out, and the rest when warps 6..9 have built the tables from the finished
-// gating.  Early results wait in tensor memory (up to 16 accumulators) for the token lists.
+// Early start: see route.cuh.  The kernel is resident while the routing kernel still runs (its blocks
+// are small enough to share the SMs), even before the layer in front has ended.  It streams the weights
+// of the shared experts' first projection at once; as soon as the router's logits are there, and beside
+// the gating, the first projection of the top_k experts of largest aggregated importance g_e (Eq. 4),
+// which are nearly always selected: over the shapes of the workloads, 1 to 64 tokens, noise 0.1 to 1, with
+// and without the bias, at most 0.1 of them is not.  An expert that is not has been read for nothing: it
+// gets no tokens and no second projection.  The first projection of all others follows when the
+// selection is known, the second projection when warps 6..9 have built the tables from the finished
+// gating.  Early results wait in tensor memory (up to 16 accumulators) for the token lists.  Nothing but
+// weights is read before the routing kernel says that its own inputs are there.
 //
 // Warp roles (352 threads): 0 TMA producer, 1 MMA issuer (owns the TMEM allocation), 2..5 and 6..9 two
-// epilogue sets that take alternate tasks (6..9 build the tables first), 10 watcher (early list, then
-// the wave counters).  The single-thread roles run in a thread chosen by elect.sync: measured on
+// epilogue sets that take alternate tasks (6..9 build the tables first), 10 watcher (early experts,
+// selection and the tasks of the first projection, then the wave counters).  The single-thread roles run in a thread chosen by elect.sync: measured on
 // B200, an MMA of 128 x 16 x 16 then issues every 39 cycles against 55 from a `lane == 0` branch
 // (the tensor core itself needs 32 to read the 4 KiB of weights), which is why one issuer is enough.
 // Even and odd k-tiles go to two accumulators that the epilogue adds: the tensor core truncates when
@@ -53,10 +59,12 @@ constexpr int kRwMaxStages = 8;
 constexpr int kRwMaxAcc = 16;
 constexpr int kRwWBytes = 32768;               // weight bytes of a stage: 8 row pairs x 2 k-tiles, or a 128-row block x 2 k-tiles
 constexpr int kRwMaxTasks = 1024;
-constexpr int kRwMaxSmem = 232448 - 2048;      // dynamic shared memory; the rest is static (barriers, lot table)
+constexpr int kRwStaticSmem = 2048;            // static shared memory at most (barriers, lots, ids)
+constexpr int kRwMaxSmem = 232448 - kRwStaticSmem;
 constexpr int kRwSets = 2;                     // epilogue sets
 constexpr int kRwMaxWaves = 4;
-constexpr int kRwLots = 2 * kRwMaxWaves + 1;   // first projection of every wave; second: wave 0, shared experts, other waves
+constexpr int kRwLots2 = kRwMaxWaves + 1;      // lots of the second projection: wave 0, shared experts, other waves
+constexpr int kRwLevels = 3;                   // task lists: shared experts, early list, all experts, second projection
 
 // division of 0 <= n by a launch constant: n / d == umulhi(n, m) while n * d < 2^32 (checked on the host)
 struct RwDiv {
@@ -76,7 +84,7 @@ struct RwPlan {
     int max_tasks;
     int tab_bytes;
     int smem_bytes;
-    int early;
+    int early, n_early;
     int split16[kRwMaxWaves - 1];   // where waves 1, 2, 3 begin, in 16ths of the first projection (16: no such wave)
     int delta;           // second-projection units that weigh as much as one first-projection unit
     RwDiv gf, gs, tf, ts, kr, ks, rb, p;   // row groups and tasks of a routed / shared expert, P2 units of their row blocks, row blocks, CTAs
@@ -116,16 +124,16 @@ static_assert(sizeof(RwTask) == 32, "layout");
 // rows of the activation box that holds T tokens
 __host__ __device__ __forceinline__ int rw_tok_rows(int T) { return T <= 8 ? 8 : (T <= 16 ? 16 : (T <= 32 ? 32 : 64)); }
 
-inline RwPlan rw_make_plan(const Shape &sh, int B, int n_sm, bool early)
+// route_smem: shared memory of a routing block that is to share an SM with a CTA of this kernel (0: none does)
+inline RwPlan rw_make_plan(const Shape &sh, int B, int n_sm, bool early, int route_smem)
 {
     RwPlan p{};
     if (sh.weight_dtype != DT_BF16 || sh.act_dtype != DT_BF16 || sh.d % 64 || sh.f % 32 || (sh.n_sh && sh.f_sh % 32) || B > kMaxTokens)
         return p;
     const int G = sh.E + sh.n_sh, n_slots = B * sh.k + sh.n_sh * B;
-    // (early start: one CTA less than SMs, because the SM that runs the gating is taken until the
-    // routing kernel ends and its CTA would start last with a full share)
     p.early = early && n_sm > 1;
-    p.n_cta = p.early ? n_sm - 1 : n_sm;
+    // experts whose first projection starts before the gating (see the header comment)
+    p.n_early = p.early ? (sh.k < 4 ? (sh.k == 3 ? 2 : 1) : sh.k) : 0;
     p.n1 = (B + 15) & ~15;
     const int trows = rw_tok_rows(B);
     const int tok2 = 2 * 2 * trows * 128, tok1 = 2 * p.n1 * 128;
@@ -141,23 +149,34 @@ inline RwPlan rw_make_plan(const Shape &sh, int B, int n_sm, bool early)
     p.kr = rw_div_make((sh.f + 127) / 128);
     p.ks = rw_div_make(sh.n_sh ? (sh.f_sh + 127) / 128 : 1);
     p.rb = rw_div_make((sh.d + 127) / 128);
-    p.p = rw_div_make(p.n_cta);
     // tasks of a CTA at most: a share of n units in groups of g, m units per task, meets n / g + 2 groups,
     // and every group adds at most one ragged task to n / m whole ones
-    const long long P = p.n_cta, U = sh.E < (long long)B * sh.k ? sh.E : (long long)B * sh.k;
+    const long long P = n_sm - 1 > 0 ? n_sm - 1 : 1, U = sh.E < (long long)B * sh.k + p.n_early ? sh.E : (long long)B * sh.k + p.n_early;
     const long long n1r = U * p.gf.d, n1s = sh.n_sh ? (long long)sh.n_sh * p.gs.d : 0;
     const long long n2r = U * p.rb.d * p.kr.d, n2s = sh.n_sh ? (long long)sh.n_sh * p.rb.d * p.ks.d : 0;
     const long long tasks = n1r / P / 8 + n1r / P / p.gf.d + n1s / P / 8 + n1s / P / p.gs.d + n2r / P / p.kr.d + n2s / P / p.ks.d +
-                            4 * (kRwLots + 2);
+                            4 * (kRwMaxWaves + kRwLots2 + 2);
     if (tasks > kRwMaxTasks) return p;
     p.max_tasks = (int)tasks;
+    const int nk = sh.d / 64;
+    p.tab_bytes = ((int)sizeof(TcGroup) * (G + 1 + sh.n_sh) + 8 * n_slots + (int)sizeof(RwTask) * p.max_tasks + 1023) & ~1023;
+    // Early start: a routing block shares every SM with a CTA of this kernel if that leaves room for three
+    // stages (two blocks on an SM share 228 KiB, 1 KiB of it reserved for each).  If not, one CTA less than
+    // SMs: the SM that runs the gating is taken until the routing kernel ends, and its CTA would start
+    // last with a full share.
+    const int full = kRwMaxSmem - p.tab_bytes - 1024, shared = 228 * 1024 - 2048 - kRwStaticSmem - route_smem - p.tab_bytes - 1024;
+    const int x_res = ((nk + 7) & ~7) * (B <= 8 ? 8 : p.n1) * 128 + 1024, st_res = kRwWBytes + ((tok2 + 1023) & ~1023);
+    const int st_tok = kRwWBytes + (((tok1 > tok2 ? tok1 : tok2) + 1023) & ~1023);
+    const bool beside = p.early && route_smem > 0 &&
+                        ((shared - x_res) / st_res >= 3 || ((full - x_res) / st_res < 3 && shared / st_tok >= 3));
+    const int budget = beside ? shared : full;
+    p.n_cta = p.early && !beside ? n_sm - 1 : n_sm;
+    p.p = rw_div_make(p.n_cta);
     // exactness of the divisions above
     auto exact = [&](long long n, const RwDiv &v) { return (unsigned long long)n * v.d < 0x100000000ull; };
     if (!exact(n1r + P, p.gf) || !exact(n1s + P, p.gs) || !exact(n2r + P, p.kr) || !exact(n2s + P, p.ks) ||
         !exact(n2r + n2s + n1r + n1s + 64 * P, p.p) || !exact(n2r + n2s + P, p.rb))
         return p;
-    p.tab_bytes = ((int)sizeof(TcGroup) * (G + 1 + sh.n_sh) + 8 * n_slots + (int)sizeof(RwTask) * p.max_tasks + 1023) & ~1023;
-    const int nk = sh.d / 64, budget = kRwMaxSmem - p.tab_bytes - 1024;
     // Hidden states resident where at least three stages fit beside them; else their tiles travel
     // with the stages, one copy more and at most one chunk of two k-tiles per stage.  Measured, us per
     // layer, three stages with resident tiles / five without: DeepSeek-V2-Lite shape at 16 tokens 54.5 /
@@ -177,11 +196,11 @@ inline RwPlan rw_make_plan(const Shape &sh, int B, int n_sm, bool early)
         if (p.stages >= (res ? 3 : 2)) { p.feasible = 1; break; }
     }
     if (!p.feasible) return p;
-    // Two waves.  Measured, us per layer, wave 1 from 10/16 / waves 1 and 2 from 8/16 and 13/16: OLMoE shape
-    // at 8 tokens 46.9 / 45.7, one token 35.0 / 36.6, DeepSeek-V2-Lite shape at 16 tokens 54.5 / 55.3,
-    // Qwen1.5-MoE shape 46.7 / 47.5, 128 experts at 13 tokens 48.7 / 49.6.
-    p.split16[0] = 10;
-    p.split16[1] = 16;
+    // Three waves.  Measured, us per layer, waves 1 and 2 from 8/16 and 13/16 / wave 1 from 10/16: OLMoE shape
+    // at 8 tokens 41.3 / 43.2, one token 31.7 / 31.5, DeepSeek-V2-Lite shape at 16 tokens 53.0 / 53.4,
+    // Qwen1.5-MoE shape 43.8 / 44.3, 128 narrow experts at 13 tokens 42.9 / 42.9, 128 wide ones at 8 76.8 / 77.0.
+    p.split16[0] = 8;
+    p.split16[1] = 13;
     p.split16[2] = 16;
     p.delta = (sh.d + 512) / 1024;
     return p;
@@ -282,18 +301,21 @@ __device__ __forceinline__ void rw_seg_task(const RwSeg &s, const RwDiv &g, int 
     len = min(1 << m, have - (q << m));
 }
 
-__global__ void __launch_bounds__(kRwThreads, 1)
+// (bound of 1024 threads: at most 64 registers, so that a routing block of 512 threads x 80 registers fits beside it)
+__global__ void __launch_bounds__(1024, 1)
 ffn_rows_kernel(const __grid_constant__ RwMaps maps, const __grid_constant__ RwArgs p)
 {
     extern __shared__ __align__(1024) uint8_t rw_smem[];
     __shared__ __align__(8) uint64_t full_bar[kRwMaxStages], empty_bar[kRwMaxStages];
-    __shared__ __align__(8) uint64_t acc_full[kRwMaxAcc], acc_empty[kRwMaxAcc], x_bar, early_bar, tab_bar, ep_bar[kRwSets];
+    __shared__ __align__(8) uint64_t acc_full[kRwMaxAcc], acc_empty[kRwMaxAcc], x_bar, in_bar, lvl_bar[kRwLevels], ep_bar[kRwSets];
     __shared__ uint32_t s_tmem;
-    __shared__ int s_lim[3];                       // tasks known at the start, with the early list, with the tables
-    __shared__ int s_n_early, s_waves;
+    __shared__ int s_lim[kRwLevels + 1];           // tasks known at each level (kRwLevels)
+    __shared__ int s_n_bad, s_U, s_waves;          // early experts without tokens; experts in s_id; waves
+    __shared__ uint16_t s_id[kMaxExperts];         // routed experts in this kernel's order: the early ones, then the others, ascending
+    __shared__ uint8_t s_sel[kMaxExperts];         // the early ones that have tokens
     __shared__ volatile int s_ready[kRwMaxWaves];  // wave w's activations are written (set by the watcher)
-    __shared__ RwSeg s_lot[kRwLots];
-    __shared__ int s_lot_first[kRwLots + 1], s_bound[kRwMaxWaves + 1];   // first task of a lot; first routed group of a wave
+    __shared__ RwSeg s_lot[kRwMaxWaves], s_lot2[kRwLots2];
+    __shared__ int s_first[kRwMaxWaves + 1], s_first2[kRwLots2 + 1], s_bound[kRwMaxWaves + 1];   // first task of a lot; first routed group of a wave
 
     const Shape &sh = p.sh;
     const Workspace &ws = p.ws;
@@ -323,6 +345,8 @@ ffn_rows_kernel(const __grid_constant__ RwMaps maps, const __grid_constant__ RwA
         start = c * q + min(c, r);
         cnt = q + (c < r ? 1 : 0);
     };
+    // where a routed expert's weights lie (offloaded experts: a device slot)
+    auto weights_of = [&](int id) -> int { return ws.slot_of ? __ldg(&ws.slot_of[id]) : id; };
     auto make_p1 = [&](RwTask *t, int a, int expert, int in, int len, int shared, int wave) {
         t->flags = (shared << 1) | (wave << 2) | (len << 8);
         t->x0 = expert * (shared ? Gs : Gf) + in;
@@ -347,8 +371,8 @@ ffn_rows_kernel(const __grid_constant__ RwMaps maps, const __grid_constant__ RwA
         if (lane < kRwMaxWaves) s_ready[lane] = 0;
         if (lane == 0) {
             mbar_init(&x_bar, 1);
-            mbar_init(&early_bar, 1);
-            mbar_init(&tab_bar, 1);
+            mbar_init(&in_bar, 1);
+            for (int l = 0; l < kRwLevels; ++l) mbar_init(&lvl_bar[l], 1);
             mbar_init(&ep_bar[0], 4);
             mbar_init(&ep_bar[1], 4);
         }
@@ -378,6 +402,12 @@ ffn_rows_kernel(const __grid_constant__ RwMaps maps, const __grid_constant__ RwA
     tc_fence_after();
     const uint32_t tmem_base = s_tmem;
     const int lim0 = s_lim[0];
+    // the hidden states may be read (see warp 3); by the one thread that issues their copies
+    auto inputs_wait = [&]() -> bool {
+        if (!mbar_wait(&in_bar, 0)) { atomicExch(ws.status, ST_MBAR_TIMEOUT); return false; }
+        asm volatile("fence.proxy.async.global;" ::: "memory");
+        return true;
+    };
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
@@ -386,7 +416,7 @@ ffn_rows_kernel(const __grid_constant__ RwMaps maps, const __grid_constant__ RwA
             const uint32_t ring_a = smem_u32(ring), full_a = smem_u32(full_bar);
             int s = 0, lim = lim0, level = 0, ready_w = 0;
             uint32_t par = 1;
-            bool alive = true;
+            bool alive = pl.x_bytes != 0 || inputs_wait();
             // second-projection stages whose weights are in flight but whose token tiles wait for the
             // activations of wave pend_w: pend_n stages from ring slot pend_s, task pend_t, k-tile pend_k on
             int pend_n = 0, pend_s = 0, pend_t = 0, pend_k = 0, pend_w = 0;
@@ -435,8 +465,8 @@ ffn_rows_kernel(const __grid_constant__ RwMaps maps, const __grid_constant__ RwA
             };
 
             for (int i = 0; alive; ++i) {
-                while (i >= lim && level < 2) {
-                    if (!mbar_wait(level == 0 ? &early_bar : &tab_bar, 0)) { atomicExch(ws.status, ST_MBAR_TIMEOUT); alive = false; break; }
+                while (i >= lim && level < kRwLevels) {
+                    if (!mbar_wait(&lvl_bar[level], 0)) { atomicExch(ws.status, ST_MBAR_TIMEOUT); alive = false; break; }
                     lim = s_lim[++level];
                 }
                 if (!alive || i >= lim) break;
@@ -500,7 +530,8 @@ ffn_rows_kernel(const __grid_constant__ RwMaps maps, const __grid_constant__ RwA
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer
         if (rw_elect()) {
-            if (pl.x_bytes) {
+            bool alive = true, x_there = pl.x_bytes == 0;
+            if (pl.x_bytes && (alive = inputs_wait())) {
                 // the hidden states' tiles, eight k-tiles per copy (past the end: zeros)
                 const uint32_t xb = smem_u32(&x_bar), xd = smem_u32(xres);
                 rw_expect(xb, (uint32_t)(((nk + 7) & ~7) * pl.xr * 128));
@@ -508,13 +539,12 @@ ffn_rows_kernel(const __grid_constant__ RwMaps maps, const __grid_constant__ RwA
             }
             int s = 0, lim = lim0, level = 0;
             uint32_t par = 0, run = 0;
-            bool alive = true, x_there = pl.x_bytes == 0;
             const uint32_t nbm = (uint32_t)pl.n_acc - 1u, nbs = (uint32_t)__ffs(pl.n_acc) - 1u;
             const uint64_t ring_d = tc_smem_desc(ring), ring_d2 = tc_smem_desc_sbo(ring, 2048u), xres_d = tc_smem_desc(xres);
             const uint32_t idesc1 = tc_idesc(pl.n1), x_step = (uint32_t)pl.xr * 8u;     // (descriptor units of 16 bytes)
             for (int i = 0; alive; ++i) {
-                while (i >= lim && level < 2) {
-                    if (!mbar_wait(level == 0 ? &early_bar : &tab_bar, 0)) { atomicExch(ws.status, ST_MBAR_TIMEOUT); alive = false; break; }
+                while (i >= lim && level < kRwLevels) {
+                    if (!mbar_wait(&lvl_bar[level], 0)) { atomicExch(ws.status, ST_MBAR_TIMEOUT); alive = false; break; }
                     lim = s_lim[++level];
                 }
                 if (!alive || i >= lim) break;
@@ -579,56 +609,179 @@ ffn_rows_kernel(const __grid_constant__ RwMaps maps, const __grid_constant__ RwA
             }
         }
     } else if (warp == 10) {
-        // ------------------------------------------------------------------ early list, then watcher
-        int n_early = 0, nt = 0;
-        if (EARLY) {
-            // bounded wait for the routing kernel's list: one tagged 64-bit word per 32 experts, each
-            // polled by a lane of its own (a release store behind everything that kernel clears; all
-            // its blocks are resident or done when this grid is scheduled)
-            const int nwords = (sh.E + 31) >> 5;
+        // ------------------------------------------------------------------ early experts, first projection's tasks; then watcher
+        // Bounded wait for words of the routing kernel, each polled by a lane of its own until its tag is
+        // there.  (They are cleared before this grid is scheduled.)
+        const int nwords = (sh.E + 31) >> 5;
+        auto poll = [&](const unsigned long long *words, int n) -> unsigned {
             unsigned long long v = 0ull;
-            bool ok = false;
             for (unsigned i = 0; i < (1u << 21); ++i) {
-                if (lane < nwords)
-                    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(reinterpret_cast<const unsigned long long *>(ws.early) + lane) : "memory");
-                if (__all_sync(0xffffffffu, lane >= nwords || (v >> 32) == 1ull)) { ok = true; break; }
+                if (lane < n)
+                    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(words + lane) : "memory");
+                if (__all_sync(0xffffffffu, lane >= n || (v >> 32) == 1ull)) return lane < n ? (unsigned)v : 0u;
                 __nanosleep(20);
             }
-            if (!ok && lane == 0) atomicExch(ws.status, ST_DEP_TIMEOUT);
-            const unsigned w = (ok && lane < nwords) ? (unsigned)v : 0u;
+            if (lane == 0) atomicExch(ws.status, ST_DEP_TIMEOUT);
+            return 0u;
+        };
+        // experts of a set (lane q: word q) to s_id[n ..], ascending; returns the new n
+        auto expand = [&](unsigned w, int n) -> int {
 #pragma unroll 1
             for (int q = 0; q < nwords; ++q) {
                 const unsigned wq = __shfl_sync(0xffffffffu, w, q);
-                // this word's experts, one per lane
-                if ((wq >> lane) & 1u) {
-                    TcGroup gr;
-                    gr.mask = 0ull; gr.group = 32 * q + lane; gr.T = 0; gr.off = 0; gr.f = sh.f;
-                    gr.p1 = 0; gr.p2 = 0;
-                    groups[n_early + __popc(wq & ((1u << lane) - 1u))] = gr;
-                }
-                n_early += __popc(wq);
+                if ((wq >> lane) & 1u) s_id[n + __popc(wq & ((1u << lane) - 1u))] = (uint16_t)(32 * q + lane);
+                n += __popc(wq);
             }
             __syncwarp();
-            // lot E: their first projection
-            int start, cnt;
-            share(n_early * Gf, sh.n_sh * Gs, start, cnt);
-            const RwSeg sg = rw_seg(start, cnt, pl.gf, 3, (int)pl.tf.d);
-            nt = sg.n;
-            for (int j = lane; j < sg.n; j += 32) {
+            return n;
+        };
+        auto open = [&](int level, int tasks_known) {
+            __syncwarp();
+            if (lane == 0) {
+                s_lim[level] = min(tasks_known, pl.max_tasks);
+                mbar_arrive(&lvl_bar[level - 1]);
+            }
+        };
+        // Two passes over the same code.  The first, with made-up inputs while there is nothing to wait for yet,
+        // brings the code into the instruction caches: it runs once per launch, and fetched cold with the
+        // weight stream on the memory system it took 3 us between the selection and the tasks.
+#pragma unroll 1
+        for (int real = EARLY ? 0 : 1; real < 2; ++real) {
+            int n_early = 0, n_bad = 0, U = 0, nt = lim0, start, cnt;
+            const int n_sh_units = sh.n_sh * Gs;
+            if (EARLY) {
+                if (real) {
+                    // all blocks of the routing kernel have arrived: logits and importances are there, what it
+                    // clears is cleared
+                    const unsigned target = __shfl_sync(0xffffffffu, poll(ws.early + kEarlyWords, 1), 0);
+                    bool there = false;
+                    for (unsigned i = 0; i < (1u << 21); ++i) {
+                        unsigned v;
+                        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(ws.ticket) : "memory");
+                        if (__all_sync(0xffffffffu, (int)(v - target) >= 0)) { there = true; break; }
+                        __nanosleep(20);
+                    }
+                    if (!there && lane == 0) atomicExch(ws.status, ST_TICKET_TIMEOUT);
+                }
+                // The n_early experts of largest importance: lane owns experts lane, lane + 32, .., as integer
+                // keys in the order of the floats whose last bits name the expert, so that no two are equal
+                // (24 bits of the importance decide, which is plenty for a guess).
+                unsigned key[kEarlyWords], won = 0u;
+#pragma unroll
+                for (int q = 0; q < kEarlyWords; ++q) {
+                    const int e = lane + 32 * q;
+                    key[q] = 0u;
+                    if (e < sh.E) {
+                        const unsigned f = real ? __float_as_uint(__ldcg(&ws.gsum[e])) : 0u;
+                        key[q] = ((f & 0x80000000u ? ~f : f | 0x80000000u) & 0xffffff00u) | (255u - (unsigned)e);
+                    }
+                }
+#pragma unroll 1
+                for (int r = 0; r < pl.n_early; ++r) {
+                    unsigned m = max(key[0], key[1]);
+                    if (nwords > 2) {
+#pragma unroll
+                        for (int q = 2; q < kEarlyWords; ++q) m = max(m, key[q]);
+                    }
+                    m = __reduce_max_sync(0xffffffffu, m);
+                    const int e = 255 - (int)(m & 255u);
+                    if (lane == (e & 31)) {
+                        won |= 1u << (e >> 5);
+#pragma unroll
+                        for (int q = 0; q < kEarlyWords; ++q)
+                            if (key[q] == m) key[q] = 0u;
+                    }
+                }
+                unsigned w = 0u;
+#pragma unroll 1
+                for (int q = 0; q < nwords; ++q) {
+                    const unsigned word = __ballot_sync(0xffffffffu, (won >> q) & 1u);
+                    if (lane == q) w = word;
+                }
+                n_early = expand(w, 0);
+                // lot E: their first projection
+                share(n_early * Gf, n_sh_units, start, cnt);
+                const RwSeg sg = rw_seg(start, cnt, pl.gf, 3, (int)pl.tf.d);
+                for (int j = lane; j < sg.n; j += 32) {
+                    int u, len;
+                    rw_seg_task(sg, pl.gf, 3, pl.tf, j, u, len);
+                    const int g = rw_div(u, pl.gf);
+                    if (nt + j < pl.max_tasks) make_p1(&tasks[nt + j], g, s_id[g], u - g * Gf, len, 0, 0);
+                }
+                nt += sg.n;
+                if (real) open(1, nt);
+                // all others, as soon as the selection is known
+                const unsigned all = real ? poll(ws.early, nwords) : w ^ (lane < nwords ? 1u : 0u);
+                U = expand(all & ~w, n_early);
+                int a = 0, ns = 0;
+#pragma unroll 1
+                for (int q = 0; q < nwords; ++q) {
+                    const unsigned wq = __shfl_sync(0xffffffffu, w, q), sq = wq & __shfl_sync(0xffffffffu, all, q), below = (1u << lane) - 1u;
+                    if ((sq >> lane) & 1u) s_sel[ns + __popc(sq & below)] = (uint8_t)(a + __popc(wq & below));
+                    a += __popc(wq);
+                    ns += __popc(sq);
+                }
+                n_bad = n_early - ns;
+            } else {
+                open(1, nt);
+                asm volatile("griddepcontrol.wait;" ::: "memory");
+                U = ws.header[2];
+                for (int a = lane; a < U; a += 32) s_id[a] = (uint16_t)ws.active[a];
+                __syncwarp();
+            }
+            // lane w: wave w begins at the first routed group whose first projection lies past split16 / 16
+            // of all of it (the early and the shared experts are in wave 0); lane 4: the end
+            int bnd = 0;
+            if (lane > 0 && lane < kRwMaxWaves) {
+                const int s16 = pl.split16[lane - 1], want = ((U * Gf + n_sh_units) * s16 >> 4) - n_sh_units;
+                bnd = s16 >= 16 ? U : min(U, max(rw_div(max(want, 0) + Gf - 1, pl.gf), max(n_early, sh.n_sh ? 0 : 1)));
+            } else if (lane >= kRwMaxWaves) {
+                bnd = U;
+            }
+            if (lane <= kRwMaxWaves) s_bound[lane] = bnd;
+            const unsigned some = __ballot_sync(0xffffffffu, lane > 0 && lane < kRwMaxWaves && bnd < U);
+            // lane w: first projection of wave w without the early experts
+            const int lo = max(bnd, n_early), hi = __shfl_down_sync(0xffffffffu, bnd, 1);
+            const int n = lane < kRwMaxWaves ? max(0, hi - lo) * Gf : 0;
+            share(n, n_sh_units + lo * Gf, start, cnt);
+            const RwSeg sg = rw_seg(start, n > 0 ? cnt : 0, pl.gf, 3, (int)pl.tf.d);
+            int first = sg.n;
+#pragma unroll
+            for (int o = 1; o < kRwMaxWaves; o <<= 1) {
+                const int t = __shfl_up_sync(0xffffffffu, first, o);
+                if (lane >= o) first += t;
+            }
+            if (lane < kRwMaxWaves) {
+                s_lot[lane] = sg;
+                s_first[lane] = nt + first - sg.n;
+                if (lane == kRwMaxWaves - 1) s_first[kRwMaxWaves] = nt + first;
+            }
+            if (lane == 0) {
+                s_waves = 1 + __popc(some);
+                s_n_bad = n_bad;
+                s_U = U;
+            }
+            __syncwarp();
+            const int end = s_first[kRwMaxWaves];
+            for (int i = nt + lane; i < end && i < pl.max_tasks; i += 32) {
+                int w = 0;
+#pragma unroll
+                for (int l = 1; l < kRwMaxWaves; ++l) w += i >= s_first[l] ? 1 : 0;
                 int u, len;
-                rw_seg_task(sg, pl.gf, 3, pl.tf, j, u, len);
-                const int g = rw_div(u, pl.gf);
-                if (lim0 + j < pl.max_tasks) make_p1(&tasks[lim0 + j], g, groups[g].group, u - g * Gf, len, 0, 0);
+                rw_seg_task(s_lot[w], pl.gf, 3, pl.tf, i - s_first[w], u, len);
+                const int gq = rw_div(u, pl.gf), a = gq + max(s_bound[w], n_early);
+                make_p1(&tasks[i], a, weights_of(s_id[a]), u - gq * Gf, len, 0, w);
+            }
+            __syncwarp();
+            if (real) {
+                if (lane == 0 && end > pl.max_tasks) atomicExch(ws.status, ST_BAD_PLAN);
+                open(2, end);
             }
         }
-        __syncwarp();
         if (lane == 0) {
-            s_lim[1] = min(lim0 + nt, pl.max_tasks);
-            s_n_early = n_early;
-            mbar_arrive(&early_bar);
             // the waves' counters (the activations of all CTAs are stored), published in shared memory, so
             // that the producer never waits on global memory
-            if (mbar_wait(&tab_bar, 0)) {
+            if (mbar_wait(&lvl_bar[kRwLevels - 1], 0)) {
                 const int nw = s_waves;
                 for (int w = 0; w < nw; ++w) {
                     bool there = false;
@@ -639,6 +792,9 @@ ffn_rows_kernel(const __grid_constant__ RwMaps maps, const __grid_constant__ RwA
                     if (!there) { atomicExch(ws.status, ST_DEP_TIMEOUT); break; }
                     __threadfence_block();
                     s_ready[w] = 1;
+                    // (every CTA has read the importances: back to zero for the next layer)
+                    if (w == 0 && EARLY && cta == 0)
+                        for (int e = 0; e < sh.E; ++e) ws.gsum[e] = 0.0f;
                 }
             } else {
                 atomicExch(ws.status, ST_MBAR_TIMEOUT);
@@ -647,117 +803,114 @@ ffn_rows_kernel(const __grid_constant__ RwMaps maps, const __grid_constant__ RwA
     } else {
         // ------------------------------------------------------------------ epilogue sets
         const int set = warp >= 6 ? 1 : 0;
+        if (warp == 3) {
+            // the inputs may be read: the routing kernel has passed its own grid dependency (and says so), or ended
+            if (EARLY) {
+                bool there = false;
+                for (unsigned i = 0; i < (1u << 21); ++i) {
+                    unsigned long long v;
+                    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(ws.early + kEarlyWords) : "memory");
+                    if (__all_sync(0xffffffffu, v != 0ull)) { there = true; break; }
+                    __nanosleep(20);
+                }
+                if (!there && lane == 0) atomicExch(ws.status, ST_DEP_TIMEOUT);
+            } else {
+                asm volatile("griddepcontrol.wait;" ::: "memory");
+            }
+            if (lane == 0) mbar_arrive(&in_bar);
+        }
         if (set == 1) {
-            // the tables, by warps 6..9 (128 threads on hardware barrier 1)
+            // the tables and the second projection's tasks, by warps 6..9 (128 threads on hardware barrier 1).
+            // The next kernel in the stream may come up once this CTA has read the words of the early start:
+            // the next layer's routing kernel clears them before anything else.
+            // Two passes over the same code, as for warp 10: the first one makes tasks of one expert at the very
+            // end of the table, where no real one of the first projection can be.
             const int tt = tid - 192;
-            asm volatile("griddepcontrol.wait;" ::: "memory");
-            asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-            const int n_active = ws.header[0], U = ws.header[2];
-            const bool el_ok = mbar_wait(&early_bar, 0);
-            const int n_early = s_n_early, b0 = s_lim[1];
-            // the group table in its final form and the slot arrays
-            for (int a = tt; a < G; a += 128) {
-                const uint4 r0 = ws.gtab[2 * a], r1 = ws.gtab[2 * a + 1];
-                if (a < n_active) {
+            bool el_ok = true;
+#pragma unroll 1
+            for (int real = EARLY ? 0 : 1; real < 2; ++real) {
+                if (real) {
+                    el_ok = mbar_wait(&lvl_bar[1], 0) && mbar_wait(&in_bar, 0);
+                    asm volatile("griddepcontrol.wait;" ::: "memory");
+                    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+                }
+                const int U = real ? s_U : 1, n_bad = real ? s_n_bad : 0, b0 = real ? s_lim[2] : pl.max_tasks - 8;
+                // the groups in their final form and the slot arrays
+                for (int a = tt; a < U; a += 128) {
+                    const int id = real ? (int)s_id[a] : 0;
                     TcGroup gr;
-                    gr.group = (int)r0.x;
-                    // offloaded experts: from here on the group id of a routed expert is the device slot its
-                    // weights lie in (a slot index is below E as well, so shared groups stay recognisable)
-                    if (ws.slot_of && gr.group < sh.E) gr.group = __ldg(&ws.slot_of[gr.group]);
-                    gr.T = (int)r0.y;
-                    gr.off = (int)r0.z;
-                    gr.f = gr.group < sh.E ? sh.f : sh.f_sh;
-                    gr.mask = (unsigned long long)r1.x | ((unsigned long long)r1.y << 32);
+                    gr.T = __ldcg(&ws.counts[id]);       // (past L1: the first pass may be ahead of the routing kernel)
+                    gr.off = __ldcg(&ws.offsets[id]);
+                    gr.mask = __ldcg(&ws.tokmask[id]);
+                    gr.group = weights_of(id);
+                    gr.f = sh.f;
                     gr.p1 = 0; gr.p2 = 0;
-                    // (the early experts must lead the final list in the order they were announced in)
-                    if (a < n_early && groups[a].group != gr.group) atomicExch(ws.status, ST_BAD_PLAN);
                     groups[a] = gr;
                 }
-            }
-            for (int i = tt; i < n_slots; i += 128) {
-                s_slot_token[i] = ws.slot_token[i];
-                s_slot_w[i] = ws.slot_w[i];
-            }
-            const int RB = (int)pl.rb.d, u2r = RB * (int)pl.kr.d, u2s = sh.n_sh ? RB * (int)pl.ks.d : 0;
-            if (warp == 6) {
-                // lane w: wave w begins at the first routed group whose first projection lies past split16 / 16
-                // of all of it (the early and the shared experts are in wave 0); lane 4: the end
-                int bnd = 0;
-                if (lane > 0 && lane < kRwMaxWaves) {
-                    const int s16 = pl.split16[lane - 1], want = ((U * Gf + sh.n_sh * Gs) * s16 >> 4) - sh.n_sh * Gs;
-                    bnd = s16 >= 16 ? U : min(U, max(rw_div(max(want, 0) + Gf - 1, pl.gf), max(n_early, sh.n_sh ? 0 : 1)));
-                } else if (lane >= kRwMaxWaves) {
-                    bnd = U;
+                for (int i = tt; i < (real ? n_slots : 0); i += 128) {
+                    s_slot_token[i] = ws.slot_token[i];
+                    s_slot_w[i] = ws.slot_w[i];
                 }
-                if (lane <= kRwMaxWaves) s_bound[lane] = bnd;
-                const unsigned some = __ballot_sync(0xffffffffu, lane > 0 && lane < kRwMaxWaves && bnd < U);
-                if (lane == 0) s_waves = 1 + __popc(some);
-                // lane l: lot l.  First projection of wave l (without the early experts), then the second
-                // projection: wave 0, shared experts, waves 1 ..
-                const bool p1 = lane < kRwMaxWaves, sx = lane == kRwMaxWaves + 1;
-                const int w = p1 ? lane : (lane <= kRwMaxWaves + 1 ? 0 : min(lane - kRwMaxWaves - 1, kRwMaxWaves - 1));
-                const int lo = __shfl_sync(0xffffffffu, bnd, w), hi = __shfl_sync(0xffffffffu, bnd, w + 1);
-                int n = p1 ? (hi - max(lo, n_early)) * Gf : (sx ? sh.n_sh * u2s : (hi - lo) * u2r);
-                if (lane >= kRwLots) n = 0;
-                const int n_pre = sh.n_sh * Gs + n_early * Gf;
-                int before = n;
+                const int RB = (int)pl.rb.d, u2r = RB * (int)pl.kr.d, u2s = sh.n_sh ? RB * (int)pl.ks.d : 0;
+                if (warp == 6) {
+                    // lane l: lot l of the second projection: wave 0, shared experts, waves 1 ..
+                    const bool sx = lane == 1;
+                    const int w = lane < 2 ? 0 : min(lane - 1, kRwMaxWaves - 1);
+                    int n = sx ? sh.n_sh * u2s : (real ? s_bound[w + 1] - s_bound[w] - (w == 0 ? n_bad : 0) : w < 2) * u2r;
+                    if (lane >= kRwLots2) n = 0;
+                    // units dealt before this lot, and how many CTAs (0 .. R - 1) have one unit of the first
+                    // projection more than the others: they get that much less of the second one, in its last lot
+                    const int n1 = sh.n_sh * Gs + U * Gf, R = n1 - rw_div(n1, pl.p) * P;
+                    int before = n;
 #pragma unroll
-                for (int o = 1; o < 16; o <<= 1) {
-                    const int t = __shfl_up_sync(0xffffffffu, before, o);
-                    if (lane >= o) before += t;
-                }
-                before += n_pre - n;
-                // CTAs 0 .. R - 1 have one unit of the first projection more than the others: they get that
-                // much less of the second one, in its last lot
-                const int f1 = __shfl_sync(0xffffffffu, before, kRwMaxWaves), R = f1 - rw_div(f1, pl.p) * P;
-                const unsigned nz = __ballot_sync(0xffffffffu, !p1 && n > 0);
-                int start, cnt;
-                const int v = n + pl.delta * R, qv = rw_div(v, pl.p);
-                if (lane == 31 - __clz(nz) && qv >= pl.delta) {
-                    const int r = v - qv * P, rot = before - rw_div(before, pl.p) * P;
-                    int c = cta - rot;
-                    if (c < 0) c += P;
-                    // CTAs before this one in the order that starts at rot, and those of them below R
-                    const int end = rot + c;
-                    const int ex = end <= P ? max(0, min(end, R) - min(rot, R)) : (R - min(rot, R)) + min(end - P, R);
-                    start = c * qv + min(c, r) - pl.delta * ex;
-                    cnt = qv + (c < r ? 1 : 0) - (cta < R ? pl.delta : 0);
-                } else {
-                    share(n, before, start, cnt);
-                }
-                const RwDiv kd = p1 ? pl.gf : (sx ? pl.ks : pl.kr);
-                const RwSeg sg = rw_seg(start, n > 0 ? cnt : 0, kd, p1 ? 3 : 24, p1 ? (int)pl.tf.d : 1);
-                int first = sg.n;
+                    for (int o = 1; o < 8; o <<= 1) {
+                        const int t = __shfl_up_sync(0xffffffffu, before, o);
+                        if (lane >= o) before += t;
+                    }
+                    before += n1 - n;
+                    const unsigned nz = __ballot_sync(0xffffffffu, n > 0);
+                    int start, cnt;
+                    const int v = n + pl.delta * R, qv = rw_div(v, pl.p);
+                    if (lane == 31 - __clz(nz) && qv >= pl.delta) {
+                        const int r = v - qv * P, rot = before - rw_div(before, pl.p) * P;
+                        int c = cta - rot;
+                        if (c < 0) c += P;
+                        // CTAs before this one in the order that starts at rot, and those of them below R
+                        const int end = rot + c;
+                        const int ex = end <= P ? max(0, min(end, R) - min(rot, R)) : (R - min(rot, R)) + min(end - P, R);
+                        start = c * qv + min(c, r) - pl.delta * ex;
+                        cnt = qv + (c < r ? 1 : 0) - (cta < R ? pl.delta : 0);
+                    } else {
+                        share(n, before, start, cnt);
+                    }
+                    const RwSeg sg = rw_seg(start, n > 0 ? cnt : 0, sx ? pl.ks : pl.kr, 24, 1);
+                    int first = sg.n;
 #pragma unroll
-                for (int o = 1; o < 16; o <<= 1) {
-                    const int t = __shfl_up_sync(0xffffffffu, first, o);
-                    if (lane >= o) first += t;
+                    for (int o = 1; o < 8; o <<= 1) {
+                        const int t = __shfl_up_sync(0xffffffffu, first, o);
+                        if (lane >= o) first += t;
+                    }
+                    if (lane < kRwLots2) {
+                        s_lot2[lane] = sg;
+                        s_first2[lane] = b0 + first - sg.n;
+                        if (lane == kRwLots2 - 1) s_first2[kRwLots2] = b0 + first;
+                    }
                 }
-                if (lane < kRwLots) {
-                    s_lot[lane] = sg;
-                    s_lot_first[lane] = b0 + first - sg.n;
-                    if (lane == kRwLots - 1) s_lot_first[kRwLots] = b0 + first;
-                }
-            }
-            asm volatile("bar.sync 1, 128;" ::: "memory");          // the group table and the lots are complete
-            const int b1 = s_lot_first[kRwLots];
-            for (int i = b0 + tt; i < b1 && i < pl.max_tasks; i += 128) {
-                int l = 0;
-#pragma unroll 1
-                while (l + 1 < kRwLots && i >= s_lot_first[l + 1]) ++l;
-                const bool p1 = l < kRwMaxWaves, sx = l == kRwMaxWaves + 1;
-                const int w = p1 ? l : (l <= kRwMaxWaves + 1 ? 0 : l - kRwMaxWaves - 1);
-                const RwDiv kd = p1 ? pl.gf : (sx ? pl.ks : pl.kr), td = p1 ? pl.tf : RwDiv{1u, 0u};
-                RwTask *t = &tasks[i];
-                int u, len;
-                rw_seg_task(s_lot[l], kd, p1 ? 3 : 24, td, i - s_lot_first[l], u, len);
-                const int gq = rw_div(u, kd), in = u - gq * (int)kd.d;
-                if (p1) {
-                    const int a = gq + max(s_bound[w], n_early);
-                    make_p1(t, a, groups[a].group, in, len, 0, w);
-                } else {
-                    const int eq = rw_div(gq, pl.rb), rbk = gq - eq * RB;
-                    const int a = sx ? U + eq : eq + s_bound[w];
+                asm volatile("bar.sync 1, 128;" ::: "memory");          // the group table and the lots are complete
+                const int b1 = s_first2[kRwLots2];
+                for (int i = b0 + tt; i < b1 && i < pl.max_tasks; i += 128) {
+                    int l = 0;
+#pragma unroll
+                    for (int j = 1; j < kRwLots2; ++j) l += i >= s_first2[j] ? 1 : 0;
+                    const bool sx = l == 1;
+                    const int w = l < 2 ? 0 : l - 1;
+                    const RwDiv kd = sx ? pl.ks : pl.kr;
+                    RwTask *t = &tasks[i];
+                    int u, len;
+                    rw_seg_task(s_lot2[l], kd, 24, RwDiv{1u, 0u}, i - s_first2[l], u, len);
+                    const int gq = rw_div(u, kd), in = u - gq * (int)kd.d, eq = rw_div(gq, pl.rb), rbk = gq - eq * RB;
+                    // (wave 0: the early experts that have tokens, then the others)
+                    const int a = sx ? GP + eq : (w > 0 || n_bad == 0 ? eq + (real ? s_bound[w] : 0) : (eq < pl.n_early - n_bad ? (int)s_sel[eq] : eq + n_bad));
                     const TcGroup &g = groups[a];
                     const int kts = ((sx ? sh.f_sh : sh.f) + 63) >> 6;
                     t->flags = 1 | (sx ? 2 : 0) | (w << 2) | (sh.d - rbk * 128 <= 64 ? 16 : 0) | (rw_tok_rows(g.T) << 8);
@@ -767,13 +920,13 @@ ffn_rows_kernel(const __grid_constant__ RwMaps maps, const __grid_constant__ RwA
                     t->a = a;
                     t->pos = rbk * 128;
                 }
-            }
-            asm volatile("bar.sync 1, 128;" ::: "memory");
-            if (tt == 0) {
-                if (!el_ok) atomicExch(ws.status, ST_MBAR_TIMEOUT);
-                if (b1 > pl.max_tasks) atomicExch(ws.status, ST_BAD_PLAN);
-                s_lim[2] = min(b1, pl.max_tasks);
-                mbar_arrive(&tab_bar);                              // (release: the tables are written)
+                asm volatile("bar.sync 1, 128;" ::: "memory");
+                if (tt == 0 && real) {
+                    if (!el_ok) atomicExch(ws.status, ST_MBAR_TIMEOUT);
+                    if (b1 > pl.max_tasks) atomicExch(ws.status, ST_BAD_PLAN);
+                    s_lim[kRwLevels] = min(b1, pl.max_tasks);
+                    mbar_arrive(&lvl_bar[kRwLevels - 1]);               // (release: the tables are written)
+                }
             }
         }
         const int q = warp & 3;                                     // TMEM lane quarter this warp may read
@@ -783,9 +936,9 @@ ffn_rows_kernel(const __grid_constant__ RwMaps maps, const __grid_constant__ RwA
         bool alive = true;
         auto wait_level = [&](int to) -> bool {
             while (level < to) {
-                if (!mbar_wait(level == 0 ? &early_bar : &tab_bar, 0)) { if (lane == 0) atomicExch(ws.status, ST_MBAR_TIMEOUT); return false; }
+                if (!mbar_wait(&lvl_bar[level], 0)) { if (lane == 0) atomicExch(ws.status, ST_MBAR_TIMEOUT); return false; }
                 lim = s_lim[++level];
-                if (level == 2) waves = s_waves;
+                if (level == kRwLevels) waves = s_waves;
             }
             return true;
         };
@@ -800,15 +953,15 @@ ffn_rows_kernel(const __grid_constant__ RwMaps maps, const __grid_constant__ RwA
             return true;
         };
         for (int i = set; alive; i += kRwSets) {
-            while (i >= lim && level < 2) { if (!wait_level(level + 1)) { alive = false; break; } }
+            while (i >= lim && level < kRwLevels) { if (!wait_level(level + 1)) { alive = false; break; } }
             if (!alive || i >= lim) break;
             const RwTask t = tasks[i];
             const uint32_t buf = (uint32_t)i & nbm;
             const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + buf * (uint32_t)pl.acc_cols;
             // (a task of the second projection, or of a later wave: this set's part of the waves before is done)
             if (!service((t.flags & 1) ? kRwMaxWaves : (t.flags >> 2) & 3)) { alive = false; break; }
-            // an early expert: its tokens and slots come with the tables
-            if (!(t.flags & 3) && level < 2) { if (!wait_level(2)) { alive = false; break; } }
+            // a routed expert: its tokens and slots come with the tables
+            if (!(t.flags & 3) && level < kRwLevels) { if (!wait_level(kRwLevels)) { alive = false; break; } }
             if (!mbar_wait(&acc_full[buf], ((uint32_t)i >> nbs) & 1u)) {
                 if (lane == 0) atomicExch(ws.status, ST_MBAR_TIMEOUT);
                 alive = false;
@@ -877,7 +1030,7 @@ ffn_rows_kernel(const __grid_constant__ RwMaps maps, const __grid_constant__ RwA
             __syncwarp();
             if (lane == 0) mbar_arrive(&acc_empty[buf]);
         }
-        if (alive && wait_level(2)) service(kRwMaxWaves);
+        if (alive && wait_level(kRwLevels)) service(kRwMaxWaves);
     }
     // every path ends here (all waits above are bounded), so the TMEM is always returned
     tc_fence_before();

@@ -114,26 +114,16 @@ __device__ __forceinline__ void gating_writeout(const Shape &sh, int B, const Wo
 }
 
 // Gating of one batch by a whole thread block (kRouteThreads threads) on the logits in the workspace.
-// s_l: shared memory for B * E + B doubles (the logits and the confidences are staged there).
+// s_l: shared memory for B * E + B doubles (the logits and the confidences are staged there) and, behind
+// them, gate_mem_bytes(E, B, k).
 template <int JE>
 __device__ __forceinline__ void gating_block(const Shape &sh, int B, const Workspace &ws, const float *__restrict__ conf,
                                              int has_gate, int32_t *__restrict__ sel_idx, float *__restrict__ sel_w,
                                              int32_t *__restrict__ n_unique, double *s_l, int ksplit, const double *__restrict__ lpart,
                                              int early = 0)
 {
-    __shared__ unsigned long long s_mask[kMaxExperts], s_gk[kMaxExperts];
-    __shared__ unsigned s_early32[8];
-    __shared__ double s_lam[kMaxTokens], s_zmax[kMaxTokens], s_den[kMaxTokens];
-    __shared__ int s_sel[kMaxTokens * kMaxTopK];
-    __shared__ float s_pw[kMaxTokens * kMaxTopK];
-    __shared__ int s_cnt[kMaxExperts], s_off[kMaxExperts + 1], s_pos[kMaxExperts];
-    __shared__ int s_U;
-    __shared__ unsigned s_star32[8];
-    __shared__ unsigned char s_star[kMaxExperts];
-    GateMem gm;
-    gm.mask = s_mask; gm.gk = s_gk; gm.lam = s_lam; gm.zmax = s_zmax; gm.den = s_den; gm.sel = s_sel; gm.pw = s_pw;
-    gm.cnt = s_cnt; gm.off = s_off; gm.pos = s_pos; gm.U = &s_U; gm.star = s_star; gm.star32 = s_star32;
-    gm.topk = reinterpret_cast<unsigned *>(s_sel);      // (the selection overwrites it: nobody reads it here)
+    // (sized by this batch and not for the largest one: a routing block shares its SM with the expert kernel)
+    const GateMem gm = gate_mem_carve(s_l + B * sh.E + B, sh.E, B, sh.k);
     const GateGroup gg{(int)threadIdx.x, (int)blockDim.x, 0};
     double *s_w = s_l + B * sh.E;
     if (ksplit > 0) {
@@ -158,36 +148,9 @@ __device__ __forceinline__ void gating_block(const Shape &sh, int B, const Works
     }
 #pragma unroll 1
     for (int b = gg.t; b < B; b += gg.n) s_w[b] = conf ? (double)conf[b] : 1.0;
-    if (early) {
-        // The expert kernel is already resident (programmatic launch) and waits for this list: the
-        // experts whose first projection it may stream while the gating below still runs.  A token's
-        // first expert by original logit stays selected whatever E* turns out to be (the bias lifts
-        // an expert by at most alpha (l_(1) - l_(k+1)) <= l_(1) - l_(k+1), so only the other k - 1 of
-        // its first k can pass it), which the caller has checked for this layer's alpha (early == 2).
-        // These experts lead the active list and the slot order, ascending, so that the expert
-        // kernel knows their groups before it knows the others.
-        if (gg.t < 8) s_early32[gg.t] = 0u;
-        __syncthreads();                                  // the logits are staged, the words cleared
-        if (early == 2) {
-#pragma unroll 1
-            for (int b = gg.t >> 5; b < B; b += gg.n >> 5) {
-                const int e = gate_top1<JE>(sh, b, s_l, gg.t & 31);
-                if ((gg.t & 31) == 0) atomicOr(&s_early32[e >> 5], 1u << (e & 31));
-            }
-        }
-        __syncthreads();
-        // one 64-bit word per 32 experts: the bits of the early experts under a tag of 1 (the words
-        // were cleared before this grid let the expert kernel be scheduled), each released by itself,
-        // so that whoever polls a word has its part of the list with the same load
-        if (gg.t < ((sh.E + 31) >> 5)) {
-            const unsigned long long v = (1ull << 32) | (unsigned long long)s_early32[gg.t];
-            asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(reinterpret_cast<unsigned long long *>(ws.early) + gg.t), "l"(v)
-                         : "memory");
-        }
-    }
     // (gating_group's first barrier orders these writes before the first read)
     gating_part1<JE>(sh, B, s_l, s_w, gg, gm, true);
-    gating_part2<JE>(sh, B, s_l, gg, gm, sel_idx, sel_w, true, early ? s_early32 : nullptr);
+    gating_part2<JE>(sh, B, s_l, gg, gm, sel_idx, sel_w, true, early ? ws.early : nullptr);
     gating_writeout(sh, B, ws, gm, has_gate, n_unique, gg);
 }
 
@@ -233,8 +196,8 @@ struct ZeroList {
     // partial sums in lpart [piece][token][row] (see route_logit_tasks); 0: by row blocks
     int ksplit;
     double *lpart;
-    // 1: the expert kernel behind this launch starts before the gating has ended (see gating_block);
-    // 2: the same, and every token's first expert by original logit is known to stay selected
+    // 1: the expert kernel behind this launch starts before the gating has ended, on the experts of largest
+    // aggregated importance (see gsum); it reads what Workspace::early holds
     int early;
 };
 
@@ -244,7 +207,8 @@ struct ZeroList {
 template <int ACT, int RT>
 __device__ __forceinline__ void route_logit_tasks(const Shape &sh, int B, const void *__restrict__ hidden,
                                                   const void *__restrict__ router, const void *__restrict__ sh_scale,
-                                                  double *__restrict__ lpart, int ksplit, int gwarp, int n_gwarps, int lane)
+                                                  double *__restrict__ lpart, int ksplit, const float *__restrict__ conf,
+                                                  float *__restrict__ gsum, int gwarp, int n_gwarps, int lane)
 {
     const int d = sh.d, n_rows = sh.E + (sh_scale ? 1 : 0), n_tg = (B + 7) >> 3;
     const int len = ((d + 4 * ksplit - 1) / (4 * ksplit)) * 4;              // columns of a piece, a multiple of 4
@@ -273,10 +237,19 @@ __device__ __forceinline__ void route_logit_tasks(const Shape &sh, int B, const 
 #pragma unroll
                 for (int i = 0; i < 4; ++i) acc[t] = fma((double)w[i], (double)x[t][i], acc[t]);
         }
+        float g = 0.0f;
 #pragma unroll
         for (int t = 0; t < 8; ++t) {
             const double v = warp_sum(acc[t]);
-            if (lane == t && b0 + t < B) lpart[((size_t)piece * B + b0 + t) * n_rows + row] = v;
+            if (lane == t && b0 + t < B) {
+                lpart[((size_t)piece * B + b0 + t) * n_rows + row] = v;
+                g = (conf ? conf[b0 + t] : 1.0f) * (float)v;
+            }
+        }
+        if (gsum && row < sh.E) {
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
+            if (lane == 0) atomicAdd(&gsum[row], g);
         }
     }
 }
@@ -285,10 +258,12 @@ __device__ __forceinline__ void route_logit_tasks(const Shape &sh, int B, const 
 // B - 1, so that every load is unconditional and issued before the first use).
 template <int ACT, int RT, int NT>
 __device__ __forceinline__ void route_pass(const Shape &sh, int B, int b0, const Workspace &ws, int row, const uint8_t *wrow,
-                                           const void *__restrict__ hidden, double *s_part)
+                                           const void *__restrict__ hidden, const float *__restrict__ conf, float *__restrict__ gsum,
+                                           double *s_part)
 {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, d = sh.d;
     const size_t ab = ACT == DT_F32 ? 4 : 2;
+    const float wb = (gsum && conf && tid < NT && b0 + tid < B) ? conf[b0 + tid] : 1.0f;
     double acc[NT];
 #pragma unroll
     for (int t = 0; t < NT; ++t) acc[t] = 0.0;
@@ -311,12 +286,21 @@ __device__ __forceinline__ void route_pass(const Shape &sh, int B, int b0, const
         if (lane == 0) s_part[warp * kRouteTok + t] = s;
     }
     __syncthreads();
-    if (tid < NT && b0 + tid < B) {
-        double s = 0.0;
+    if (tid < 32) {
+        float g = 0.0f;
+        if (tid < NT && b0 + tid < B) {
+            double s = 0.0;
 #pragma unroll
-        for (int w = 0; w < kRouteThreads / 32; ++w) s += s_part[w * kRouteTok + tid];
-        if (row < sh.E) ws.logits[(size_t)(b0 + tid) * sh.E + row] = s;
-        else ws.gate_logit[b0 + tid] = s;
+            for (int w = 0; w < kRouteThreads / 32; ++w) s += s_part[w * kRouteTok + tid];
+            if (row < sh.E) ws.logits[(size_t)(b0 + tid) * sh.E + row] = s;
+            else ws.gate_logit[b0 + tid] = s;
+            g = wb * (float)s;
+        }
+        if (gsum && row < sh.E) {
+#pragma unroll
+            for (int o = NT >> 1; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
+            if (tid == 0) atomicAdd(&gsum[row], g);
+        }
     }
     __syncthreads();
 }
@@ -324,7 +308,7 @@ __device__ __forceinline__ void route_pass(const Shape &sh, int B, int b0, const
 // Router logits and gating in one launch.  A block computes one row of the router (row E is the
 // shared-expert gate vector) against one group of the batch's tokens in float64; block 0 then
 // runs the gating for the whole batch once every block has arrived (atomic ticket).
-// Dynamic shared memory: max(B * E + B, 16 * kRouteTok) doubles.
+// Dynamic shared memory: B * E + B doubles and gate_mem_bytes(E, B, k), at least 16 * kRouteTok doubles.
 // JE: experts per lane in the gating (2, 4 or 8 for up to 64, 128, 256 experts): a kernel of its own
 // for each, so that the gating code of a launch is one straight piece
 // THREADS: kRouteThreads, or kRouteThreadsBig for the kernel of the larger batches (warp tasks only)
@@ -337,25 +321,46 @@ __device__ __forceinline__ void route_body(const Shape &sh, int B, const Workspa
     extern __shared__ double s_dyn[];
     __shared__ int s_last;
     const int tid = threadIdx.x;
-    // Programmatic dependent launch: everything this kernel writes is read by the previous
-    // layer's kernels, so it waits for them first; the FFN kernel that follows may come up now
-    // and do its own set-up (both instructions do nothing in a plain launch).
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // Programmatic dependent launch: everything this kernel writes is read by the kernels of the layer in
+    // front, so it waits for them before it does; only the lists that the expert kernel of this layer
+    // polls are cleared before (the expert kernel in front lets this grid start once it has read
+    // them).  The expert kernel of this layer may come up once every block has passed
+    // launch_dependents, that is, while the layer in front still runs: it sets itself up and
+    // streams weights that do not depend on any routing.  (Both instructions do nothing in a plain launch.)
     if (zl.early && blockIdx.x == 0) {
-        // the expert kernel of this layer polls these words from the moment it is scheduled, which is
-        // after every block of this grid has passed the next instruction: they are cleared by then
-        if (tid < 8) {
-            asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(reinterpret_cast<unsigned long long *>(ws.early) + tid), "l"(0ull)
-                         : "memory");
+        if (tid <= kEarlyWords) {
+            asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(ws.early + tid), "l"(0ull) : "memory");
             __threadfence();
         }
         __syncthreads();
     }
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // what this block will read first, into L2 while it waits: its router row (the hidden states come from
+    // the kernel in front and are there already, or from the caller's memory: a prefetch changes nothing)
+    if (zl.ksplit == 0) {
+        const int n_rows_p = sh.E + (sh_scale ? 1 : 0), row_p = (int)blockIdx.x % n_rows_p;
+        const size_t rbytes = (size_t)sh.d * (RT == DT_F32 ? 4 : 2), hbytes = (size_t)B * sh.d * (ACT == DT_F32 ? 4 : 2);
+        const uint8_t *wr = row_p < sh.E ? reinterpret_cast<const uint8_t *>(router) + (size_t)row_p * rbytes
+                                         : reinterpret_cast<const uint8_t *>(sh_scale);
+        const size_t o = (size_t)tid * 128;
+        if (o < rbytes) asm volatile("prefetch.global.L2 [%0];" ::"l"(wr + o));
+        const size_t ho = ((size_t)blockIdx.x * THREADS + tid) * 128;
+        if (ho < hbytes) asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const uint8_t *>(hidden) + ho));
+    }
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     // (block 0: where the arrival counter stood when the launch before had ended; see below)
-    unsigned ticket_base = 0u;
-    if (blockIdx.x == 0 && tid == 0)
-        asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(ticket_base) : "l"(ws.ticket + 1) : "memory");
+    const int n_rows = sh.E + (sh_scale ? 1 : 0), n_grp = zl.groups > 1 ? zl.groups : 1;
+    // (early start: the expert kernel accumulates into what this grid clears, so the blocks that only clear
+    // arrive on the counter as well)
+    const int n_arrive = zl.early || zl.ksplit > 0 ? (int)gridDim.x : n_rows * n_grp;
+    unsigned ticket_target = 0u;
+    if (blockIdx.x == 0 && tid == 0) {
+        asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(ticket_target) : "l"(ws.ticket + 1) : "memory");
+        ticket_target += (unsigned)n_arrive;
+        if (zl.early)
+            asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(ws.early + kEarlyWords), "l"((1ull << 32) | (unsigned long long)ticket_target)
+                         : "memory");
+    }
 #pragma unroll
     for (int z = 0; z < 3; ++z) {
         uint4 *p = reinterpret_cast<uint4 *>(zl.ptr[z]);
@@ -374,22 +379,14 @@ __device__ __forceinline__ void route_body(const Shape &sh, int B, const Workspa
     // A row block takes one router row and one group of tokens: a larger batch is split over
     // several sets of row blocks (as many as fit on the SMs beside each other), because a block
     // takes 16 tokens per pass and its passes run one after the other (B = 64: 22 us in one set).
-    const int n_rows = sh.E + (sh_scale ? 1 : 0);
-    int n_arrive = 0;
     if (zl.ksplit > 0) {
         // larger batches: the logit pass as warp tasks over all blocks of the grid (a row block takes
         // 16 tokens per pass and its passes run one after the other: 22 us at 64 tokens)
-        n_arrive = (int)gridDim.x;
-        route_logit_tasks<ACT, RT>(sh, B, hidden, router, sh_scale, zl.lpart, zl.ksplit, (tid >> 5) * (int)gridDim.x + (int)blockIdx.x,
+        route_logit_tasks<ACT, RT>(sh, B, hidden, router, sh_scale, zl.lpart, zl.ksplit, conf, zl.early ? ws.gsum : nullptr, (tid >> 5) * (int)gridDim.x + (int)blockIdx.x,
                                    (THREADS / 32) * (int)gridDim.x, tid & 31);
         __syncthreads();
     } else if constexpr (THREADS == kRouteThreads) {
-    const int n_grp = zl.groups > 1 ? zl.groups : 1;
-    n_arrive = n_rows * n_grp;
-    // (early start of the expert kernel: it accumulates into what this grid clears as soon as the
-    // list above is out, so the blocks that only clear arrive on the counter as well)
-    if ((int)blockIdx.x >= n_arrive && !zl.early) return;
-    if (zl.early) n_arrive = (int)gridDim.x;
+    if ((int)blockIdx.x >= n_arrive) return;
     if ((int)blockIdx.x < n_rows * n_grp) {
     const int row = (int)blockIdx.x % n_rows, grp = (int)blockIdx.x / n_rows, d = sh.d;
     const int tg = 4 * ((B + 4 * n_grp - 1) / (4 * n_grp));            // tokens per group, a multiple of 4
@@ -397,11 +394,12 @@ __device__ __forceinline__ void route_body(const Shape &sh, int B, const Workspa
     const size_t rb = RT == DT_F32 ? 4 : 2;
     const uint8_t *wrow = row < sh.E ? reinterpret_cast<const uint8_t *>(router) + (size_t)row * d * rb
                                      : reinterpret_cast<const uint8_t *>(sh_scale);
+    float *const gsum = zl.early ? ws.gsum : nullptr;
     for (int b0 = b_lo; b0 < b_hi;) {
         const int left = b_hi - b0;
-        if (left > 8) { route_pass<ACT, RT, 16>(sh, B, b0, ws, row, wrow, hidden, s_dyn); b0 += 16; }
-        else if (left > 4) { route_pass<ACT, RT, 8>(sh, B, b0, ws, row, wrow, hidden, s_dyn); b0 += 8; }
-        else { route_pass<ACT, RT, 4>(sh, B, b0, ws, row, wrow, hidden, s_dyn); b0 += 4; }
+        if (left > 8) { route_pass<ACT, RT, 16>(sh, B, b0, ws, row, wrow, hidden, conf, gsum, s_dyn); b0 += 16; }
+        else if (left > 4) { route_pass<ACT, RT, 8>(sh, B, b0, ws, row, wrow, hidden, conf, gsum, s_dyn); b0 += 8; }
+        else { route_pass<ACT, RT, 4>(sh, B, b0, ws, row, wrow, hidden, conf, gsum, s_dyn); b0 += 4; }
     }
     }
     }
@@ -418,9 +416,8 @@ __device__ __forceinline__ void route_body(const Shape &sh, int B, const Workspa
     // barriers on both sides extend the ordering to the block's other threads; the other blocks
     // wait for nothing.
     if (tid == 0) {
-        unsigned target = 0u;
+        const unsigned target = ticket_target;
         if (blockIdx.x == 0) {
-            target = ticket_base + (unsigned)n_arrive;
             asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(ws.ticket + 1), "r"(target) : "memory");
         }
         unsigned t;
@@ -443,8 +440,10 @@ __device__ __forceinline__ void route_body(const Shape &sh, int B, const Workspa
     gating_block<JE>(sh, B, ws, conf, sh_scale ? 1 : 0, sel_idx, sel_w, n_unique, s_dyn, zl.ksplit, zl.lpart, zl.early);
 }
 
+// (bound of 768 threads instead of 512: at most 80 registers, so that a block fits beside a CTA of the
+// expert kernel, 352 threads x 64 registers)
 template <int ACT, int RT, int JE>
-__global__ void __launch_bounds__(kRouteThreads)
+__global__ void __launch_bounds__(768, 1)
 route_kernel(Shape sh, int B, Workspace ws, const void *__restrict__ hidden, const void *__restrict__ router,
              const void *__restrict__ sh_scale, const float *__restrict__ conf, int32_t *__restrict__ sel_idx,
              float *__restrict__ sel_w, int32_t *__restrict__ n_unique, ZeroList zl)

@@ -202,10 +202,11 @@ cudaLaunchConfig_t pdl_config(s2moe_ctx *ctx, int grid, int block, size_t smem, 
     return lc;
 }
 
-size_t route_smem(int B, int E)
+size_t route_smem(int B, int E, int k)
 {
-    const size_t a = (size_t)B * E + (size_t)B, b = (size_t)(kRouteThreads / 32) * kRouteTok;
-    return sizeof(double) * (a > b ? a : b);
+    const size_t a = sizeof(double) * ((size_t)B * E + (size_t)B) + gate_mem_bytes(E, B, k);
+    const size_t b = sizeof(double) * (size_t)(kRouteThreads / 32) * kRouteTok;
+    return align_up(a > b ? a : b, 16);
 }
 
 template <int ACT, int RT>
@@ -253,7 +254,7 @@ void launch_route_t(s2moe_ctx *ctx, const Shape &sh, const LayerPtrs &lp, int B,
     }
     LaunchScope scope(ctx, KC_ROUTER, st);
     if (zg.ksplit > 0) {
-        cudaLaunchConfig_t lc = pdl_config(ctx, grid, kRouteThreadsBig, route_smem(B, sh.E), st, zl.early != 0);
+        cudaLaunchConfig_t lc = pdl_config(ctx, grid, kRouteThreadsBig, route_smem(B, sh.E, sh.k), st, zl.early != 0);
         if (sh.E <= 64)
             cudaLaunchKernelEx(&lc, route_kernel_big<ACT, RT, 2>, sh, B, ctx->ws, hidden, (const void *)lp.router,
                                (const void *)lp.sh_scale, conf, sel_idx, sel_w, n_unique, zg);
@@ -265,7 +266,7 @@ void launch_route_t(s2moe_ctx *ctx, const Shape &sh, const LayerPtrs &lp, int B,
                                (const void *)lp.sh_scale, conf, sel_idx, sel_w, n_unique, zg);
         return;
     }
-    cudaLaunchConfig_t lc = pdl_config(ctx, grid, kRouteThreads, route_smem(B, sh.E), st, zl.early != 0);
+    cudaLaunchConfig_t lc = pdl_config(ctx, grid, kRouteThreads, route_smem(B, sh.E, sh.k), st, zl.early != 0);
     if (sh.E <= 64)
         cudaLaunchKernelEx(&lc, route_kernel<ACT, RT, 2>, sh, B, ctx->ws, hidden, (const void *)lp.router,
                            (const void *)lp.sh_scale, conf, sel_idx, sel_w, n_unique, zg);
@@ -291,6 +292,11 @@ template <int ACT, int RT>
 cudaError_t prepare_route_t(int bytes)
 {
     cudaError_t e = cudaFuncSetAttribute(route_kernel<ACT, RT, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    // (an SM changes its split between L1 and shared memory only when it is empty: the routing blocks ask
+    // for the split of the expert kernel they share the SMs with)
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(route_kernel<ACT, RT, 2>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(route_kernel<ACT, RT, 4>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(route_kernel<ACT, RT, 8>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(route_kernel<ACT, RT, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(route_kernel<ACT, RT, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(route_kernel_big<ACT, RT, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
@@ -301,7 +307,7 @@ cudaError_t prepare_route_t(int bytes)
 
 cudaError_t prepare_route()
 {
-    const int bytes = (int)route_smem(kMaxTokens, kMaxExperts);
+    const int bytes = (int)route_smem(kMaxTokens, kMaxExperts, kMaxTopK);
     cudaError_t e = prepare_route_t<DT_F32, DT_F32>(bytes);
     if (e == cudaSuccess) e = prepare_route_t<DT_F32, DT_BF16>(bytes);
     if (e == cudaSuccess) e = prepare_route_t<DT_BF16, DT_F32>(bytes);
@@ -517,7 +523,7 @@ int plan_for(const s2moe_ctx *ctx, int B, StPlan *out)
         return tp.feasible ? 4 : 0;
     }
     if ((want == 0 || want == 3) && s0.weight_dtype == DT_BF16) {
-        if (!ctx->rw_maps.empty() && rw_make_plan(s0, B, ctx->n_sm, false).feasible) return 3;
+        if (!ctx->rw_maps.empty() && rw_make_plan(s0, B, ctx->n_sm, false, 0).feasible) return 3;
         if (want == 3) return 0;
     } else if (want == 0 || want == 3) {
         const TcPlan tp = tc_make_plan(s0, B, ctx->n_sm, B * s0.k + s0.n_sh * B, B >= ctx->bf16_kg2_from ? 2 : 1);
@@ -591,7 +597,7 @@ int verify_one(s2moe_ctx *ctx, int layer, int B, const void *hidden, const float
     // fetched between the two kernels)
     const bool want_early = plan == 3 && ctx->early_start && ctx->use_pdl && !ctx->offload && sh.weight_dtype == DT_BF16;
     const bool rows3 = plan == 3 && sh.weight_dtype == DT_BF16;
-    const RwPlan rp = rows3 ? rw_make_plan(sh, B, ctx->n_sm, want_early) : RwPlan{};
+    const RwPlan rp = rows3 ? rw_make_plan(sh, B, ctx->n_sm, want_early, B < ctx->route_task_from ? (int)route_smem(B, sh.E, sh.k) + 256 : 0) : RwPlan{};
     const TcPlan tp3 = plan == 3 && !rows3 ? tc_make_plan(sh, B, ctx->n_sm, B * sh.k + sh.n_sh * B) : TcPlan{};
     // what the FFN kernels accumulate into is cleared by the routing kernel's blocks
     ZeroList zl{};
@@ -609,12 +615,7 @@ int verify_one(s2moe_ctx *ctx, int layer, int B, const void *hidden, const float
             zl.perm_n16 = (size_t)B * sh.d * 2 / 16;
         }
     }
-    if (rows3 && rp.early) {
-        // a token's first expert by original logit stays selected for alpha < 1 (see gating_block);
-        // otherwise only the shared experts start early
-        const bool bias_on = sh.alpha > 0.0 && sh.cap < sh.E && sh.k < sh.E;
-        zl.early = (!bias_on || sh.alpha <= 0.999999) ? 2 : 1;
-    }
+    zl.early = rows3 && rp.early;
     if (plan != 4) launch_route(ctx, sh, lp, B, hidden, conf, sel_idx, sel_w, n_unique, zl, st);
     if (ctx->offload) {
         const int rc = fetch_experts(ctx, layer, st);
@@ -792,7 +793,7 @@ int create_impl(const s2moe_config *config, const s2moe_layer_weights *layers, i
     const size_t o_up1 = take(4 * (size_t)(G + 2)), o_up2 = take(4 * (size_t)(G + 2));
     const size_t o_tm = take(8 * (size_t)G);
     const size_t o_gtab = take(32 * (size_t)(G + 1));
-    const size_t o_early = take(4 * (size_t)(kMaxTokens + 4));
+    const size_t o_early = take(8 * (size_t)(kEarlyWords + 1)), o_gsum = take(4 * (size_t)kMaxExperts);
     const size_t o_hperm = take(sh.weight_dtype == DT_Q4B32 ? 2 * (size_t)T * sh.d : 0);
     const size_t o_lpart = take(sizeof(double) * 8 * (size_t)T * (E + 1));
     const size_t o_sth = take(ab * (size_t)L * T * sh.d), o_stc = take(4 * (size_t)L * T);
@@ -837,7 +838,8 @@ int create_impl(const s2moe_config *config, const s2moe_layer_weights *layers, i
     ws.upfx1 = (int32_t *)(base + o_up1); ws.upfx2 = (int32_t *)(base + o_up2);
     ws.tokmask = (unsigned long long *)(base + o_tm);
     ws.gtab = (uint4 *)(base + o_gtab);
-    ws.early = (int32_t *)(base + o_early);
+    ws.early = (unsigned long long *)(base + o_early);
+    ws.gsum = (float *)(base + o_gsum);
     ctx->hperm = base + o_hperm;
     ctx->lpart = (double *)(base + o_lpart);
     ctx->pre = (float *)(base + o_pre);
@@ -1206,6 +1208,7 @@ int s2moe_last_device_status(s2moe_ctx *ctx, int32_t *host_out)
         // so that the next call starts clean whatever the abandoned wait left behind
         CU(ctx, cudaMemset(ctx->ws.status, 0, 4));
         CU(ctx, cudaMemset(ctx->ws.ticket, 0, 16));
+        CU(ctx, cudaMemset(ctx->ws.gsum, 0, sizeof(float) * kMaxExperts));
         return S2MOE_ETIMEOUT;
     }
     return S2MOE_OK;
@@ -1387,7 +1390,7 @@ int s2moe_route_noalloc(const s2moe_config *cfg, int32_t n_tokens, const void *r
     sh.alpha = (double)cfg->alpha;
     if (cudaMemsetAsync(zero_begin, 0, (size_t)(zero_end - zero_begin), st) != cudaSuccess) return S2MOE_ECUDA;
     const int rows = sh.E + (gate_vec ? 1 : 0);
-    const size_t smem = route_smem(n_tokens, sh.E);
+    const size_t smem = route_smem(n_tokens, sh.E, sh.k);
     const bool af = sh.act_dtype == DT_F32, rf = sh.router_dtype == DT_F32;
     // (the no-allocation entry covers up to 128 experts: two or four per lane in the gating)
 #define S2MOE_ROUTE_NA(A, R)                                                                                         \
