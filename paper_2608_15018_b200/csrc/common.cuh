@@ -14,7 +14,7 @@ constexpr int kMaxTokens = 64;
 constexpr int kMaxExperts = 256;
 constexpr int kMaxTopK = 16;
 constexpr int kMaxShared = 4;
-constexpr int kEarlyWords = kMaxExperts / 32;   // words of one list of Workspace::early
+constexpr int kEarlyWords = kMaxExperts / 32;   // words of the list in Workspace::early
 
 enum : int { DT_F32 = 0, DT_BF16 = 1, DT_Q4B32 = 2 };
 

@@ -84,7 +84,7 @@ struct RwPlan {
     int max_tasks;
     int tab_bytes;
     int smem_bytes;
-    int early, n_early;
+    int early, n_early;           // early start; its experts
     int split16[kRwMaxWaves - 1];   // where waves 1, 2, 3 begin, in 16ths of the first projection (16: no such wave)
     int delta;           // second-projection units that weigh as much as one first-projection unit
     RwDiv gf, gs, tf, ts, kr, ks, rb, p;   // row groups and tasks of a routed / shared expert, P2 units of their row blocks, row blocks, CTAs
@@ -133,7 +133,8 @@ inline RwPlan rw_make_plan(const Shape &sh, int B, int n_sm, bool early, int rou
     const int G = sh.E + sh.n_sh, n_slots = B * sh.k + sh.n_sh * B;
     p.early = early && n_sm > 1;
     // experts whose first projection starts before the gating (see the header comment)
-    p.n_early = p.early ? (sh.k < 4 ? (sh.k == 3 ? 2 : 1) : sh.k) : 0;
+    // (one or two tokens select little more than top_k: some are left for a second wave)
+    p.n_early = p.early ? (sh.k < 4 ? (sh.k == 3 ? 2 : 1) : (B <= 2 ? (3 * sh.k + 2) / 4 : sh.k)) : 0;
     p.n1 = (B + 15) & ~15;
     const int trows = rw_tok_rows(B);
     const int tok2 = 2 * 2 * trows * 128, tok1 = 2 * p.n1 * 128;
@@ -196,11 +197,12 @@ inline RwPlan rw_make_plan(const Shape &sh, int B, int n_sm, bool early, int rou
         if (p.stages >= (res ? 3 : 2)) { p.feasible = 1; break; }
     }
     if (!p.feasible) return p;
-    // Three waves.  Measured, us per layer, waves 1 and 2 from 8/16 and 13/16 / wave 1 from 10/16: OLMoE shape
-    // at 8 tokens 41.3 / 43.2, one token 31.7 / 31.5, DeepSeek-V2-Lite shape at 16 tokens 53.0 / 53.4,
-    // Qwen1.5-MoE shape 43.8 / 44.3, 128 narrow experts at 13 tokens 42.9 / 42.9, 128 wide ones at 8 76.8 / 77.0.
+    // Two waves.  Measured, us per layer, wave 1 from 8/16 / waves 1 and 2 from 8/16 and 13/16: OLMoE shape at 8
+    // tokens 40.9 / 41.0, one token 32.1 / 32.4, DeepSeek-V2-Lite shape at 16 tokens 51.7 / 52.4, at 64
+    // 126.5 / 127.9, Qwen1.5-MoE shape 42.3 / 43.1, 128 narrow experts at 13 tokens 38.3 / 38.2, 128 wide ones
+    // at 8 75.4 / 76.2.
     p.split16[0] = 8;
-    p.split16[1] = 13;
+    p.split16[1] = 16;
     p.split16[2] = 16;
     p.delta = (sh.d + 512) / 1024;
     return p;
@@ -676,29 +678,32 @@ ffn_rows_kernel(const __grid_constant__ RwMaps maps, const __grid_constant__ RwA
                         key[q] = ((f & 0x80000000u ? ~f : f | 0x80000000u) & 0xffffff00u) | (255u - (unsigned)e);
                     }
                 }
+                auto take = [&](auto words) {
 #pragma unroll 1
-                for (int r = 0; r < pl.n_early; ++r) {
-                    unsigned m = max(key[0], key[1]);
-                    if (nwords > 2) {
+                    for (int r = 0; r < pl.n_early; ++r) {
+                        unsigned m = key[0];
 #pragma unroll
-                        for (int q = 2; q < kEarlyWords; ++q) m = max(m, key[q]);
-                    }
-                    m = __reduce_max_sync(0xffffffffu, m);
-                    const int e = 255 - (int)(m & 255u);
-                    if (lane == (e & 31)) {
-                        won |= 1u << (e >> 5);
+                        for (int q = 1; q < words(); ++q) m = max(m, key[q]);
+                        m = __reduce_max_sync(0xffffffffu, m);
 #pragma unroll
-                        for (int q = 0; q < kEarlyWords; ++q)
-                            if (key[q] == m) key[q] = 0u;
+                        for (int q = 0; q < words(); ++q) {
+                            won |= key[q] == m ? 1u << q : 0u;
+                            key[q] = key[q] == m ? 0u : key[q];
+                        }
                     }
-                }
+                };
+                if (nwords <= 2) take([] { return 2; });
+                else take([] { return kEarlyWords; });
+                // (the set as words, lane q: word q, and its experts in ascending order)
                 unsigned w = 0u;
 #pragma unroll 1
                 for (int q = 0; q < nwords; ++q) {
                     const unsigned word = __ballot_sync(0xffffffffu, (won >> q) & 1u);
+                    if ((word >> lane) & 1u) s_id[n_early + __popc(word & ((1u << lane) - 1u))] = (uint16_t)(32 * q + lane);
                     if (lane == q) w = word;
+                    n_early += __popc(word);
                 }
-                n_early = expand(w, 0);
+                __syncwarp();
                 // lot E: their first projection
                 share(n_early * Gf, n_sh_units, start, cnt);
                 const RwSeg sg = rw_seg(start, cnt, pl.gf, 3, (int)pl.tf.d);
@@ -944,7 +949,9 @@ ffn_rows_kernel(const __grid_constant__ RwMaps maps, const __grid_constant__ RwA
         };
         // this set's activations of every wave below `upto` are stored: arrive on the waves' counters
         auto service = [&](int upto) -> bool {
-            if (upto > waves) upto = waves;
+            if (arrived >= min(upto, waves)) return true;
+            if (!wait_level(kRwLevels)) return false;                // (the counters are clear once the routing kernel has ended)
+            upto = min(upto, waves);
             if (arrived >= upto) return true;
             asm volatile("fence.proxy.async.global;" ::: "memory");  // the activations are read by TMA copies of other CTAs
             if (!tc_bar(&ep_bar[set], ep_phase, lane)) return false;

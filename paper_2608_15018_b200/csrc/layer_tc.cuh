@@ -444,7 +444,7 @@ layer_tc_kernel(const __grid_constant__ TcMaps maps, TcArgs p)
         const int E = sh.E, B = p.B, k = sh.k, n_rows = E + (rt.sh_scale ? 1 : 0), n_routed = B * k;
         const int EW = (E + 31) >> 5;                              // bit words of an expert set
         double *s_l = reinterpret_cast<double *>(gate_area), *s_w = s_l + B * E, *s_gl = s_w + B;   // logits, confidences, gate logits
-        const GateMem gm = gate_mem_carve(s_gl + B, E, B, k);
+        const GateMem gm = gate_mem_carve(s_l + ((B * E + 2 * B + 1) & ~1), E, B, k);
         const bool bias_on = sh.alpha > 0.0 && sh.cap < E && k < E;
         // ---- stage the logits: the pieces of a row added in ascending order (all loads first)
 #pragma unroll 1
@@ -537,9 +537,9 @@ layer_tc_kernel(const __grid_constant__ TcMaps maps, TcArgs p)
         gate_sync(gg);
         if (gg.t == 0) s_tab = 1;
         // ---- the gating, first part: E*, lambda_b, every token's first k experts by original logit
-        if (E <= 64) gating_part1<2>(sh, B, s_l, s_w, gg, gm, false, true, true);
-        else if (E <= 128) gating_part1<4>(sh, B, s_l, s_w, gg, gm, false, true, true);
-        else gating_part1<8>(sh, B, s_l, s_w, gg, gm, false, true, true);
+        if (E <= 64) gating_part1<2>(sh, B, s_l, s_w, gg, gm, true, true);
+        else if (E <= 128) gating_part1<4>(sh, B, s_l, s_w, gg, gm, true, true);
+        else gating_part1<8>(sh, B, s_l, s_w, gg, gm, true, true);
         // ---- second lot of early groups: an expert of E* that is among a token's first k stays in that
         // token's top-k whatever the bias does to the others (at most its rank of them pass it), so
         // E* intersected with the union of the tokens' first k can start now
@@ -585,9 +585,9 @@ layer_tc_kernel(const __grid_constant__ TcMaps maps, TcArgs p)
         if (gg.t == 0) s_tab = 2;
         // ---- the gating, second part; CTA 0 also writes the call's outputs
         const bool writer = blockIdx.x == 0;
-        if (E <= 64) gating_part2<2>(sh, B, s_l, gg, gm, writer ? rt.sel_idx : nullptr, writer ? rt.sel_w : nullptr, false);
-        else if (E <= 128) gating_part2<4>(sh, B, s_l, gg, gm, writer ? rt.sel_idx : nullptr, writer ? rt.sel_w : nullptr, false);
-        else gating_part2<8>(sh, B, s_l, gg, gm, writer ? rt.sel_idx : nullptr, writer ? rt.sel_w : nullptr, false);
+        if (E <= 64) gating_part2<2>(sh, B, s_l, gg, gm, writer ? rt.sel_idx : nullptr, writer ? rt.sel_w : nullptr);
+        else if (E <= 128) gating_part2<4>(sh, B, s_l, gg, gm, writer ? rt.sel_idx : nullptr, writer ? rt.sel_w : nullptr);
+        else gating_part2<8>(sh, B, s_l, gg, gm, writer ? rt.sel_idx : nullptr, writer ? rt.sel_w : nullptr);
         // ---- the tables in their final form.  Group order: the early groups, then the other selected
         // experts in ascending order; slots stay in expert order (routed first, then shared).
         const int U = *gm.U, n_active = U + sh.n_sh;

@@ -120,10 +120,10 @@ template <int JE>
 __device__ __forceinline__ void gating_block(const Shape &sh, int B, const Workspace &ws, const float *__restrict__ conf,
                                              int has_gate, int32_t *__restrict__ sel_idx, float *__restrict__ sel_w,
                                              int32_t *__restrict__ n_unique, double *s_l, int ksplit, const double *__restrict__ lpart,
-                                             int early = 0)
+                                             int early)
 {
     // (sized by this batch and not for the largest one: a routing block shares its SM with the expert kernel)
-    const GateMem gm = gate_mem_carve(s_l + B * sh.E + B, sh.E, B, sh.k);
+    const GateMem gm = gate_mem_carve(s_l + ((B * sh.E + B + 1) & ~1), sh.E, B, sh.k);
     const GateGroup gg{(int)threadIdx.x, (int)blockDim.x, 0};
     double *s_w = s_l + B * sh.E;
     if (ksplit > 0) {
@@ -148,9 +148,9 @@ __device__ __forceinline__ void gating_block(const Shape &sh, int B, const Works
     }
 #pragma unroll 1
     for (int b = gg.t; b < B; b += gg.n) s_w[b] = conf ? (double)conf[b] : 1.0;
-    // (gating_group's first barrier orders these writes before the first read)
-    gating_part1<JE>(sh, B, s_l, s_w, gg, gm, true);
-    gating_part2<JE>(sh, B, s_l, gg, gm, sel_idx, sel_w, true, early ? ws.early : nullptr);
+    __syncthreads();                                      // the logits are staged
+    gating_part1<JE>(sh, B, s_l, s_w, gg, gm);
+    gating_part2<JE>(sh, B, s_l, gg, gm, sel_idx, sel_w, early ? ws.early : nullptr);
     gating_writeout(sh, B, ws, gm, has_gate, n_unique, gg);
 }
 
@@ -201,6 +201,36 @@ struct ZeroList {
     int early;
 };
 
+// Sums over the warp of NT values per lane in log2(32) steps for all of them together (halving the
+// number of values a lane holds while that is more than one): lane l ends up with the sum of value
+// l / (32 / NT).  16 values take 16 + 1 shuffles instead of 80.
+template <int NT>
+__device__ __forceinline__ double warp_sums(double (&a)[NT], int lane)
+{
+    int o = 16;
+#pragma unroll
+    for (int n = NT / 2; n > 0; n >>= 1, o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int t = 0; t < n; ++t) {
+            const double send = up ? a[t] : a[t + n], keep = up ? a[t + n] : a[t];
+            a[t] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+    }
+#pragma unroll
+    for (; o > 0; o >>= 1) a[0] += __shfl_xor_sync(0xffffffffu, a[0], o);
+    return a[0];
+}
+
+// x * 2^-896 exactly, subnormal numbers included, by moving the bits of the binary32 number into place (a
+// conversion instruction has a quarter of the rate of the fused multiply-add it feeds); the other
+// factor carries the 2^896
+__device__ __forceinline__ double scaled_double(float x, bool bf16)
+{
+    const uint32_t u = __float_as_uint(x);
+    return __hiloint2double((int)(((u >> 3) & 0x0fffffffu) | (u & 0x80000000u)), bf16 ? 0 : (int)(u << 29));
+}
+
 // Router logits by the warps of the whole grid: a task is one router row (row E: the shared
 // experts' gate vector) x 8 tokens x one piece of the contraction, float64 accumulation; its
 // partial sums go to lpart[piece][token][row], which the gating adds up in a fixed order.
@@ -232,23 +262,24 @@ __device__ __forceinline__ void route_logit_tasks(const Shape &sh, int B, const 
                 const int bt = min(b0 + t, B - 1);           // past the batch: the last token again (not stored)
                 load4_plain<ACT>(reinterpret_cast<const uint8_t *>(hidden) + (size_t)bt * d * ab, c, x[t]);
             }
+            double wd[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) wd[i] = (double)w[i] * 0x1p896;
 #pragma unroll
             for (int t = 0; t < 8; ++t)
 #pragma unroll
-                for (int i = 0; i < 4; ++i) acc[t] = fma((double)w[i], (double)x[t][i], acc[t]);
+                for (int i = 0; i < 4; ++i) acc[t] = fma(wd[i], scaled_double(x[t][i], ACT == DT_BF16), acc[t]);
         }
+        const double v = warp_sums<8>(acc, lane);             // token lane / 4
+        const int bt = b0 + (lane >> 2);
         float g = 0.0f;
-#pragma unroll
-        for (int t = 0; t < 8; ++t) {
-            const double v = warp_sum(acc[t]);
-            if (lane == t && b0 + t < B) {
-                lpart[((size_t)piece * B + b0 + t) * n_rows + row] = v;
-                g = (conf ? conf[b0 + t] : 1.0f) * (float)v;
-            }
+        if ((lane & 3) == 0 && bt < B) {
+            lpart[((size_t)piece * B + bt) * n_rows + row] = v;
+            g = (gsum && conf ? conf[bt] : 1.0f) * (float)v;
         }
         if (gsum && row < sh.E) {
 #pragma unroll
-            for (int o = 4; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
+            for (int o = 16; o > 2; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
             if (lane == 0) atomicAdd(&gsum[row], g);
         }
     }
@@ -261,9 +292,12 @@ __device__ __forceinline__ void route_pass(const Shape &sh, int B, int b0, const
                                            const void *__restrict__ hidden, const float *__restrict__ conf, float *__restrict__ gsum,
                                            double *s_part)
 {
+    static_assert(kRouteThreads == 32 * 16 && NT <= 16, "16 partial sums per token");
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, d = sh.d;
     const size_t ab = ACT == DT_F32 ? 4 : 2;
-    const float wb = (gsum && conf && tid < NT && b0 + tid < B) ? conf[b0 + tid] : 1.0f;
+    const int tok = tid >> 4;                             // token whose partial sums this thread adds up at the end
+    const bool mine = tok < NT && b0 + tok < B;
+    const float wb = (gsum && conf && mine) ? conf[b0 + tok] : 1.0f;
     double acc[NT];
 #pragma unroll
     for (int t = 0; t < NT; ++t) acc[t] = 0.0;
@@ -275,39 +309,37 @@ __device__ __forceinline__ void route_pass(const Shape &sh, int B, int b0, const
             const int bt = min(b0 + t, B - 1);
             load4_plain<ACT>(reinterpret_cast<const uint8_t *>(hidden) + (size_t)bt * d * ab, c, x[t]);
         }
+        double wd[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) wd[i] = (double)w[i] * 0x1p896;
 #pragma unroll
         for (int t = 0; t < NT; ++t)
 #pragma unroll
-            for (int i = 0; i < 4; ++i) acc[t] = fma((double)w[i], (double)x[t][i], acc[t]);
+            for (int i = 0; i < 4; ++i) acc[t] = fma(wd[i], scaled_double(x[t][i], ACT == DT_BF16), acc[t]);
     }
-#pragma unroll
-    for (int t = 0; t < NT; ++t) {
-        const double s = warp_sum(acc[t]);
-        if (lane == 0) s_part[warp * kRouteTok + t] = s;
-    }
+    const double v = warp_sums<NT>(acc, lane);
+    if ((lane & (32 / NT - 1)) == 0) s_part[warp * kRouteTok + lane / (32 / NT)] = v;
     __syncthreads();
-    if (tid < 32) {
-        float g = 0.0f;
-        if (tid < NT && b0 + tid < B) {
-            double s = 0.0;
+    if (tid < 16 * NT) {                                  // (whole warps: two tokens each)
+        double s = s_part[(tid & 15) * kRouteTok + tok];
 #pragma unroll
-            for (int w = 0; w < kRouteThreads / 32; ++w) s += s_part[w * kRouteTok + tid];
-            if (row < sh.E) ws.logits[(size_t)(b0 + tid) * sh.E + row] = s;
-            else ws.gate_logit[b0 + tid] = s;
-            g = wb * (float)s;
+        for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        float g = mine ? wb * (float)s : 0.0f;
+        if ((tid & 15) == 0 && mine) {
+            if (row < sh.E) ws.logits[(size_t)(b0 + tok) * sh.E + row] = s;
+            else ws.gate_logit[b0 + tok] = s;
         }
         if (gsum && row < sh.E) {
-#pragma unroll
-            for (int o = NT >> 1; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
-            if (tid == 0) atomicAdd(&gsum[row], g);
+            g += __shfl_xor_sync(0xffffffffu, g, 16);
+            if (lane == 0) atomicAdd(&gsum[row], g);
         }
     }
     __syncthreads();
 }
 
 // Router logits and gating in one launch.  A block computes one row of the router (row E is the
-// shared-expert gate vector) against one group of the batch's tokens in float64; block 0 then
-// runs the gating for the whole batch once every block has arrived (atomic ticket).
+// shared-expert gate vector) against one group of the batch's tokens in float64; block 0, which has no
+// row, runs the gating for the whole batch once every block has arrived (atomic ticket).
 // Dynamic shared memory: B * E + B doubles and gate_mem_bytes(E, B, k), at least 16 * kRouteTok doubles.
 // JE: experts per lane in the gating (2, 4 or 8 for up to 64, 128, 256 experts): a kernel of its own
 // for each, so that the gating code of a launch is one straight piece
@@ -337,104 +369,98 @@ __device__ __forceinline__ void route_body(const Shape &sh, int B, const Workspa
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // what this block will read first, into L2 while it waits: its router row (the hidden states come from
     // the kernel in front and are there already, or from the caller's memory: a prefetch changes nothing)
-    if (zl.ksplit == 0) {
-        const int n_rows_p = sh.E + (sh_scale ? 1 : 0), row_p = (int)blockIdx.x % n_rows_p;
+    if (zl.ksplit == 0 && blockIdx.x > 0) {
+        const int row_p = ((int)blockIdx.x - 1) % (sh.E + (sh_scale ? 1 : 0));
         const size_t rbytes = (size_t)sh.d * (RT == DT_F32 ? 4 : 2), hbytes = (size_t)B * sh.d * (ACT == DT_F32 ? 4 : 2);
         const uint8_t *wr = row_p < sh.E ? reinterpret_cast<const uint8_t *>(router) + (size_t)row_p * rbytes
                                          : reinterpret_cast<const uint8_t *>(sh_scale);
         const size_t o = (size_t)tid * 128;
         if (o < rbytes) asm volatile("prefetch.global.L2 [%0];" ::"l"(wr + o));
-        const size_t ho = ((size_t)blockIdx.x * THREADS + tid) * 128;
+        const size_t ho = ((size_t)(blockIdx.x - 1) * THREADS + tid) * 128;
         if (ho < hbytes) asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const uint8_t *>(hidden) + ho));
     }
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    // (block 0: where the arrival counter stood when the launch before had ended; see below)
     const int n_rows = sh.E + (sh_scale ? 1 : 0), n_grp = zl.groups > 1 ? zl.groups : 1;
-    // (early start: the expert kernel accumulates into what this grid clears, so the blocks that only clear
-    // arrive on the counter as well)
-    const int n_arrive = zl.early || zl.ksplit > 0 ? (int)gridDim.x : n_rows * n_grp;
+    const int n_arrive = zl.ksplit > 0 ? (int)gridDim.x - 1 : n_rows * n_grp;   // blocks 1 .. n_arrive; those past that only clear
+    const int rblk = (int)blockIdx.x - 1;
+    const size_t rb = RT == DT_F32 ? 4 : 2;
+    // block 0: where the arrival counter stood when the launch before had ended (that launch is over: a
+    // kernel lets this one start only when its own routing kernel has ended); see below
     unsigned ticket_target = 0u;
     if (blockIdx.x == 0 && tid == 0) {
         asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(ticket_target) : "l"(ws.ticket + 1) : "memory");
         ticket_target += (unsigned)n_arrive;
-        if (zl.early)
-            asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(ws.early + kEarlyWords), "l"((1ull << 32) | (unsigned long long)ticket_target)
-                         : "memory");
     }
-#pragma unroll
-    for (int z = 0; z < 3; ++z) {
-        uint4 *p = reinterpret_cast<uint4 *>(zl.ptr[z]);
-        for (unsigned long long i = (unsigned long long)blockIdx.x * THREADS + tid; i < zl.n16[z];
-             i += (unsigned long long)gridDim.x * THREADS)
-            p[i] = make_uint4(0u, 0u, 0u, 0u);
-    }
-    for (unsigned long long i = (unsigned long long)blockIdx.x * THREADS + tid; i < zl.perm_n16;
-         i += (unsigned long long)gridDim.x * THREADS) {
-        const uint4 v = zl.perm_src[i];             // halves h0..h7 (bf16)
-        zl.perm_dst[i] = make_uint4(bf16x2_to_f16x2(__byte_perm(v.x, v.z, 0x5410)), bf16x2_to_f16x2(__byte_perm(v.x, v.z, 0x7632)),
-                                    bf16x2_to_f16x2(__byte_perm(v.y, v.w, 0x5410)), bf16x2_to_f16x2(__byte_perm(v.y, v.w, 0x7632)));
-    }
-    // blocks past the router's rows exist only to help with the clearing and the copy above (a
-    // layer with few experts and wide accumulators would otherwise clear megabytes with a few blocks)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (zl.early && blockIdx.x == 0 && tid == 0)
+        asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(ws.early + kEarlyWords), "l"((1ull << 32) | (unsigned long long)ticket_target)
+                     : "memory");
     // A row block takes one router row and one group of tokens: a larger batch is split over
     // several sets of row blocks (as many as fit on the SMs beside each other), because a block
     // takes 16 tokens per pass and its passes run one after the other (B = 64: 22 us in one set).
     if (zl.ksplit > 0) {
-        // larger batches: the logit pass as warp tasks over all blocks of the grid (a row block takes
-        // 16 tokens per pass and its passes run one after the other: 22 us at 64 tokens)
-        route_logit_tasks<ACT, RT>(sh, B, hidden, router, sh_scale, zl.lpart, zl.ksplit, conf, zl.early ? ws.gsum : nullptr, (tid >> 5) * (int)gridDim.x + (int)blockIdx.x,
-                                   (THREADS / 32) * (int)gridDim.x, tid & 31);
+        // larger batches: the logit pass as warp tasks over all blocks but the first
+        if (rblk >= 0)
+            route_logit_tasks<ACT, RT>(sh, B, hidden, router, sh_scale, zl.lpart, zl.ksplit, conf, zl.early ? ws.gsum : nullptr, (tid >> 5) * n_arrive + rblk,
+                                       (THREADS / 32) * n_arrive, tid & 31);
         __syncthreads();
     } else if constexpr (THREADS == kRouteThreads) {
-    if ((int)blockIdx.x >= n_arrive) return;
-    if ((int)blockIdx.x < n_rows * n_grp) {
-    const int row = (int)blockIdx.x % n_rows, grp = (int)blockIdx.x / n_rows, d = sh.d;
-    const int tg = 4 * ((B + 4 * n_grp - 1) / (4 * n_grp));            // tokens per group, a multiple of 4
-    const int b_lo = min(B, grp * tg), b_hi = min(B, b_lo + tg);
-    const size_t rb = RT == DT_F32 ? 4 : 2;
-    const uint8_t *wrow = row < sh.E ? reinterpret_cast<const uint8_t *>(router) + (size_t)row * d * rb
-                                     : reinterpret_cast<const uint8_t *>(sh_scale);
-    float *const gsum = zl.early ? ws.gsum : nullptr;
-    for (int b0 = b_lo; b0 < b_hi;) {
-        const int left = b_hi - b0;
-        if (left > 8) { route_pass<ACT, RT, 16>(sh, B, b0, ws, row, wrow, hidden, conf, gsum, s_dyn); b0 += 16; }
-        else if (left > 4) { route_pass<ACT, RT, 8>(sh, B, b0, ws, row, wrow, hidden, conf, gsum, s_dyn); b0 += 8; }
-        else { route_pass<ACT, RT, 4>(sh, B, b0, ws, row, wrow, hidden, conf, gsum, s_dyn); b0 += 4; }
+        if (rblk >= 0 && rblk < n_arrive) {
+            const int row = rblk % n_rows, grp = rblk / n_rows;
+            const int tg = 4 * ((B + 4 * n_grp - 1) / (4 * n_grp));            // tokens per group, a multiple of 4
+            const int b_lo = min(B, grp * tg), b_hi = min(B, b_lo + tg);
+            const uint8_t *wrow = row < sh.E ? reinterpret_cast<const uint8_t *>(router) + (size_t)row * sh.d * rb
+                                             : reinterpret_cast<const uint8_t *>(sh_scale);
+            float *const gsum = zl.early ? ws.gsum : nullptr;
+            for (int b0 = b_lo; b0 < b_hi;) {
+                const int left = b_hi - b0;
+                if (left > 8) { route_pass<ACT, RT, 16>(sh, B, b0, ws, row, wrow, hidden, conf, gsum, s_dyn); b0 += 16; }
+                else if (left > 4) { route_pass<ACT, RT, 8>(sh, B, b0, ws, row, wrow, hidden, conf, gsum, s_dyn); b0 += 8; }
+                else { route_pass<ACT, RT, 4>(sh, B, b0, ws, row, wrow, hidden, conf, gsum, s_dyn); b0 += 4; }
+            }
+        }
     }
-    }
-    }
-    if (zl.early) __syncthreads();                        // all of this block's clearing, before its arrival
     // Block 0 runs the gating once every row has arrived (its SM tends to be the same from layer
     // to layer, so part of the gating code is still in its instruction cache: measured 0.6 % of
-    // a layer against letting the last block to arrive do it).  Every block adds one arrival, with
-    // release and acquire semantics by one thread, to a counter that is never reset; block 0
+    // a layer against letting the last block to arrive do it).  Every row block adds one arrival, released
+    // by one thread, to a counter that is never reset; block 0
     // polls it, bounded, for the value it has when all blocks of THIS launch have arrived: the
     // value it will end on was left in the word behind the counter by the launch before (launches of
     // a context follow each other in stream order), and block 0 leaves the next one there, whether
     // its wait succeeded or not, since the late blocks still arrive.  So a wait that ran out poisons
-    // nothing, and the waiting path is one atomic and one polled load, as short as it can be.  The
+    // nothing, and the waiting path is one reduction and one polled load, as short as it can be.  The
     // barriers on both sides extend the ordering to the block's other threads; the other blocks
     // wait for nothing.
-    if (tid == 0) {
-        const unsigned target = ticket_target;
-        if (blockIdx.x == 0) {
-            asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(ws.ticket + 1), "r"(target) : "memory");
-        }
-        unsigned t;
-        asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(t) : "l"(ws.ticket) : "memory");
+    if (tid == 0 && rblk >= 0 && rblk < n_arrive)
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(ws.ticket) : "memory");
+    if (blockIdx.x == 0 && tid == 0) {
+        asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(ws.ticket + 1), "r"(ticket_target) : "memory");
         int ok = 0;
-        if (blockIdx.x == 0) {
-            ok = (int)(t + 1u - target) >= 0 ? 1 : 0;
-            for (unsigned i = 0; i < (1u << 22) && !ok; ++i) {
-                unsigned v;
-                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(ws.ticket) : "memory");
-                if ((int)(v - target) >= 0) ok = 1;
-                else __nanosleep(20);
-            }
-            if (!ok) atomicExch(ws.status, ST_TICKET_TIMEOUT);
+        for (unsigned i = 0; i < (1u << 22) && !ok; ++i) {
+            unsigned v;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(ws.ticket) : "memory");
+            if ((int)(v - ticket_target) >= 0) ok = 1;
+            else __nanosleep(20);
         }
+        if (!ok) atomicExch(ws.status, ST_TICKET_TIMEOUT);
         s_last = ok;
     }
+    // What the kernels behind accumulate into is cleared after the arrival (they touch it once this grid
+    // has ended), by all blocks but the one that runs the gating.
+    if (blockIdx.x > 0) {
+        const unsigned first = blockIdx.x - 1u, blocks = gridDim.x - 1u;
+#pragma unroll
+        for (int z = 0; z < 3; ++z) {
+            uint4 *p = reinterpret_cast<uint4 *>(zl.ptr[z]);
+            for (unsigned long long i = (unsigned long long)first * THREADS + tid; i < zl.n16[z]; i += (unsigned long long)blocks * THREADS)
+                p[i] = make_uint4(0u, 0u, 0u, 0u);
+        }
+        for (unsigned long long i = (unsigned long long)first * THREADS + tid; i < zl.perm_n16; i += (unsigned long long)blocks * THREADS) {
+            const uint4 v = zl.perm_src[i];             // halves h0..h7 (bf16)
+            zl.perm_dst[i] = make_uint4(bf16x2_to_f16x2(__byte_perm(v.x, v.z, 0x5410)), bf16x2_to_f16x2(__byte_perm(v.x, v.z, 0x7632)),
+                                        bf16x2_to_f16x2(__byte_perm(v.y, v.w, 0x5410)), bf16x2_to_f16x2(__byte_perm(v.y, v.w, 0x7632)));
+        }
+    }
+    if (blockIdx.x > 0) return;
     __syncthreads();
     if (!s_last) return;
     gating_block<JE>(sh, B, ws, conf, sh_scale ? 1 : 0, sel_idx, sel_w, n_unique, s_dyn, zl.ksplit, zl.lpart, zl.early);

@@ -204,7 +204,7 @@ cudaLaunchConfig_t pdl_config(s2moe_ctx *ctx, int grid, int block, size_t smem, 
 
 size_t route_smem(int B, int E, int k)
 {
-    const size_t a = sizeof(double) * ((size_t)B * E + (size_t)B) + gate_mem_bytes(E, B, k);
+    const size_t a = sizeof(double) * ((size_t)B * E + (size_t)B + 1) + gate_mem_bytes(E, B, k);
     const size_t b = sizeof(double) * (size_t)(kRouteThreads / 32) * kRouteTok;
     return align_up(a > b ? a : b, 16);
 }
@@ -242,7 +242,7 @@ void launch_route_t(s2moe_ctx *ctx, const Shape &sh, const LayerPtrs &lp, int B,
         if (want > (unsigned long long)grid) grid = (int)(want > (unsigned long long)ctx->n_sm ? (unsigned long long)ctx->n_sm : want);
     } else {
     if (B > 4) {
-        const int fit = ctx->n_sm / rows, want = (B + 3) / 4;
+        const int fit = (ctx->n_sm - 1) / rows, want = (B + 3) / 4;
         zg.groups = fit < 1 ? 1 : (want < fit ? want : fit);
     }
     grid = rows * zg.groups;
@@ -252,6 +252,8 @@ void launch_route_t(s2moe_ctx *ctx, const Shape &sh, const LayerPtrs &lp, int B,
         if (grid < rows * zg.groups) grid = rows * zg.groups;
     }
     }
+    // (and block 0, which runs the gating; not more than one block per SM: a second one would wait for the first)
+    if (grid < ctx->n_sm || grid == rows * zg.groups) ++grid;
     LaunchScope scope(ctx, KC_ROUTER, st);
     if (zg.ksplit > 0) {
         cudaLaunchConfig_t lc = pdl_config(ctx, grid, kRouteThreadsBig, route_smem(B, sh.E, sh.k), st, zl.early != 0);
@@ -1396,10 +1398,10 @@ int s2moe_route_noalloc(const s2moe_config *cfg, int32_t n_tokens, const void *r
 #define S2MOE_ROUTE_NA(A, R)                                                                                         \
     do {                                                                                                             \
         if (sh.E <= 64)                                                                                              \
-            route_kernel<A, R, 2><<<rows, kRouteThreads, smem, st>>>(sh, n_tokens, ws, hidden, router, gate_vec, conf, \
+            route_kernel<A, R, 2><<<rows + 1, kRouteThreads, smem, st>>>(sh, n_tokens, ws, hidden, router, gate_vec, conf, \
                                                                      sel_idx, sel_w, n_unique, ZeroList{});          \
         else                                                                                                         \
-            route_kernel<A, R, 4><<<rows, kRouteThreads, smem, st>>>(sh, n_tokens, ws, hidden, router, gate_vec, conf, \
+            route_kernel<A, R, 4><<<rows + 1, kRouteThreads, smem, st>>>(sh, n_tokens, ws, hidden, router, gate_vec, conf, \
                                                                      sel_idx, sel_w, n_unique, ZeroList{});          \
     } while (0)
     if (af && rf) S2MOE_ROUTE_NA(DT_F32, DT_F32);
