@@ -22,6 +22,14 @@ __device__ __forceinline__ float warp_sum_f(float v)
     return v;
 }
 
+// Programmatic dependent launch (both instructions do nothing in a plain launch): the kernel in front
+// must have ended before anything it wrote is read; the one behind may come up from then on.
+__device__ __forceinline__ void simple_dependency()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 struct GroupView {
     const uint8_t *gate, *up, *down;        // first row of this group's matrices
     const uint8_t *sgate, *sup, *sdown;     // first scale
@@ -65,6 +73,7 @@ __global__ void __launch_bounds__(kSimpleWarps * 32)
 ffn_gateup_simple(Shape sh, LayerPtrs lp, Workspace ws, const void *__restrict__ hidden)
 {
     extern __shared__ float s_x[];  // [tok chunk][k chunk]
+    simple_dependency();
     if ((int)blockIdx.y >= ws.header[0]) return;
     const int group = ws.active[blockIdx.y];
     const GroupView g = group_view(sh, lp, ws, group);
@@ -134,6 +143,7 @@ __global__ void __launch_bounds__(kSimpleWarps * 32)
 ffn_down_simple(Shape sh, LayerPtrs lp, Workspace ws, float *__restrict__ y)
 {
     extern __shared__ float s_x[];
+    simple_dependency();
     if ((int)blockIdx.y >= ws.header[0]) return;
     const int group = ws.active[blockIdx.y];
     const GroupView g = group_view(sh, lp, ws, group);

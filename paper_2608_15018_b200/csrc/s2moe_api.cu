@@ -325,16 +325,19 @@ void launch_simple(s2moe_ctx *ctx, const LayerPtrs &lp, const void *hidden, floa
     const Shape &sh = ctx->shape;
     const int groups = sh.E + sh.n_sh;
     const int fmax = sh.n_sh > 0 && sh.f_sh > sh.f ? sh.f_sh : sh.f;
-    const dim3 block(kSimpleWarps * 32);
     const dim3 g1((fmax + kSimpleWarps - 1) / kSimpleWarps, groups);
     const dim3 g2((sh.d + kSimpleWarps - 1) / kSimpleWarps, groups);
     {
         LaunchScope scope(ctx, KC_GATEUP, st);
-        ffn_gateup_simple<WT, ACT><<<g1, block, kSimpleSmem, st>>>(sh, lp, ctx->ws, hidden);
+        cudaLaunchConfig_t lc = pdl_config(ctx, 1, kSimpleWarps * 32, kSimpleSmem, st);
+        lc.gridDim = g1;
+        cudaLaunchKernelEx(&lc, ffn_gateup_simple<WT, ACT>, sh, lp, ctx->ws, hidden);
     }
     {
         LaunchScope scope(ctx, KC_DOWN, st);
-        ffn_down_simple<WT><<<g2, block, kSimpleSmem, st>>>(sh, lp, ctx->ws, out);
+        cudaLaunchConfig_t lc = pdl_config(ctx, 1, kSimpleWarps * 32, kSimpleSmem, st);
+        lc.gridDim = g2;
+        cudaLaunchKernelEx(&lc, ffn_down_simple<WT>, sh, lp, ctx->ws, out);
     }
 }
 
