@@ -60,8 +60,6 @@ struct Workspace {
     int32_t *upfx1;        // [n_active + 1] first phase-1 stage of each active group
     int32_t *upfx2;        // [n_active + 1] first phase-2 stage of each active group
     unsigned long long *tokmask;   // [E + n_sh] bit b set: token b is bucketed to the group
-    uint4 *gtab;           // [n_active][2] {group, tokens, first slot, 0}, {mask lo, mask hi, 0, 0}: the
-                           // active groups in their final form, or NULL when nobody reads it
     unsigned long long *early;   // kEarlyWords + 1 words, or NULL.  {1 << 32 | bits of 32 experts}: the selected experts, as soon as
                            // they are known; the last word: {1 << 32 | value of the arrival counter when all routing
                            // blocks of the launch have arrived}, once the launch's inputs may be read

@@ -50,7 +50,7 @@
 #include <cuda.h>
 
 #include "common.cuh"
-#include "ffn_tc.cuh"
+#include "tc_common.cuh"
 
 namespace s2moe {
 
@@ -208,16 +208,6 @@ inline RwPlan rw_make_plan(const Shape &sh, int B, int n_sm, bool early, int rou
     return p;
 }
 
-__device__ __forceinline__ bool rw_elect()
-{
-    uint32_t p;
-    asm volatile(
-        "{\n\t.reg .pred P;\n\t"
-        "elect.sync _|P, 0xffffffff;\n\t"
-        "selp.u32 %0, 1, 0, P;\n\t}"
-        : "=r"(p));
-    return p != 0;
-}
 __device__ __forceinline__ void rw_tma_gateup(uint32_t dst, const CUtensorMap *map, int kt, int grp, uint32_t bar, uint64_t policy)
 {
     asm volatile(
@@ -413,7 +403,7 @@ ffn_rows_kernel(const __grid_constant__ RwMaps maps, const __grid_constant__ RwA
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
-        if (rw_elect()) {
+        if (tc_elect()) {
             const uint64_t wpolicy = l2_evict_first_policy();
             const uint32_t ring_a = smem_u32(ring), full_a = smem_u32(full_bar);
             int s = 0, lim = lim0, level = 0, ready_w = 0;
@@ -531,7 +521,7 @@ ffn_rows_kernel(const __grid_constant__ RwMaps maps, const __grid_constant__ RwA
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer
-        if (rw_elect()) {
+        if (tc_elect()) {
             bool alive = true, x_there = pl.x_bytes == 0;
             if (pl.x_bytes && (alive = inputs_wait())) {
                 // the hidden states' tiles, eight k-tiles per copy (past the end: zeros)

@@ -1,5 +1,5 @@
-// The whole verification layer in ONE launch (kernel plan 4): the tcgen05 expert kernel of
-// ffn_tc.cuh with a routing stage in front of its roles.
+// The whole verification layer in ONE launch (kernel plan 4): a split-K tcgen05 expert kernel with a
+// routing stage in front of its roles.
 //
 // Its CTAs first clear what the layer accumulates into and share the router's logit pass (a task
 // is one router row x 8 tokens x one piece of the contraction, float64), meet once (a bounded
@@ -13,7 +13,7 @@
 // (up to eight buffers) until the gating has produced the token lists their epilogue needs.
 // CTA 0 writes the layer's routing outputs.
 //
-// Measured on B200 against the two launches of plans 3 (routing kernel, then ffn_tc_kernel): slower
+// Measured on B200 against the two launches of plans 3 (routing kernel, then the split-K expert kernel they had then): slower
 // on every workload here (OLMoE shape 56.7 against 49.8 us per layer, DeepSeek-V2-Lite shape 70.8
 // against 63.4, Qwen1.5-MoE shape 64.2 against 57.6, Mixtral int4 167 against 140): inside the busy
 // CTAs the gating takes two to three times as long as on a block of its own (its last table is
@@ -22,16 +22,22 @@
 // is offered on demand and the two-launch form stays the default.
 //
 // Everything that is the same in both kernels (PTX helpers, group table, tensor maps, the roles'
-// inner loops) follows ffn_tc.cuh; the differences are the routing stage, the staged unit tables
+// inner loops) follows ffn_q4.cuh; the differences are the routing stage, the staged unit tables
 // (more_units), the eight segments and the number of accumulator buffers.
 #pragma once
 
-#include "ffn_tc.cuh"
+#include "tc_common.cuh"
 #include "gating.cuh"
 #include "route.cuh"
 
 namespace s2moe {
 namespace fused {
+
+constexpr int kTcThreads = 352;                // warps: producer, MMA issuer 0, 4 epilogue, MMA issuer 1, 4 converters
+constexpr int kTcQ4DeqWarps = 8;               // block-int4 weights: warps that dequantise
+constexpr int kTcQ4Threads = kTcThreads + 32 * kTcQ4DeqWarps + 64;   // ... and two more MMA issuers behind them
+constexpr int kTcMaxAStages = 6;               // stages of dequantised weight tiles
+constexpr int kTcMaxUnits = 192;               // units of one CTA decoded once into shared memory
 
 struct TcPlan {
     int feasible;
@@ -690,7 +696,6 @@ layer_tc_kernel(const __grid_constant__ TcMaps maps, TcArgs p)
         if (writer) {
             // the layer's routing outputs and the bucketing arrays in the workspace (debug reads)
             Workspace wsw = ws;
-            wsw.gtab = nullptr;
             for (int b = gg.t; b < B; b += gg.n) ws.gate_logit[b] = s_gl[b];
             for (int i = gg.t; i < B * E; i += gg.n) ws.logits[i] = s_l[i];
             gate_sync(gg);
@@ -773,7 +778,7 @@ layer_tc_kernel(const __grid_constant__ TcMaps maps, TcArgs p)
                     // packed k-tiles (32 bytes of every row each) and the 8 scales per row of the 256
                     // columns they lie in (x in scales; kt0 is a multiple of 4)
                     const int mi = (shared ? 3 : 0) + pu.mat;
-                    const CUtensorMap *pm = &maps.m[KG == 1 ? mi : (KG == 2 ? 15 + mi : 21 + mi)];
+                    const CUtensorMap *pm = &maps.m[mi];
                     uint8_t *stage = ring + (size_t)s * pl.stage_bytes;
                     mbar_expect_tx(&full_bar[s], KG * kTcQ4Packed + kTcQ4Scales);
                     tma_load_2d_stream(stage, pm, pkt * 32, row0, &full_bar[s], wpolicy);

@@ -28,13 +28,7 @@ __device__ __forceinline__ void gating_writeout(const Shape &sh, int B, const Wo
         ws.counts[e] = gm.cnt[e];
         ws.offsets[e] = gm.off[e];
         ws.tokmask[e] = gm.mask[e];
-        if (gm.cnt[e] > 0) {
-            ws.active[gm.pos[e]] = e;
-            if (ws.gtab) {
-                ws.gtab[2 * gm.pos[e]] = make_uint4((unsigned)e, (unsigned)gm.cnt[e], (unsigned)gm.off[e], 0u);
-                ws.gtab[2 * gm.pos[e] + 1] = make_uint4((unsigned)gm.mask[e], (unsigned)(gm.mask[e] >> 32), 0u, 0u);
-            }
-        }
+        if (gm.cnt[e] > 0) ws.active[gm.pos[e]] = e;
     }
     // bucket the (token, choice) pairs: tokens ascending inside an expert
 #pragma unroll 1
@@ -59,10 +53,6 @@ __device__ __forceinline__ void gating_writeout(const Shape &sh, int B, const Wo
             ws.offsets[E + s] = n_routed + s * B;
             ws.active[U + s] = E + s;
             ws.tokmask[E + s] = all;
-            if (ws.gtab) {
-                ws.gtab[2 * (U + s)] = make_uint4((unsigned)(E + s), (unsigned)B, (unsigned)(n_routed + s * B), 0u);
-                ws.gtab[2 * (U + s) + 1] = make_uint4((unsigned)all, (unsigned)(all >> 32), 0u, 0u);
-            }
         }
     }
     if (sh.plan == 2) {
@@ -185,7 +175,7 @@ struct ZeroList {
     unsigned long long n16[3];
     // int4 tensor-core path: a binary16 copy of the bf16 hidden states whose columns are permuted
     // inside every group of 8 (position p holds column [0,4,1,5,2,6,3,7][p]), the order in which
-    // the dequantising warps of the FFN kernel get the nibbles of a 32-bit word for free
+    // the dequantising warps of the expert kernel get the nibbles of a 32-bit word for free
     const uint4 *perm_src;
     uint4 *perm_dst;
     unsigned long long perm_n16;
@@ -394,6 +384,16 @@ __device__ __forceinline__ void route_body(const Shape &sh, int B, const Workspa
     if (zl.early && blockIdx.x == 0 && tid == 0)
         asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(ws.early + kEarlyWords), "l"((1ull << 32) | (unsigned long long)ticket_target)
                      : "memory");
+    // (before the logit pass, whose end and arrival release it: the expert kernel copies it with TMA as soon as
+    // all blocks have arrived)
+    if (zl.perm_n16 && rblk >= 0 && rblk < n_arrive) {
+        for (unsigned long long i = (unsigned long long)rblk * THREADS + tid; i < zl.perm_n16; i += (unsigned long long)n_arrive * THREADS) {
+            const uint4 v = zl.perm_src[i];             // halves h0..h7 (bf16)
+            zl.perm_dst[i] = make_uint4(bf16x2_to_f16x2(__byte_perm(v.x, v.z, 0x5410)), bf16x2_to_f16x2(__byte_perm(v.x, v.z, 0x7632)),
+                                        bf16x2_to_f16x2(__byte_perm(v.y, v.w, 0x5410)), bf16x2_to_f16x2(__byte_perm(v.y, v.w, 0x7632)));
+        }
+        asm volatile("fence.proxy.async.global;" ::: "memory");
+    }
     // A row block takes one router row and one group of tokens: a larger batch is split over
     // several sets of row blocks (as many as fit on the SMs beside each other), because a block
     // takes 16 tokens per pass and its passes run one after the other (B = 64: 22 us in one set).
@@ -453,11 +453,6 @@ __device__ __forceinline__ void route_body(const Shape &sh, int B, const Workspa
             uint4 *p = reinterpret_cast<uint4 *>(zl.ptr[z]);
             for (unsigned long long i = (unsigned long long)first * THREADS + tid; i < zl.n16[z]; i += (unsigned long long)blocks * THREADS)
                 p[i] = make_uint4(0u, 0u, 0u, 0u);
-        }
-        for (unsigned long long i = (unsigned long long)first * THREADS + tid; i < zl.perm_n16; i += (unsigned long long)blocks * THREADS) {
-            const uint4 v = zl.perm_src[i];             // halves h0..h7 (bf16)
-            zl.perm_dst[i] = make_uint4(bf16x2_to_f16x2(__byte_perm(v.x, v.z, 0x5410)), bf16x2_to_f16x2(__byte_perm(v.x, v.z, 0x7632)),
-                                        bf16x2_to_f16x2(__byte_perm(v.y, v.w, 0x5410)), bf16x2_to_f16x2(__byte_perm(v.y, v.w, 0x7632)));
         }
     }
     if (blockIdx.x > 0) return;

@@ -14,7 +14,7 @@
 #include "ffn_simple.cuh"
 #include "ffn_stream.cuh"
 #include "expand.cuh"
-#include "ffn_tc.cuh"
+#include "ffn_q4.cuh"
 #include "ffn_rows.cuh"
 #include "route.cuh"
 #include "layer_tc.cuh"
@@ -46,8 +46,6 @@ struct s2moe_ctx {
     double *lpart = nullptr;              // partial router logits [piece][token][row] (logit pass by warp tasks)
     int route_task_from = 48;             // batches of this many tokens and more take the logit pass by warp tasks
     bool early_start = true;              // bf16 tensor-core plan: the expert kernel starts under the gating (S2MOE_NO_EARLY=1: off)
-    int wave_split[2] = {0, 16};          // S2MOE_WAVES=a,b: where waves 1 and 2 of the bf16 expert kernel begin (16ths; 0: the built-in)
-    int bf16_kg2_from = 2;                // batches of this many tokens and more: two k-tiles per ring stage (bf16)
     float *pre = nullptr;                 // plan 3: fp32 pre-activations [gate|up][slot][f]
     std::vector<TcMaps> tc_maps;          // plan 3: per layer, weight maps filled at create
     std::vector<RwMaps> rw_maps;          // plan 3 with bf16 weights: the same for ffn_rows_kernel
@@ -381,9 +379,9 @@ bool make_map(const s2moe_ctx *ctx, CUtensorMap *out, const void *base, uint64_t
 }
 
 // 2-D tensor of `elem_bytes`-wide elements [rows][cols], box = box_cols x 128 rows (packed int4
-// weights as bytes, their scales as 16-bit words); out-of-range elements read as zero.  Byte boxes
-// of 32, 64 or 128 bytes are swizzled over their own width, so that threads which each read one
-// 16-byte chunk of consecutive rows do not meet in the same shared-memory banks.
+// weights as bytes, their scales as 16-bit words); out-of-range elements read as zero.  The byte boxes
+// of 128 columns are swizzled, so that threads which each read one 16-byte chunk of consecutive rows
+// do not meet in the same shared-memory banks.
 bool make_map_plain(const s2moe_ctx *ctx, CUtensorMap *out, const void *base, uint64_t rows, uint64_t cols,
                     uint32_t box_cols, int elem_bytes)
 {
@@ -395,10 +393,7 @@ bool make_map_plain(const s2moe_ctx *ctx, CUtensorMap *out, const void *base, ui
     return ((EncodeTiledFn)ctx->encode_tiled)(out, elem_bytes == 1 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_UINT16,
                                               2, const_cast<void *>(base), dims, strides, box, estr,
                                               CU_TENSOR_MAP_INTERLEAVE_NONE,
-                                              elem_bytes != 1   ? CU_TENSOR_MAP_SWIZZLE_NONE
-                                              : box_cols == 128 ? CU_TENSOR_MAP_SWIZZLE_128B
-                                              : box_cols == 64  ? CU_TENSOR_MAP_SWIZZLE_64B
-                                                                : CU_TENSOR_MAP_SWIZZLE_32B,
+                                              elem_bytes == 1 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
                                               CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                                               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
@@ -412,21 +407,6 @@ bool make_map_hilo(const s2moe_ctx *ctx, CUtensorMap *out, const void *base, uin
     const cuuint64_t dims[3] = {cols, rows, 2};
     const cuuint64_t strides[2] = {cols * 2, plane_bytes};
     const cuuint32_t box[3] = {64, box_rows, 2};
-    const cuuint32_t estr[3] = {1, 1, 1};
-    return ((EncodeTiledFn)ctx->encode_tiled)(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(base), dims,
-                                              strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                                              CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-// bf16 weights as {64 columns, rows, k-tiles of 64 columns}, box = 64 x 128 x 2: two k-tiles of a
-// 128-row block in one copy, each a 16 KiB tile with the 128-byte swizzle
-bool make_map_w2(const s2moe_ctx *ctx, CUtensorMap *out, const void *base, uint64_t rows, uint64_t cols)
-{
-    if (!ctx->encode_tiled || !base || rows == 0 || cols % 64) return false;
-    const cuuint64_t dims[3] = {64, rows, cols / 64};
-    const cuuint64_t strides[2] = {cols * 2, 128};
-    const cuuint32_t box[3] = {64, 128, 2};
     const cuuint32_t estr[3] = {1, 1, 1};
     return ((EncodeTiledFn)ctx->encode_tiled)(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(base), dims,
                                               strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -531,8 +511,7 @@ int plan_for(const s2moe_ctx *ctx, int B, StPlan *out)
         if (!ctx->rw_maps.empty() && rw_make_plan(s0, B, ctx->n_sm, false, 0).feasible) return 3;
         if (want == 3) return 0;
     } else if (want == 0 || want == 3) {
-        const TcPlan tp = tc_make_plan(s0, B, ctx->n_sm, B * s0.k + s0.n_sh * B, B >= ctx->bf16_kg2_from ? 2 : 1);
-        if (tp.feasible && !ctx->tc_maps.empty()) return 3;
+        if (!ctx->tc_maps.empty() && q4_make_plan(s0, B, ctx->n_sm, false).feasible) return 3;
         if (want == 3) return 0;
     }
     const StPlan pl = st_make_plan(s0, B, ctx->n_sm, B * s0.k + s0.n_sh * B);
@@ -597,13 +576,13 @@ int verify_one(s2moe_ctx *ctx, int layer, int B, const void *hidden, const float
     if (plan == 0) return S2MOE_EINVAL;
     sh.plan = plan;
     sh.op_cap = pl.op_cap;
-    // tensor-core plan with bf16 weights: the expert kernel starts while the gating still runs, on the
-    // experts the routing kernel announces before it (not with offloaded experts: their weights are
-    // fetched between the two kernels)
-    const bool want_early = plan == 3 && ctx->early_start && ctx->use_pdl && !ctx->offload && sh.weight_dtype == DT_BF16;
+    // tensor-core plan: the expert kernel starts while the gating still runs, on what the routing kernel
+    // announces (not with offloaded experts: their weights are fetched between the two kernels)
+    const bool want_early = plan == 3 && ctx->early_start && ctx->use_pdl && !ctx->offload;
     const bool rows3 = plan == 3 && sh.weight_dtype == DT_BF16;
     const RwPlan rp = rows3 ? rw_make_plan(sh, B, ctx->n_sm, want_early, B < ctx->route_task_from ? (int)route_smem(B, sh.E, sh.k) + 256 : 0) : RwPlan{};
-    const TcPlan tp3 = plan == 3 && !rows3 ? tc_make_plan(sh, B, ctx->n_sm, B * sh.k + sh.n_sh * B) : TcPlan{};
+    const bool q4_3 = plan == 3 && !rows3;
+    const Q4Plan qp = q4_3 ? q4_make_plan(sh, B, ctx->n_sm, want_early) : Q4Plan{};
     // what the FFN kernels accumulate into is cleared by the routing kernel's blocks
     ZeroList zl{};
     zl.ptr[0] = out;
@@ -620,7 +599,7 @@ int verify_one(s2moe_ctx *ctx, int layer, int B, const void *hidden, const float
             zl.perm_n16 = (size_t)B * sh.d * 2 / 16;
         }
     }
-    zl.early = rows3 && rp.early;
+    zl.early = (rows3 && rp.early) || (q4_3 && qp.early);
     if (plan != 4) launch_route(ctx, sh, lp, B, hidden, conf, sel_idx, sel_w, n_unique, zl, st);
     if (ctx->offload) {
         const int rc = fetch_experts(ctx, layer, st);
@@ -650,44 +629,33 @@ int verify_one(s2moe_ctx *ctx, int layer, int B, const void *hidden, const float
         cudaLaunchConfig_t lc = pdl_config(ctx, rp.n_cta, kRwThreads, rp.smem_bytes, st, rp.early != 0);
         cudaLaunchKernelEx(&lc, ffn_rows_kernel, maps, a);
     } else if (plan == 3 || plan == 4) {
-
         const fused::TcPlan tp4 = plan == 4 ? fused::tc_make_plan(sh, B, ctx->n_sm, B * sh.k + sh.n_sh * B) : fused::TcPlan{};
-        const bool q4 = plan == 4 ? tp4.q4 != 0 : tp3.q4 != 0;
-        const int tokb = plan == 4 ? tp4.tokb : tp3.tokb, kg = plan == 4 ? tp4.kg : tp3.kg;
+        const bool q4 = sh.weight_dtype == DT_Q4B32;
         TcMaps maps = ctx->tc_maps[layer];
         const size_t n_routed = (size_t)B * sh.k;
         const uint64_t plane = (uint64_t)((const uint8_t *)ctx->act_lo - (const uint8_t *)ctx->act_hi);
         bool ok;
         if (q4) {
-            ok = make_map_ktiles(ctx, &maps.m[6], ctx->hperm, (uint64_t)B, (uint64_t)sh.d, (uint32_t)tokb / 128, (uint32_t)kg) &&
-                 make_map_hilo_ktiles(ctx, &maps.m[7], ctx->act_hi, n_routed, (uint64_t)sh.f, plane, (uint32_t)kg);
+            const int tokb = plan == 4 ? tp4.tokb : qp.tokb;
+            ok = make_map_ktiles(ctx, &maps.m[6], ctx->hperm, (uint64_t)B, (uint64_t)sh.d, (uint32_t)tokb / 128, kTcQ4KG) &&
+                 make_map_hilo_ktiles(ctx, &maps.m[7], ctx->act_hi, n_routed, (uint64_t)sh.f, plane, kTcQ4KG);
             if (ok && sh.n_sh)
                 ok = make_map_hilo_ktiles(ctx, &maps.m[8], ctx->act_hi + n_routed * sh.f, (uint64_t)sh.n_sh * B,
-                                          (uint64_t)sh.f_sh, plane, (uint32_t)kg);
-        } else if (plan == 3 && tp3.kg == 2) {
-            // two k-tiles per stage: the token tiles of both in one copy (see make_map_ktiles)
-            // (resident hidden-state tiles are loaded once, k-tile by k-tile, through the plain 2-D map)
-            ok = (tp3.x_bytes ? make_map(ctx, &maps.m[6], hidden, (uint64_t)B, (uint64_t)sh.d, (uint32_t)tp3.rows1)
-                              : make_map_ktiles(ctx, &maps.m[6], hidden, (uint64_t)B, (uint64_t)sh.d, (uint32_t)tp3.tokb / 128, 2)) &&
-                 make_map_hilo_ktiles(ctx, &maps.m[7], ctx->act_hi, n_routed, (uint64_t)sh.f, plane, 2);
-            if (ok && sh.n_sh)
-                ok = make_map_hilo_ktiles(ctx, &maps.m[8], ctx->act_hi + n_routed * sh.f, (uint64_t)sh.n_sh * B,
-                                          (uint64_t)sh.f_sh, plane, 2);
+                                          (uint64_t)sh.f_sh, plane, kTcQ4KG);
         } else {
-            ok = make_map(ctx, &maps.m[6], hidden, (uint64_t)B, (uint64_t)sh.d, plan == 3 ? (uint32_t)tp3.rows1 : 16u) &&
+            ok = make_map(ctx, &maps.m[6], hidden, (uint64_t)B, (uint64_t)sh.d, 16) &&
                  make_map_hilo(ctx, &maps.m[7], ctx->act_hi, n_routed, (uint64_t)sh.f, plane);
             if (ok && sh.n_sh)
                 ok = make_map_hilo(ctx, &maps.m[8], ctx->act_hi + n_routed * sh.f, (uint64_t)sh.n_sh * B, (uint64_t)sh.f_sh, plane);
         }
         if (!ok) return S2MOE_ECUDA;
         if (plan == 3) {
-            TcArgs a;
-            a.sh = sh; a.ws = ctx->ws; a.plan = tp3; a.y = out; a.pre = ctx->pre;
-            a.act_hi = ctx->act_hi; a.act_lo = ctx->act_lo; a.B = B; a.early = tp3.early;
+            Q4Args a;
+            a.sh = sh; a.ws = ctx->ws; a.plan = qp; a.y = out; a.pre = ctx->pre;
+            a.act_hi = ctx->act_hi; a.act_lo = ctx->act_lo; a.B = B;
             LaunchScope scope(ctx, KC_TC, st);
-            cudaLaunchConfig_t lc = pdl_config(ctx, tp3.n_cta, q4 ? kTcQ4Threads : kTcThreads, tp3.smem_bytes, st, tp3.early != 0);
-            if (q4) cudaLaunchKernelEx(&lc, ffn_tc_kernel<true>, maps, a);
-            else cudaLaunchKernelEx(&lc, ffn_tc_kernel<false>, maps, a);
+            cudaLaunchConfig_t lc = pdl_config(ctx, qp.n_cta, kQ4Threads, qp.smem_bytes, st, qp.early != 0);
+            cudaLaunchKernelEx(&lc, ffn_q4_kernel, maps, a);
         } else {
             fused::TcArgs a;
             a.sh = sh; a.ws = ctx->ws; a.plan = tp4; a.y = out; a.pre = ctx->pre;
@@ -703,7 +671,7 @@ int verify_one(s2moe_ctx *ctx, int layer, int B, const void *hidden, const float
             const bool bias_on = sh.alpha > 0.0 && sh.cap < sh.E && sh.k < sh.E;
             a.rt.early = (!bias_on || sh.alpha <= 1.0) ? 1 : 0;
             LaunchScope scope(ctx, KC_LAYER, st);
-            cudaLaunchConfig_t lc = pdl_config(ctx, tp4.n_cta, q4 ? kTcQ4Threads : kTcThreads, tp4.smem_bytes, st);
+            cudaLaunchConfig_t lc = pdl_config(ctx, tp4.n_cta, q4 ? fused::kTcQ4Threads : fused::kTcThreads, tp4.smem_bytes, st);
             if (q4) cudaLaunchKernelEx(&lc, fused::layer_tc_kernel<true>, maps, a);
             else cudaLaunchKernelEx(&lc, fused::layer_tc_kernel<false>, maps, a);
         }
@@ -797,7 +765,6 @@ int create_impl(const s2moe_config *config, const s2moe_layer_weights *layers, i
     const size_t o_ahi = take(2 * act_floats), o_alo = take(2 * act_floats);
     const size_t o_up1 = take(4 * (size_t)(G + 2)), o_up2 = take(4 * (size_t)(G + 2));
     const size_t o_tm = take(8 * (size_t)G);
-    const size_t o_gtab = take(32 * (size_t)(G + 1));
     const size_t o_early = take(8 * (size_t)(kEarlyWords + 1)), o_gsum = take(4 * (size_t)kMaxExperts);
     const size_t o_hperm = take(sh.weight_dtype == DT_Q4B32 ? 2 * (size_t)T * sh.d : 0);
     const size_t o_lpart = take(sizeof(double) * 8 * (size_t)T * (E + 1));
@@ -814,17 +781,10 @@ int create_impl(const s2moe_config *config, const s2moe_layer_weights *layers, i
     {
         const char *no_pdl = std::getenv("S2MOE_NO_PDL");
         ctx->use_pdl = !(no_pdl && no_pdl[0] == '1');
-        const char *kgv = std::getenv("S2MOE_BF16_KG2_FROM");
-        if (kgv && std::atoi(kgv) > 0) ctx->bf16_kg2_from = std::atoi(kgv);
         const char *tf = std::getenv("S2MOE_ROUTE_TASKS_FROM");
         if (tf && tf[0]) ctx->route_task_from = std::atoi(tf);
         const char *pg = std::getenv("S2MOE_PDL_IN_GRAPH");
         ctx->pdl_in_graph = pg && pg[0] == '1';
-        const char *wv = std::getenv("S2MOE_WAVES");
-        if (wv && wv[0]) {
-            int a = 0, b = 16;
-            if (std::sscanf(wv, "%d,%d", &a, &b) >= 1 && a > 0 && a <= 16 && b >= a && b <= 16) { ctx->wave_split[0] = a; ctx->wave_split[1] = b; }
-        }
         const char *ne = std::getenv("S2MOE_NO_EARLY");
         ctx->early_start = !(ne && ne[0] == '1');
     }
@@ -842,7 +802,6 @@ int create_impl(const s2moe_config *config, const s2moe_layer_weights *layers, i
     ws.act = (float *)(base + o_act); ws.sync = (int32_t *)(base + o_sync);
     ws.upfx1 = (int32_t *)(base + o_up1); ws.upfx2 = (int32_t *)(base + o_up2);
     ws.tokmask = (unsigned long long *)(base + o_tm);
-    ws.gtab = (uint4 *)(base + o_gtab);
     ws.early = (unsigned long long *)(base + o_early);
     ws.gsum = (float *)(base + o_gsum);
     ctx->hperm = base + o_hperm;
@@ -860,43 +819,29 @@ int create_impl(const s2moe_config *config, const s2moe_layer_weights *layers, i
             ctx->tc_maps.resize(config->n_layers);
             const bool q4 = sh.weight_dtype == DT_Q4B32;
             bool ok = cudaFuncSetAttribute(ffn_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kRwMaxSmem) == cudaSuccess &&
-                      cudaFuncSetAttribute(ffn_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcMaxSmem) == cudaSuccess &&
-                      cudaFuncSetAttribute(ffn_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcMaxSmem) == cudaSuccess &&
+                      cudaFuncSetAttribute(ffn_q4_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcMaxSmem) == cudaSuccess &&
                       cudaFuncSetAttribute(fused::layer_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcMaxSmem) == cudaSuccess &&
                       cudaFuncSetAttribute(fused::layer_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcMaxSmem) == cudaSuccess;
-            // the int4 variant needs contraction lengths that are multiples of 256 (see tc_make_plan)
+            // the int4 variant needs contraction lengths that are multiples of 256 (see q4_make_plan)
             if (q4 && (sh.d % 256 || sh.f % 256 || (sh.n_sh && sh.f_sh % 256))) ok = false;
             for (int l = 0; l < config->n_layers && ok; ++l) {
                 const LayerPtrs &lp = ctx->layers[l];
                 TcMaps &m = ctx->tc_maps[l];
                 std::memset(&m, 0, sizeof(m));
                 if (q4) {
+                    // the packed matrices (boxes of four k-tiles) and their scales
                     const uint64_t Ef = (uint64_t)n_w_experts * sh.f, Ed = (uint64_t)n_w_experts * sh.d;
-                    ok = make_map_plain(ctx, &m.m[0], lp.w_gate, Ef, (uint64_t)sh.d / 2, 32, 1) &&
-                         make_map_plain(ctx, &m.m[1], lp.w_up, Ef, (uint64_t)sh.d / 2, 32, 1) &&
-                         make_map_plain(ctx, &m.m[2], lp.w_down, Ed, (uint64_t)sh.f / 2, 32, 1) &&
+                    ok = make_map_plain(ctx, &m.m[0], lp.w_gate, Ef, (uint64_t)sh.d / 2, 128, 1) &&
+                         make_map_plain(ctx, &m.m[1], lp.w_up, Ef, (uint64_t)sh.d / 2, 128, 1) &&
+                         make_map_plain(ctx, &m.m[2], lp.w_down, Ed, (uint64_t)sh.f / 2, 128, 1) &&
                          make_map_plain(ctx, &m.m[9], lp.s_gate, Ef, (uint64_t)sh.d / 32, 8, 2) &&
                          make_map_plain(ctx, &m.m[10], lp.s_up, Ef, (uint64_t)sh.d / 32, 8, 2) &&
                          make_map_plain(ctx, &m.m[11], lp.s_down, Ed, (uint64_t)sh.f / 32, 8, 2);
-                    // the packed matrices again with boxes of two and of four k-tiles
-                    for (int j = 1; j <= 2 && ok; ++j) {
-                        const int base = 15 + 6 * (j - 1);
-                        const uint32_t bc = 32u << j;
-                        ok = make_map_plain(ctx, &m.m[base + 0], lp.w_gate, Ef, (uint64_t)sh.d / 2, bc, 1) &&
-                             make_map_plain(ctx, &m.m[base + 1], lp.w_up, Ef, (uint64_t)sh.d / 2, bc, 1) &&
-                             make_map_plain(ctx, &m.m[base + 2], lp.w_down, Ed, (uint64_t)sh.f / 2, bc, 1);
-                        if (ok && sh.n_sh) {
-                            const uint64_t Sf = (uint64_t)sh.n_sh * sh.f_sh, Sd = (uint64_t)sh.n_sh * sh.d;
-                            ok = make_map_plain(ctx, &m.m[base + 3], lp.sh_gate, Sf, (uint64_t)sh.d / 2, bc, 1) &&
-                                 make_map_plain(ctx, &m.m[base + 4], lp.sh_up, Sf, (uint64_t)sh.d / 2, bc, 1) &&
-                                 make_map_plain(ctx, &m.m[base + 5], lp.sh_down, Sd, (uint64_t)sh.f_sh / 2, bc, 1);
-                        }
-                    }
                     if (ok && sh.n_sh) {
                         const uint64_t Sf = (uint64_t)sh.n_sh * sh.f_sh, Sd = (uint64_t)sh.n_sh * sh.d;
-                        ok = make_map_plain(ctx, &m.m[3], lp.sh_gate, Sf, (uint64_t)sh.d / 2, 32, 1) &&
-                             make_map_plain(ctx, &m.m[4], lp.sh_up, Sf, (uint64_t)sh.d / 2, 32, 1) &&
-                             make_map_plain(ctx, &m.m[5], lp.sh_down, Sd, (uint64_t)sh.f_sh / 2, 32, 1) &&
+                        ok = make_map_plain(ctx, &m.m[3], lp.sh_gate, Sf, (uint64_t)sh.d / 2, 128, 1) &&
+                             make_map_plain(ctx, &m.m[4], lp.sh_up, Sf, (uint64_t)sh.d / 2, 128, 1) &&
+                             make_map_plain(ctx, &m.m[5], lp.sh_down, Sd, (uint64_t)sh.f_sh / 2, 128, 1) &&
                              make_map_plain(ctx, &m.m[12], lp.sh_s_gate, Sf, (uint64_t)sh.d / 32, 8, 2) &&
                              make_map_plain(ctx, &m.m[13], lp.sh_s_up, Sf, (uint64_t)sh.d / 32, 8, 2) &&
                              make_map_plain(ctx, &m.m[14], lp.sh_s_down, Sd, (uint64_t)sh.f_sh / 32, 8, 2);
@@ -910,17 +855,6 @@ int create_impl(const s2moe_config *config, const s2moe_layer_weights *layers, i
                     ok = make_map(ctx, &m.m[3], lp.sh_gate, (uint64_t)sh.n_sh * sh.f_sh, (uint64_t)sh.d, 128) &&
                          make_map(ctx, &m.m[4], lp.sh_up, (uint64_t)sh.n_sh * sh.f_sh, (uint64_t)sh.d, 128) &&
                          make_map(ctx, &m.m[5], lp.sh_down, (uint64_t)sh.n_sh * sh.d, (uint64_t)sh.f_sh, 128);
-                // the same matrices with two k-tiles per copy (maps 9..14), where every contraction
-                // length is a multiple of 64
-                if (ok && sh.d % 64 == 0 && sh.f % 64 == 0 && (sh.n_sh == 0 || sh.f_sh % 64 == 0)) {
-                    ok = make_map_w2(ctx, &m.m[9], lp.w_gate, (uint64_t)n_w_experts * sh.f, (uint64_t)sh.d) &&
-                         make_map_w2(ctx, &m.m[10], lp.w_up, (uint64_t)n_w_experts * sh.f, (uint64_t)sh.d) &&
-                         make_map_w2(ctx, &m.m[11], lp.w_down, (uint64_t)n_w_experts * sh.d, (uint64_t)sh.f);
-                    if (ok && sh.n_sh)
-                        ok = make_map_w2(ctx, &m.m[12], lp.sh_gate, (uint64_t)sh.n_sh * sh.f_sh, (uint64_t)sh.d) &&
-                             make_map_w2(ctx, &m.m[13], lp.sh_up, (uint64_t)sh.n_sh * sh.f_sh, (uint64_t)sh.d) &&
-                             make_map_w2(ctx, &m.m[14], lp.sh_down, (uint64_t)sh.n_sh * sh.d, (uint64_t)sh.f_sh);
-                }
             }
             if (!ok) ctx->tc_maps.clear();
             if (ok && !q4) {
