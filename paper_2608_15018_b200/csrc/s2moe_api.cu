@@ -44,7 +44,7 @@ struct s2moe_ctx {
     bool pdl_in_graph = false;            // S2MOE_PDL_IN_GRAPH=1: also under stream capture
     void *hperm = nullptr;                // int4 plan 3: column-permuted copy of the hidden states
     double *lpart = nullptr;              // partial router logits [piece][token][row] (logit pass by warp tasks)
-    int route_task_from = 48;             // batches of this many tokens and more take the logit pass by warp tasks
+    int route_task_from = 48;             // batches of this many tokens and more may take the logit pass by warp tasks (route_by_tasks)
     bool early_start = true;              // bf16 tensor-core plan: the expert kernel starts under the gating (S2MOE_NO_EARLY=1: off)
     float *pre = nullptr;                 // plan 3: fp32 pre-activations [gate|up][slot][f]
     std::vector<TcMaps> tc_maps;          // plan 3: per layer, weight maps filled at create
@@ -207,6 +207,18 @@ size_t route_smem(int B, int E, int k)
     return align_up(a > b ? a : b, 16);
 }
 
+// Whether the logit pass of a batch runs as warp tasks over a grid of 1024-thread blocks instead of by row
+// blocks.  Row blocks leave room for the expert kernel on their SM, which streams the shared experts meanwhile,
+// and take a pass per 16 tokens; where two sets of them run beside each other that is at most two passes.
+// Measured, us per layer, tasks / row blocks: DeepSeek-V2-Lite shape 64 tokens 125.9 / 122.7, 48 tokens 112.1 /
+// 110.2, OLMoE shape 64 tokens 71.6 / 68.4, Qwen1.5-MoE shape 64 tokens 77.3 / 74.8, Mixtral int4 64 tokens
+// 178 / 175.  With one set (more than 73 rows on 148 SMs), at 64 tokens: 96 experts 72.0 / 73.2, 128
+// experts 82.1 / 82.1, 160 experts 96.5 / 106.4, 256 experts 113.5 / 118.4.
+bool route_by_tasks(const s2moe_ctx *ctx, int rows, int B)
+{
+    return ctx->lpart && B >= ctx->route_task_from && (ctx->n_sm - 1) / rows < 2;
+}
+
 template <int ACT, int RT>
 void launch_route_t(s2moe_ctx *ctx, const Shape &sh, const LayerPtrs &lp, int B, const void *hidden, const float *conf,
                     int32_t *sel_idx, float *sel_w, int32_t *n_unique, const ZeroList &zl, cudaStream_t st)
@@ -223,8 +235,7 @@ void launch_route_t(s2moe_ctx *ctx, const Shape &sh, const LayerPtrs &lp, int B,
     zg.ksplit = 0;
     zg.lpart = nullptr;
     int grid;
-    const int task_from = ctx->route_task_from;
-    if (ctx->lpart && B >= task_from) {
+    if (route_by_tasks(ctx, rows, B)) {
         // the logit pass as warp tasks: pieces of the contraction so that the warps of a full grid
         // have about one task each
         const int tgs = (B + 7) / 8, warps = ctx->n_sm * (kRouteThreadsBig / 32);
@@ -580,7 +591,8 @@ int verify_one(s2moe_ctx *ctx, int layer, int B, const void *hidden, const float
     // announces (not with offloaded experts: their weights are fetched between the two kernels)
     const bool want_early = plan == 3 && ctx->early_start && ctx->use_pdl && !ctx->offload;
     const bool rows3 = plan == 3 && sh.weight_dtype == DT_BF16;
-    const RwPlan rp = rows3 ? rw_make_plan(sh, B, ctx->n_sm, want_early, B < ctx->route_task_from ? (int)route_smem(B, sh.E, sh.k) + 256 : 0) : RwPlan{};
+    const bool by_tasks = route_by_tasks(ctx, sh.E + (lp.sh_scale ? 1 : 0), B);
+    const RwPlan rp = rows3 ? rw_make_plan(sh, B, ctx->n_sm, want_early, by_tasks ? 0 : (int)route_smem(B, sh.E, sh.k) + 256) : RwPlan{};
     const bool q4_3 = plan == 3 && !rows3;
     const Q4Plan qp = q4_3 ? q4_make_plan(sh, B, ctx->n_sm, want_early) : Q4Plan{};
     // what the FFN kernels accumulate into is cleared by the routing kernel's blocks

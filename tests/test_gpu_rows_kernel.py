@@ -28,6 +28,17 @@ def test_few_and_many_experts(E, k, B):
     assert rep.plan == 3 and rep.tokens_checked == B
 
 
+@pytest.mark.parametrize("shared_gate", [False, True])
+@pytest.mark.parametrize("E,B", [(72, 48), (73, 64), (74, 64), (74, 47), (100, 48)])
+def test_both_forms_of_the_logit_pass(E, B, shared_gate):
+    """Two sets of row blocks fit beside each other up to 73 router rows (148 SMs); with more rows, batches of
+    48 tokens and more take the logit pass by warp tasks."""
+    wl = CONFIGS["cfg3"].with_(d_model=512, d_ff=96, d_ff_shared=64 if shared_gate else 0, n_shared=int(shared_gate),
+                               shared_gate=shared_gate, n_experts=E, top_k=4, cap=20, sigma=1.0, seed=E)
+    rep, _ = run_case(wl, n_tokens=B, plan=3)
+    assert rep.plan == 3 and rep.tokens_checked == B
+
+
 @pytest.mark.parametrize("layout", ["up_first", "tied"])
 def test_layouts_of_gate_and_up(layout):
     wl = CONFIGS["cfg3"].with_(d_model=320, d_ff=352, d_ff_shared=416, n_experts=10, top_k=2, cap=4, n_layers=1)
