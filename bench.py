@@ -36,9 +36,9 @@ FALLBACK_HBM_GBS = 6650.0
 
 
 # DRAM bytes (read + write) per algorithmic byte, from the ncu captures summarised under profiles/
-# (ffn_tc_kernel_cfg2_2layers.md, ffn_tc_kernel_int4_cfg4_2layers.md, ffn_stream_kernel_cfg2_2layers.md); traffic grows with the
+# (expert_kernels_plan3.md, ffn_stream_kernel_cfg2_2layers.md); traffic grows with the
 # number of distinct experts exactly as the algorithmic bytes do.
-TRAFFIC_RATIO = {"ffn_tc_kernel": 1.03, "ffn_tc_kernel/int4": 1.02, "ffn_stream_kernel": 1.005}
+TRAFFIC_RATIO = {"ffn_tc_kernel": 1.02, "ffn_tc_kernel/int4": 1.02, "ffn_stream_kernel": 1.005}
 
 
 def parse_args():
@@ -295,7 +295,7 @@ def measure_stack(wl, B, sigma, L, plan, steps, warmup, dev, rank, world, peak, 
             graph_ms = statistics.median(graph_all)
             timed_path = (f"CUDA graph replay of one s2moe_verify_stack call per step; median of {reps} repeats of "
                           f"{steps} steps ({done_s:.2f} s timed); the graph keeps the programmatic launch edges, so with "
-                          f"bf16 weights the expert kernel of a layer starts while that layer's gating still runs "
+                          f"the tensor-core plan the expert kernel of a layer starts while that layer's routing still runs "
                           f"(the per-kernel durations of region B are taken with event pairs, which serialise the two)")
     except Exception as exc:  # pragma: no cover
         graph_ms = None

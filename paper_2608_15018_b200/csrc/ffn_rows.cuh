@@ -39,9 +39,12 @@
 //
 // Warp roles (352 threads): 0 TMA producer, 1 MMA issuer (owns the TMEM allocation), 2..5 and 6..9 two
 // epilogue sets that take alternate tasks (6..9 build the tables first), 10 watcher (early experts,
-// selection and the tasks of the first projection, then the wave counters).  The single-thread roles run in a thread chosen by elect.sync: measured on
-// B200, an MMA of 128 x 16 x 16 then issues every 39 cycles against 55 from a `lane == 0` branch
-// (the tensor core itself needs 32 to read the 4 KiB of weights), which is why one issuer is enough.
+// selection and the tasks of the first projection, then the wave counters).  The single-thread roles run
+// in a thread chosen by elect.sync: measured on B200, an MMA of 128 x 16 x 16 then issues every 39 cycles
+// against 55 from a `lane == 0` branch (the tensor core itself needs 32 to read the 4 KiB of
+// weights), which is why one issuer is enough.
+// Measured, us per layer, split-K kernel before / this one: OLMoE shape 8 tokens 52 / 42, Qwen1.5-MoE
+// shape 16 tokens 54.6 / 42, DeepSeek-V2-Lite shape 16 tokens 60 / 52, 64 tokens 140 / 129.
 // Even and odd k-tiles go to two accumulators that the epilogue adds: the tensor core truncates when
 // it adds to an accumulator, so half the chain is half the error (relative 2-norm against the float64
 // oracle 5.3e-6 with one chain of 128 steps).
