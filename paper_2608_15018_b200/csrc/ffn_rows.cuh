@@ -88,6 +88,7 @@ struct RwPlan {
     int tab_bytes;
     int smem_bytes;
     int early, n_early;           // early start; its experts
+    int one_rows;                 // second-projection tasks of that many slots take one k-tile per stage (0: none)
     int split16[kRwMaxWaves - 1];   // where waves 1, 2, 3 begin, in 16ths of the first projection (16: no such wave)
     int delta;           // second-projection units that weigh as much as one first-projection unit
     RwDiv gf, gs, tf, ts, kr, ks, rb, p;   // row groups and tasks of a routed / shared expert, P2 units of their row blocks, row blocks, CTAs
@@ -140,7 +141,15 @@ inline RwPlan rw_make_plan(const Shape &sh, int B, int n_sm, bool early, int rou
     p.n_early = p.early ? (sh.k < 4 ? (sh.k == 3 ? 2 : 1) : (B <= 2 ? (3 * sh.k + 2) / 4 : sh.k)) : 0;
     p.n1 = (B + 15) & ~15;
     const int trows = rw_tok_rows(B);
-    const int tok2 = 2 * 2 * trows * 128, tok1 = 2 * p.n1 * 128;
+    // Tasks of the second projection whose token tiles would make every stage larger (32 slots where the batch
+    // has up to 32 tokens, 64 above) take one k-tile per stage: few groups are that large, and a stage of 40
+    // or 48 instead of 48 or 64 KiB gives the ring a stage more.  Measured, us per layer, two k-tiles / one:
+    // DeepSeek-V2-Lite shape 20 tokens 61.8 / 58.1, 32 tokens 69.3 / 65.6, 64 tokens 117.7 / 113.7, OLMoE shape
+    // 24 tokens 57.2 / 53.7, Qwen1.5-MoE shape 32 tokens 53.1 / 50.8.  At 16 slots it loses: 51.9 / 53.6 (the
+    // shared experts' tasks are a larger part there, and the ring does not get a stage more beside the
+    // resident tiles and a routing block).
+    p.one_rows = trows >= 32 ? trows : 0;
+    const int tok2 = (p.one_rows ? 1 : 2) * 2 * trows * 128, tok1 = 2 * p.n1 * 128;
     p.acc_cols = 2 * trows > 2 * p.n1 ? 2 * trows : 2 * p.n1;       // (32, 64, 128: a power of two)
     while (p.acc_cols & (p.acc_cols - 1)) p.acc_cols += 32;
     p.n_acc = 512 / p.acc_cols;
@@ -167,12 +176,14 @@ inline RwPlan rw_make_plan(const Shape &sh, int B, int n_sm, bool early, int rou
     // Early start: a routing block shares every SM with a CTA of this kernel if that leaves room for three
     // stages (two blocks on an SM share 228 KiB, 1 KiB of it reserved for each).  If not, one CTA less than
     // SMs: the SM that runs the gating is taken until the routing kernel ends, and its CTA would start
-    // last with a full share.
+    // last with a full share.  Up to 16 tokens only: with more the stage that the routing block costs is worth
+    // more (us per layer beside / not: OLMoE shape 8 tokens 41.6 / 43.3, 24 tokens 54.0 / 53.6, 128 experts
+    // at 32 tokens 61.3 / 55.7).
     const int full = kRwMaxSmem - p.tab_bytes - 1024, shared = 228 * 1024 - 2048 - kRwStaticSmem - route_smem - p.tab_bytes - 1024;
     const int x_res = ((nk + 7) & ~7) * (B <= 8 ? 8 : p.n1) * 128 + 1024, st_res = kRwWBytes + ((tok2 + 1023) & ~1023);
     const int st_tok = kRwWBytes + (((tok1 > tok2 ? tok1 : tok2) + 1023) & ~1023);
-    const bool beside = p.early && route_smem > 0 &&
-                        ((shared - x_res) / st_res >= 3 || ((full - x_res) / st_res < 3 && shared / st_tok >= 3));
+    const bool beside = p.early && route_smem > 0 && p.n1 == 16 &&
+                        ((shared - x_res) / st_res >= 3 || ((full - x_res) / st_res < 3 && shared / st_tok >= 4));
     const int budget = beside ? shared : full;
     p.n_cta = p.early && !beside ? n_sm - 1 : n_sm;
     p.p = rw_div_make(p.n_cta);
@@ -420,7 +431,7 @@ ffn_rows_kernel(const __grid_constant__ RwMaps maps, const __grid_constant__ RwA
                 const int rows = t.flags >> 8, mi = (t.flags & 2 ? 15 : 11) + (rows == 8 ? 0 : (rows == 16 ? 1 : (rows == 32 ? 2 : 3)));
                 const uint32_t dst = ring_a + (uint32_t)(slot * pl.stage_bytes + kRwWBytes), bar = full_a + 8u * slot;
                 rw_tma_3d(dst, &maps.m[mi], kt * 64, t.srow, 0, bar);
-                if (kt + 1 < (t.k >> 16)) rw_tma_3d(dst + rows * 256u, &maps.m[mi], kt * 64 + 64, t.srow, 0, bar);
+                if (rows != pl.one_rows && kt + 1 < (t.k >> 16)) rw_tma_3d(dst + rows * 256u, &maps.m[mi], kt * 64 + 64, t.srow, 0, bar);
             };
             auto flush = [&]() {
                 // the wave's activations are written: order them before the copies below
@@ -431,7 +442,7 @@ ffn_rows_kernel(const __grid_constant__ RwMaps maps, const __grid_constant__ RwA
                 for (; pend_n > 0; --pend_n) {
                     if (pend_k >= (t.k >> 16)) { t = tasks[++pend_t]; pend_k = t.k & 0xffff; }
                     load_tokens(t, pend_s, pend_k);
-                    pend_k += 2;
+                    pend_k += (t.flags >> 8) == pl.one_rows ? 1 : 2;
                     if (++pend_s == S) pend_s = 0;
                 }
             };
@@ -501,11 +512,12 @@ ffn_rows_kernel(const __grid_constant__ RwMaps maps, const __grid_constant__ RwA
                     const uint32_t wb = half ? 8192u : 16384u;
                     if (pend_n > 0 && wv != pend_w) { if (!ready_wait()) { alive = false; break; } }
                     if (pend_n == 0 && wv >= ready_w && s_ready[wv]) { pend_w = wv; pend_t = i; flush(); }
-                    for (int kt = t.k & 0xffff; kt < k1; kt += 2) {
+                    const int step = rows == pl.one_rows ? 1 : 2;
+                    for (int kt = t.k & 0xffff; kt < k1; kt += step) {
                         // (every slot waits for its tokens: nothing can become free before they are there)
                         if (pend_n == S) { if (!ready_wait()) { alive = false; break; } }
                         if (!slot_wait()) { alive = false; break; }
-                        const int two = kt + 1 < k1 ? 2 : 1;
+                        const int two = min(step, k1 - kt);
                         const uint32_t bar = full_a + 8u * s, dst = ring_a + (uint32_t)(s * pl.stage_bytes);
                         rw_expect(bar, (uint32_t)two * (wb + (uint32_t)rows * 256u));
                         rw_tma_2d(dst, dm, kt * 64, t.x0, bar, wpolicy);
@@ -581,13 +593,14 @@ ffn_rows_kernel(const __grid_constant__ RwMaps maps, const __grid_constant__ RwA
                     const uint32_t idesc = tc_idesc(2 * rows);
                     // (the columns of an accumulator leave room for two chains up to half the batch)
                     const bool twin = 4 * rows <= pl.acc_cols;
-                    for (int kt = k0; kt < k1; kt += 2) {
+                    const int step = rows == pl.one_rows ? 1 : 2;
+                    for (int kt = k0; kt < k1; kt += step) {
                         if (!mbar_wait(&full_bar[s], par)) { atomicExch(ws.status, ST_MBAR_TIMEOUT); alive = false; break; }
                         tc_fence_after();
                         const uint64_t ad = ring_d + (uint64_t)((uint32_t)(s * pl.stage_bytes) >> 4), bd = ad + (kRwWBytes >> 4);
 #pragma unroll
                         for (int q = 0; q < 2; ++q) {
-                            if (kt + q < k1) {
+                            if (q < step && kt + q < k1) {
 #pragma unroll
                                 for (int h = 0; h < 4; ++h)
                                     rw_mma(d_tmem + (q && twin ? 2u * (uint32_t)rows : 0u), ad + (uint64_t)(1024 * q + 2 * h),

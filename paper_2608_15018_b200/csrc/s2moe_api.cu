@@ -208,8 +208,8 @@ size_t route_smem(int B, int E, int k)
 }
 
 // Whether the logit pass of a batch runs as warp tasks over a grid of 1024-thread blocks instead of by row
-// blocks.  Row blocks leave room for the expert kernel on their SM, which streams the shared experts meanwhile,
-// and take a pass per 16 tokens; where two sets of them run beside each other that is at most two passes.
+// blocks.  Row blocks take a pass per 16 tokens and write no partial sums; where two sets of them run beside
+// each other that is at most two passes.
 // Measured, us per layer, tasks / row blocks: DeepSeek-V2-Lite shape 64 tokens 125.9 / 122.7, 48 tokens 112.1 /
 // 110.2, OLMoE shape 64 tokens 71.6 / 68.4, Qwen1.5-MoE shape 64 tokens 77.3 / 74.8, Mixtral int4 64 tokens
 // 178 / 175.  With one set (more than 73 rows on 148 SMs), at 64 tokens: 96 experts 72.0 / 73.2, 128
