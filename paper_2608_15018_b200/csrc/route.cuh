@@ -430,6 +430,10 @@ __device__ __forceinline__ void route_body(const Shape &sh, int B, const Workspa
     // nothing, and the waiting path is one reduction and one polled load, as short as it can be.  The
     // barriers on both sides extend the ordering to the block's other threads; the other blocks
     // wait for nothing.
+    // The arrival is one thread's and covers the whole block only behind a barrier.  A logit pass ends with one,
+    // but a row block whose group of tokens is empty (12 rows, 64 tokens: 12 groups of 8 tokens, 4 of them empty)
+    // makes no pass and has written its part of the binary16 copy all the same.
+    if (zl.perm_n16) __syncthreads();
     if (tid == 0 && rblk >= 0 && rblk < n_arrive)
         asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(ws.ticket) : "memory");
     if (blockIdx.x == 0 && tid == 0) {

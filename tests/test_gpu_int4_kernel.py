@@ -33,3 +33,13 @@ def test_more_units_than_the_table_of_a_cta_holds():
     wl = CONFIGS["cfg4"].with_(d_model=256, d_ff=14336, n_experts=256, top_k=16, cap=256, sigma=1.0, n_layers=1)
     rep, _ = run_case(wl, n_tokens=64, plan=3, tok_list=list(range(0, 64, 9)))
     assert rep.plan == 3
+
+
+@pytest.mark.parametrize("B", [57, 64])
+def test_row_blocks_without_tokens(B):
+    """12 router rows and a wide model: a third of the row blocks gets no tokens, and some of them still write a
+    part of the binary16 copy of the hidden states that the expert kernel reads behind their arrival."""
+    wl = CONFIGS["cfg4"].with_(d_model=8192, d_ff=256, n_experts=12, top_k=3, cap=5, sigma=1.0, seed=B)
+    for _ in range(4):
+        rep, _ = run_case(wl, n_tokens=B, plan=3)
+        assert rep.plan == 3 and rep.tokens_checked == B
