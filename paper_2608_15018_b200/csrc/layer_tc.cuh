@@ -387,9 +387,9 @@ layer_tc_kernel(const __grid_constant__ TcMaps maps, TcArgs p)
         {
             const int nwarps = (int)blockDim.x >> 5;
             if (sh.router_dtype == DT_F32)
-                route_logit_tasks<DT_BF16, DT_F32>(sh, p.B, rt.hidden, rt.router, rt.sh_scale, rt.lpart, pl.ksplit, nullptr, nullptr, warp * P + (int)blockIdx.x, nwarps * P, lane);
+                route_logit_tasks<DT_BF16, DT_F32, true>(sh, p.B, rt.hidden, rt.router, rt.sh_scale, rt.lpart, pl.ksplit, nullptr, nullptr, warp * P + (int)blockIdx.x, nwarps * P, lane);
             else
-                route_logit_tasks<DT_BF16, DT_BF16>(sh, p.B, rt.hidden, rt.router, rt.sh_scale, rt.lpart, pl.ksplit, nullptr, nullptr, warp * P + (int)blockIdx.x, nwarps * P, lane);
+                route_logit_tasks<DT_BF16, DT_BF16, true>(sh, p.B, rt.hidden, rt.router, rt.sh_scale, rt.lpart, pl.ksplit, nullptr, nullptr, warp * P + (int)blockIdx.x, nwarps * P, lane);
         }
         tc_fence_before();
         __syncthreads();

@@ -106,11 +106,12 @@ __device__ __forceinline__ void gating_writeout(const Shape &sh, int B, const Wo
 // Gating of one batch by a whole thread block (kRouteThreads threads) on the logits in the workspace.
 // s_l: shared memory for B * E + B doubles (the logits and the confidences are staged there) and, behind
 // them, gate_mem_bytes(E, B, k).
-template <int JE>
+// repair(): called by the block if `nonfinite`, with the logits staged (repair_logits).
+template <int JE, class Repair>
 __device__ __forceinline__ void gating_block(const Shape &sh, int B, const Workspace &ws, const float *__restrict__ conf,
                                              int has_gate, int32_t *__restrict__ sel_idx, float *__restrict__ sel_w,
                                              int32_t *__restrict__ n_unique, double *s_l, int ksplit, const double *__restrict__ lpart,
-                                             int early)
+                                             int early, bool nonfinite, Repair repair)
 {
     // (sized by this batch and not for the largest one: a routing block shares its SM with the expert kernel)
     const GateMem gm = gate_mem_carve(s_l + ((B * sh.E + B + 1) & ~1), sh.E, B, sh.k);
@@ -139,6 +140,7 @@ __device__ __forceinline__ void gating_block(const Shape &sh, int B, const Works
 #pragma unroll 1
     for (int b = gg.t; b < B; b += gg.n) s_w[b] = conf ? (double)conf[b] : 1.0;
     __syncthreads();                                      // the logits are staged
+    if (nonfinite) repair();
     gating_part1<JE>(sh, B, s_l, s_w, gg, gm);
     gating_part2<JE>(sh, B, s_l, gg, gm, sel_idx, sel_w, early ? ws.early : nullptr);
     gating_writeout(sh, B, ws, gm, has_gate, n_unique, gg);
@@ -212,19 +214,82 @@ __device__ __forceinline__ double warp_sums(double (&a)[NT], int lane)
     return a[0];
 }
 
-// x * 2^-896 exactly, subnormal numbers included, by moving the bits of the binary32 number into place (a
-// conversion instruction has a quarter of the rate of the fused multiply-add it feeds); the other
-// factor carries the 2^896
+// x * 2^-896 exactly for every finite x, subnormal numbers included, by moving the bits of the binary32
+// number into place (a conversion instruction has a quarter of the rate of the fused multiply-add it
+// feeds); the other factor carries the 2^896.  An infinity or a NaN comes out as some finite number: a batch
+// that holds one is found by nonfinite_scan, and its tokens get their logits from repair_logits.
 __device__ __forceinline__ double scaled_double(float x, bool bf16)
 {
     const uint32_t u = __float_as_uint(x);
     return __hiloint2double((int)(((u >> 3) & 0x0fffffffu) | (u & 0x80000000u)), bf16 ? 0 : (int)(u << 29));
 }
 
+// Whether the thread's share of n16 16-byte units (thread t of n) holds an infinity or a NaN: an exponent field
+// of all ones carries into the sign's place.  Block 0, which has no logits to form, looks through the batch while
+// it waits for the others, eight loads in flight per thread (256 KB, 64 tokens of 2048, in some 3 us).
+// Measured against the alternatives in the logit pass itself (0 * x summed beside it) and in slices
+// beside it (marks in memory that block 0 collects): those cost 0.6 to 1.1 us per layer at 13 and 64 tokens, and at 1.
+template <int ACT>
+__device__ __forceinline__ bool nonfinite_scan(const void *__restrict__ hidden, int n16, int t, int n)
+{
+    const uint32_t keep = ACT == DT_F32 ? 0x7fffffffu : 0x7fff7fffu, one = ACT == DT_F32 ? 0x00800000u : 0x00800080u;
+    uint32_t bad = 0u;
+#pragma unroll 1
+    for (int i = t; i < n16; i += 8 * n) {
+        uint4 v[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            v[j] = i + j * n < n16 ? __ldg(reinterpret_cast<const uint4 *>(hidden) + i + j * n) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            bad |= ((v[j].x & keep) + one) | ((v[j].y & keep) + one) | ((v[j].z & keep) + one) | ((v[j].w & keep) + one);
+    }
+    return (bad & ~keep) != 0u;
+}
+
+// The logits of the tokens with an infinity or a NaN by plain float64 arithmetic on the stored values (a warp per
+// token and row), by a whole block; s_l [B][E] and the workspace get them.  Out of line: it runs for no other batch.
+template <int ACT, int RT>
+__device__ __noinline__ void repair_logits(int B, int d, int E, int n_rows, const void *hidden, const void *router, const void *sh_scale,
+                                           double *s_l, double *logits, double *gate_logit)
+{
+    __shared__ unsigned long long s_marks;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const size_t row = (size_t)d * (ACT == DT_F32 ? 4 : 2);
+    if (threadIdx.x == 0) s_marks = 0ull;
+    __syncthreads();
+    for (int b = warp; b < B; b += nw)
+        if (nonfinite_scan<ACT>(reinterpret_cast<const uint8_t *>(hidden) + (size_t)b * row, (int)(row / 16), lane, 32))
+            atomicOr(&s_marks, 1ull << b);
+    __syncthreads();
+    for (unsigned long long marks = s_marks; marks; marks &= marks - 1ull) {
+        const int b = __ffsll((long long)marks) - 1;
+        for (int r = warp; r < n_rows; r += nw) {
+            const uint8_t *w = r < E ? reinterpret_cast<const uint8_t *>(router) + (size_t)r * d * (RT == DT_F32 ? 4 : 2)
+                                     : reinterpret_cast<const uint8_t *>(sh_scale);
+            double v = 0.0;
+            for (int c = lane * 4; c < d; c += 128) {
+                float a[4], h[4];
+                load4_plain<RT>(w, c, a);
+                load4_plain<ACT>(reinterpret_cast<const uint8_t *>(hidden) + (size_t)b * row, c, h);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) v = fma((double)a[i], (double)h[i], v);
+            }
+            v = warp_sum(v);
+            if (lane == 0) {
+                if (r < E) s_l[b * E + r] = logits[b * E + r] = v;
+                else gate_logit[b] = v;
+            }
+        }
+    }
+    __syncthreads();
+}
+
 // Router logits by the warps of the whole grid: a task is one router row (row E: the shared
 // experts' gate vector) x 8 tokens x one piece of the contraction, float64 accumulation; its
 // partial sums go to lpart[piece][token][row], which the gating adds up in a fixed order.
-template <int ACT, int RT>
+// EXACT: by conversion instructions, for a caller that does not look for infinities and NaN (see scaled_double).
+template <int ACT, int RT, bool EXACT>
 __device__ __forceinline__ void route_logit_tasks(const Shape &sh, int B, const void *__restrict__ hidden,
                                                   const void *__restrict__ router, const void *__restrict__ sh_scale,
                                                   double *__restrict__ lpart, int ksplit, const float *__restrict__ conf,
@@ -254,11 +319,12 @@ __device__ __forceinline__ void route_logit_tasks(const Shape &sh, int B, const 
             }
             double wd[4];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) wd[i] = (double)w[i] * 0x1p896;
+            for (int i = 0; i < 4; ++i) wd[i] = EXACT ? (double)w[i] : (double)w[i] * 0x1p896;
 #pragma unroll
             for (int t = 0; t < 8; ++t)
 #pragma unroll
-                for (int i = 0; i < 4; ++i) acc[t] = fma(wd[i], scaled_double(x[t][i], ACT == DT_BF16), acc[t]);
+                for (int i = 0; i < 4; ++i)
+                    acc[t] = fma(wd[i], EXACT ? (double)x[t][i] : scaled_double(x[t][i], ACT == DT_BF16), acc[t]);
         }
         const double v = warp_sums<8>(acc, lane);             // token lane / 4
         const int bt = b0 + (lane >> 2);
@@ -400,7 +466,7 @@ __device__ __forceinline__ void route_body(const Shape &sh, int B, const Workspa
     if (zl.ksplit > 0) {
         // larger batches: the logit pass as warp tasks over all blocks but the first
         if (rblk >= 0)
-            route_logit_tasks<ACT, RT>(sh, B, hidden, router, sh_scale, zl.lpart, zl.ksplit, conf, zl.early ? ws.gsum : nullptr, (tid >> 5) * n_arrive + rblk,
+            route_logit_tasks<ACT, RT, false>(sh, B, hidden, router, sh_scale, zl.lpart, zl.ksplit, conf, zl.early ? ws.gsum : nullptr, (tid >> 5) * n_arrive + rblk,
                                        (THREADS / 32) * n_arrive, tid & 31);
         __syncthreads();
     } else if constexpr (THREADS == kRouteThreads) {
@@ -448,6 +514,8 @@ __device__ __forceinline__ void route_body(const Shape &sh, int B, const Workspa
         if (!ok) atomicExch(ws.status, ST_TICKET_TIMEOUT);
         s_last = ok;
     }
+    bool bad = false;
+    if (blockIdx.x == 0 && tid >= 32) bad = nonfinite_scan<ACT>(hidden, B * sh.d / (ACT == DT_F32 ? 4 : 8), tid - 32, THREADS - 32);
     // What the kernels behind accumulate into is cleared after the arrival (they touch it once this grid
     // has ended), by all blocks but the one that runs the gating.
     if (blockIdx.x > 0) {
@@ -460,9 +528,10 @@ __device__ __forceinline__ void route_body(const Shape &sh, int B, const Workspa
         }
     }
     if (blockIdx.x > 0) return;
-    __syncthreads();
+    bad = __syncthreads_or(bad) != 0;
     if (!s_last) return;
-    gating_block<JE>(sh, B, ws, conf, sh_scale ? 1 : 0, sel_idx, sel_w, n_unique, s_dyn, zl.ksplit, zl.lpart, zl.early);
+    gating_block<JE>(sh, B, ws, conf, sh_scale ? 1 : 0, sel_idx, sel_w, n_unique, s_dyn, zl.ksplit, zl.lpart, zl.early, bad,
+                     [&]() { repair_logits<ACT, RT>(B, sh.d, sh.E, n_rows, hidden, router, sh_scale, s_dyn, ws.logits, ws.gate_logit); });
 }
 
 // (bound of 768 threads instead of 512: at most 80 registers, so that a block fits beside a CTA of the
