@@ -121,10 +121,10 @@ typedef struct {
                                  (the kernel then starts while the routing still runs, on the
                                  shared experts and on the top_k experts of largest aggregated
                                  importance g_e (Eq. 4); one that turns out not to be selected
-                                 has been read for nothing.  The weights may be read as soon as
-                                 the call is on the stream; not for offloaded contexts), or with
-                                 block-int4 weights when d_model, d_ff and d_ff_shared are
-                                 multiples of 256 (it starts when the selection is known, before
+                                 has been read for nothing.  No weight is read before the work
+                                 in front of the call on its stream has ended; not for offloaded
+                                 contexts), or with block-int4 weights when d_model, d_ff and
+                                 d_ff_shared are multiples of 256 (it starts when the selection is known, before
                                  the gating has ended; the int4 values reach the
                                  tensor core as binary16 q * scale, rounded once: up to
                                  2^-12 relative per weight; block scales below 2^-17 lose

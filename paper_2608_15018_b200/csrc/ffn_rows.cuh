@@ -35,7 +35,9 @@
 // gets no tokens and no second projection.  The first projection of all others follows when the
 // selection is known, the second projection when warps 6..9 have built the tables from the finished
 // gating.  Early results wait in tensor memory (up to 16 accumulators) for the token lists.  Nothing but
-// weights is read before the routing kernel says that its own inputs are there.
+// weights is read before the routing kernel says that its own inputs are there, and no weights either in
+// the first layer of a call: what is in front of that in the stream is the caller's and may be writing them.
+// (In a later layer the library's own kernels are in front, and those of the first layer have waited.)
 //
 // Warp roles (352 threads): 0 TMA producer, 1 MMA issuer (owns the TMEM allocation), 2..5 and 6..9 two
 // epilogue sets that take alternate tasks (6..9 build the tables first), 10 watcher (early experts,
@@ -101,6 +103,7 @@ struct RwArgs {
     float *y;
     __nv_bfloat16 *act_hi, *act_lo;
     int B;
+    int first;           // first layer of a call: the kernel in front in the stream may be the caller's and write weights
     int mode;            // bit 0 / 1: in the gate|up maps of the routed / shared experts W_up comes first;
                          // bit 2 / 3: the two matrices are too far apart for one map (make_gateup_maps)
 };
@@ -422,7 +425,7 @@ ffn_rows_kernel(const __grid_constant__ RwMaps maps, const __grid_constant__ RwA
             const uint32_t ring_a = smem_u32(ring), full_a = smem_u32(full_bar);
             int s = 0, lim = lim0, level = 0, ready_w = 0;
             uint32_t par = 1;
-            bool alive = pl.x_bytes != 0 || inputs_wait();
+            bool alive = (pl.x_bytes != 0 && !p.first) || inputs_wait();
             // second-projection stages whose weights are in flight but whose token tiles wait for the
             // activations of wave pend_w: pend_n stages from ring slot pend_s, task pend_t, k-tile pend_k on
             int pend_n = 0, pend_s = 0, pend_t = 0, pend_k = 0, pend_w = 0;

@@ -577,7 +577,8 @@ int fetch_experts(s2moe_ctx *ctx, int layer, cudaStream_t st)
     return S2MOE_OK;
 }
 
-int verify_one(s2moe_ctx *ctx, int layer, int B, const void *hidden, const float *conf, float *out,
+// first: the first layer of a call (see RwArgs::first)
+int verify_one(s2moe_ctx *ctx, int layer, bool first, int B, const void *hidden, const float *conf, float *out,
                int32_t *sel_idx, float *sel_w, int32_t *n_unique, cudaStream_t st)
 {
     Shape sh = ctx->shape;
@@ -637,6 +638,7 @@ int verify_one(s2moe_ctx *ctx, int layer, int B, const void *hidden, const float
         RwArgs a;
         a.sh = sh; a.ws = ctx->ws; a.plan = rp; a.y = out; a.act_hi = ctx->act_hi; a.act_lo = ctx->act_lo; a.B = B;
         a.mode = ctx->rw_mode[layer];
+        a.first = first ? 1 : 0;
         LaunchScope scope(ctx, KC_TC, st);
         cudaLaunchConfig_t lc = pdl_config(ctx, rp.n_cta, kRwThreads, rp.smem_bytes, st, rp.early != 0);
         cudaLaunchKernelEx(&lc, ffn_rows_kernel, maps, a);
@@ -1019,7 +1021,7 @@ int s2moe_verify_layer(s2moe_ctx *ctx, int32_t layer, int32_t n_tokens, const vo
     if (rc != S2MOE_OK) return rc;
     if (layer < 0 || layer >= ctx->cfg.n_layers) return S2MOE_ERANGE;
     if (n_tokens == 0) return S2MOE_OK;
-    return verify_one(ctx, layer, n_tokens, hidden, conf, out, sel_idx, sel_w, n_unique,
+    return verify_one(ctx, layer, true, n_tokens, hidden, conf, out, sel_idx, sel_w, n_unique,
                       (cudaStream_t)cuda_stream);
 }
 
@@ -1031,7 +1033,7 @@ int s2moe_verify_stack(s2moe_ctx *ctx, int32_t n_tokens, const void *hidden, con
     const Shape &sh = ctx->shape;
     const size_t ab = sh.act_dtype == DT_F32 ? 4 : 2, B = (size_t)n_tokens;
     for (int l = 0; l < ctx->cfg.n_layers; ++l) {
-        rc = verify_one(ctx, l, n_tokens, (const uint8_t *)hidden + (size_t)l * B * sh.d * ab,
+        rc = verify_one(ctx, l, l == 0, n_tokens, (const uint8_t *)hidden + (size_t)l * B * sh.d * ab,
                         conf ? conf + (size_t)l * B : nullptr, out + (size_t)l * B * sh.d,
                         sel_idx + (size_t)l * B * sh.k, sel_w + (size_t)l * B * sh.k, n_unique + l,
                         (cudaStream_t)cuda_stream);
@@ -1087,7 +1089,7 @@ int s2moe_verify_stack_host(s2moe_ctx *ctx, int32_t n_tokens, const void *hidden
             CU(ctx, cudaEventRecord(ctx->ev_copy[0], ctx->cs_in));
             CU(ctx, cudaStreamWaitEvent(st, ctx->ev_copy[0], 0));
         }
-        rc = verify_one(ctx, l, n_tokens, (const uint8_t *)ctx->st_hidden + (size_t)l * hb,
+        rc = verify_one(ctx, l, l == 0, n_tokens, (const uint8_t *)ctx->st_hidden + (size_t)l * hb,
                         conf_host ? ctx->st_conf + (size_t)l * B : nullptr, ctx->st_out + (size_t)l * B * sh.d,
                         d_sel + (size_t)l * B * sh.k, d_selw + (size_t)l * B * sh.k, d_nu + l, st);
         if (rc == S2MOE_OK && (l + 1 == cut1 || l + 1 == cut2) && l + 1 > done) {
