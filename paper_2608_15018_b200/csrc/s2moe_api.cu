@@ -502,33 +502,58 @@ bool make_rows_maps(const s2moe_ctx *ctx, const LayerPtrs &lp, uint64_t n_w_expe
     return true;
 }
 
+// How a batch runs: kernel plan (0: the demanded one does not cover it) and the layout that goes with it.
+struct LayerPlan {
+    int plan = 0;
+    StPlan st{};
+    RwPlan rows{};
+    Q4Plan q4{};
+};
+
 // The plan a batch of B tokens runs with: the streaming kernel when it is allowed and its
 // shared-memory layout fits, else the CUDA-core kernels; 0 when plan 2 was demanded and does not fit.
-int plan_for(const s2moe_ctx *ctx, int B, StPlan *out)
+// gate_row: the router has a row for the shared experts' gate.  This is the one place that decides: what
+// it returns is launched as it is.
+LayerPlan plan_for(const s2moe_ctx *ctx, int B, bool gate_row)
 {
     const Shape &s0 = ctx->shape;
     const int want = ctx->cfg.kernel_plan;
-    if (want == 1) return 1;
+    LayerPlan p;
+    p.plan = 1;
+    if (want == 1) return p;
     if (want == 4) {
         // the whole layer in one launch, on demand only: measured slower than routing kernel + expert
         // kernel on every workload here (the gating runs two to three times longer inside the busy
         // CTAs than on a block of its own, and delays the first hand-over between the projections).
         // An offloaded context meets the host between routing and the experts: two launches.
-        if (ctx->offload || ctx->tc_maps.empty()) return 0;
+        p.plan = 0;
+        if (ctx->offload || ctx->tc_maps.empty()) return p;
         const fused::TcPlan tp = fused::tc_make_plan(s0, B, ctx->n_sm, B * s0.k + s0.n_sh * B);
-        return tp.feasible ? 4 : 0;
+        if (tp.feasible) p.plan = 4;
+        return p;
     }
-    if ((want == 0 || want == 3) && s0.weight_dtype == DT_BF16) {
-        if (!ctx->rw_maps.empty() && rw_make_plan(s0, B, ctx->n_sm, false, 0).feasible) return 3;
-        if (want == 3) return 0;
-    } else if (want == 0 || want == 3) {
-        if (!ctx->tc_maps.empty() && q4_make_plan(s0, B, ctx->n_sm, false).feasible) return 3;
-        if (want == 3) return 0;
+    if (want == 0 || want == 3) {
+        // tensor-core plan: the expert kernel starts while the gating still runs, on what the routing kernel
+        // announces (not with offloaded experts: their weights are fetched between the two kernels)
+        const bool early = ctx->early_start && ctx->use_pdl && !ctx->offload;
+        p.plan = 3;
+        if (s0.weight_dtype == DT_BF16 && !ctx->rw_maps.empty()) {
+            const bool by_tasks = route_by_tasks(ctx, s0.E + (gate_row ? 1 : 0), B);
+            p.rows = rw_make_plan(s0, B, ctx->n_sm, early, by_tasks ? 0 : (int)route_smem(B, s0.E, s0.k) + 256);
+            // (the early start needs tables for experts that may turn out not to be selected: without it
+            // there are fewer tasks)
+            if (!p.rows.feasible && early) p.rows = rw_make_plan(s0, B, ctx->n_sm, false, 0);
+            if (p.rows.feasible) return p;
+        } else if (s0.weight_dtype != DT_BF16 && !ctx->tc_maps.empty()) {
+            p.q4 = q4_make_plan(s0, B, ctx->n_sm, early);
+            if (p.q4.feasible) return p;
+        }
+        p.plan = 0;
+        if (want == 3) return p;
     }
-    const StPlan pl = st_make_plan(s0, B, ctx->n_sm, B * s0.k + s0.n_sh * B);
-    if (out) *out = pl;
-    if (pl.feasible) return 2;
-    return want == 2 ? 0 : 1;
+    p.st = st_make_plan(s0, B, ctx->n_sm, B * s0.k + s0.n_sh * B);
+    p.plan = p.st.feasible ? 2 : want == 2 ? 0 : 1;
+    return p;
 }
 
 // Expert offloading, between the routing kernel and the FFN kernel of a layer: read the list of
@@ -583,19 +608,15 @@ int verify_one(s2moe_ctx *ctx, int layer, bool first, int B, const void *hidden,
 {
     Shape sh = ctx->shape;
     const LayerPtrs &lp = ctx->layers[layer];
-    StPlan pl{};
-    const int plan = plan_for(ctx, B, &pl);
+    const LayerPlan how = plan_for(ctx, B, lp.sh_scale != nullptr);
+    const int plan = how.plan;
+    const StPlan &pl = how.st;
+    const RwPlan &rp = how.rows;
+    const Q4Plan &qp = how.q4;
     if (plan == 0) return S2MOE_EINVAL;
     sh.plan = plan;
     sh.op_cap = pl.op_cap;
-    // tensor-core plan: the expert kernel starts while the gating still runs, on what the routing kernel
-    // announces (not with offloaded experts: their weights are fetched between the two kernels)
-    const bool want_early = plan == 3 && ctx->early_start && ctx->use_pdl && !ctx->offload;
-    const bool rows3 = plan == 3 && sh.weight_dtype == DT_BF16;
-    const bool by_tasks = route_by_tasks(ctx, sh.E + (lp.sh_scale ? 1 : 0), B);
-    const RwPlan rp = rows3 ? rw_make_plan(sh, B, ctx->n_sm, want_early, by_tasks ? 0 : (int)route_smem(B, sh.E, sh.k) + 256) : RwPlan{};
-    const bool q4_3 = plan == 3 && !rows3;
-    const Q4Plan qp = q4_3 ? q4_make_plan(sh, B, ctx->n_sm, want_early) : Q4Plan{};
+    const bool rows3 = plan == 3 && sh.weight_dtype == DT_BF16, q4_3 = plan == 3 && !rows3;
     // what the FFN kernels accumulate into is cleared by the routing kernel's blocks
     ZeroList zl{};
     zl.ptr[0] = out;
@@ -943,7 +964,7 @@ int s2moe_create_offloaded(const s2moe_config *config, const s2moe_layer_weights
     std::memcpy(ctx->host_w.data(), layers, sizeof(LayerPtrs) * (size_t)L);
     // every batch size up to max_tokens must run on the tcgen05 kernel
     bool ok = !ctx->tc_maps.empty();
-    for (int B = 1; B <= config->max_tokens && ok; ++B) ok = plan_for(ctx, B, nullptr) == 3;
+    for (int B = 1; B <= config->max_tokens && ok; ++B) ok = plan_for(ctx, B, layers[0].sh_scale != nullptr).plan == 3;
     ctx->caches.resize((size_t)L);
     for (int l = 0; l < L && ok; ++l)
         ok = ctx->caches[(size_t)l].init(E, res->n_slots, res->n_pinned ? res->pinned + (size_t)l * res->n_pinned : nullptr,
@@ -1172,7 +1193,7 @@ int s2moe_last_cuda_error(const s2moe_ctx *ctx) { return ctx ? ctx->last_cuda : 
 int s2moe_kernel_plan(const s2moe_ctx *ctx, int32_t n_tokens)
 {
     if (!ctx || n_tokens < 1 || n_tokens > ctx->cfg.max_tokens) return 0;
-    return plan_for(ctx, n_tokens, nullptr);
+    return plan_for(ctx, n_tokens, ctx->layers[0].sh_scale != nullptr).plan;
 }
 
 int64_t s2moe_kernel_launches(const s2moe_ctx *ctx) { return ctx ? ctx->launches : 0; }

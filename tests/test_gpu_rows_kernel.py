@@ -62,3 +62,11 @@ def test_large_expert_count_and_width_still_run():
     wl = CONFIGS["cfg2"].with_(d_model=64, d_ff=14336, n_experts=256, top_k=16, cap=256, sigma=1.0, n_layers=1)
     rep, _ = run_case(wl, n_tokens=64, plan=3, tok_list=list(range(0, 64, 9)))
     assert rep.plan == 3
+
+
+def test_early_start_that_does_not_fit():
+    """One token of one wide expert: the plan fits for the expert that is selected, but not for one more that the
+    early start would read beside it, so the batch runs without the early start."""
+    wl = CONFIGS["cfg2"].with_(d_model=64, d_ff=400000, n_experts=2, top_k=1, cap=2, n_layers=1)
+    rep, _ = run_case(wl, n_tokens=1, plan=3)
+    assert rep.plan == 3 and rep.tokens_checked == 1
