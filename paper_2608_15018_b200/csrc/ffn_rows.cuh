@@ -63,7 +63,6 @@ constexpr int kRwThreads = 352;
 constexpr int kRwMaxStages = 8;
 constexpr int kRwMaxAcc = 16;
 constexpr int kRwWBytes = 32768;               // weight bytes of a stage: 8 row pairs x 2 k-tiles, or a 128-row block x 2 k-tiles
-constexpr int kRwMaxTasks = 1024;
 constexpr int kRwStaticSmem = 2048;            // static shared memory at most (barriers, lots, ids)
 constexpr int kRwMaxSmem = 232448 - kRwStaticSmem;
 constexpr int kRwSets = 2;                     // epilogue sets
@@ -71,12 +70,19 @@ constexpr int kRwMaxWaves = 4;
 constexpr int kRwLots2 = kRwMaxWaves + 1;      // lots of the second projection: wave 0, shared experts, other waves
 constexpr int kRwLevels = 3;                   // task lists: shared experts, early list, all experts, second projection
 
-// division of 0 <= n by a launch constant: n / d == umulhi(n, m) while n * d < 2^32 (checked on the host)
+// Division of 0 <= n < 2^31 by a launch constant d: with L = ceil(log2 d) and m = floor(2^(31 + L) / d) + 1, which
+// has 32 bits, n / d is n * m >> (31 + L): m * d exceeds 2^(31 + L) by at most 2^L, which n times is less than 2^(31 + L).
 struct RwDiv {
     unsigned d, m;
+    int s;               // L - 1
 };
-inline RwDiv rw_div_make(unsigned d) { return RwDiv{d, d <= 1 ? 0u : (unsigned)((0x100000000ull + d - 1) / d)}; }
-__device__ __forceinline__ int rw_div(int n, const RwDiv &v) { return v.d <= 1 ? n : (int)__umulhi((unsigned)n, v.m); }
+inline RwDiv rw_div_make(unsigned d)
+{
+    int L = 0;
+    while (L < 31 && (1u << L) < d) ++L;
+    return d <= 1 ? RwDiv{d, 0u, 0} : RwDiv{d, (unsigned)((1ull << (31 + L)) / d + 1), L - 1};
+}
+__device__ __forceinline__ int rw_div(int n, const RwDiv &v) { return v.d <= 1 ? n : (int)(__umulhi((unsigned)n, v.m) >> v.s); }
 
 struct RwPlan {
     int feasible;
@@ -172,7 +178,11 @@ inline RwPlan rw_make_plan(const Shape &sh, int B, int n_sm, bool early, int rou
     const long long n2r = U * p.rb.d * p.kr.d, n2s = sh.n_sh ? (long long)sh.n_sh * p.rb.d * p.ks.d : 0;
     const long long tasks = n1r / P / 8 + n1r / P / p.gf.d + n1s / P / 8 + n1s / P / p.gs.d + n2r / P / p.kr.d + n2s / P / p.ks.d +
                             4 * (kRwMaxWaves + kRwLots2 + 2);
-    if (tasks > kRwMaxTasks) return p;
+    // (unit numbers are 31-bit, those of the first projection also 8 times over; k-tiles are kept in 15 bits)
+    if (8 * (n1r + n1s) + 64 * P >= 1ll << 31 || n1r + n1s + n2r + n2s + 128 * P + 64 * P * (sh.d / 1024 + 1) >= 1ll << 31 ||
+        p.kr.d >= 1u << 14 || p.ks.d >= 1u << 14)
+        return p;
+    // (as many as there are: a table that leaves no room for two stages makes the plan infeasible)
     p.max_tasks = (int)tasks;
     const int nk = sh.d / 64;
     p.tab_bytes = ((int)sizeof(TcGroup) * (G + 1 + sh.n_sh) + 8 * n_slots + (int)sizeof(RwTask) * p.max_tasks + 1023) & ~1023;
@@ -190,11 +200,6 @@ inline RwPlan rw_make_plan(const Shape &sh, int B, int n_sm, bool early, int rou
     const int budget = beside ? shared : full;
     p.n_cta = p.early && !beside ? n_sm - 1 : n_sm;
     p.p = rw_div_make(p.n_cta);
-    // exactness of the divisions above
-    auto exact = [&](long long n, const RwDiv &v) { return (unsigned long long)n * v.d < 0x100000000ull; };
-    if (!exact(n1r + P, p.gf) || !exact(n1s + P, p.gs) || !exact(n2r + P, p.kr) || !exact(n2s + P, p.ks) ||
-        !exact(n2r + n2s + n1r + n1s + 64 * P, p.p) || !exact(n2r + n2s + P, p.rb))
-        return p;
     // Hidden states resident where at least three stages fit beside them; else their tiles travel
     // with the stages, one copy more and at most one chunk of two k-tiles per stage.  Measured, us per
     // layer, three stages with resident tiles / five without: DeepSeek-V2-Lite shape at 16 tokens 54.5 /
@@ -921,7 +926,7 @@ ffn_rows_kernel(const __grid_constant__ RwMaps maps, const __grid_constant__ RwA
                     const RwDiv kd = sx ? pl.ks : pl.kr;
                     RwTask *t = &tasks[i];
                     int u, len;
-                    rw_seg_task(s_lot2[l], kd, 24, RwDiv{1u, 0u}, i - s_first2[l], u, len);
+                    rw_seg_task(s_lot2[l], kd, 24, RwDiv{1u, 0u, 0}, i - s_first2[l], u, len);
                     const int gq = rw_div(u, kd), in = u - gq * (int)kd.d, eq = rw_div(gq, pl.rb), rbk = gq - eq * RB;
                     // (wave 0: the early experts that have tokens, then the others)
                     const int a = sx ? GP + eq : (w > 0 || n_bad == 0 ? eq + (real ? s_bound[w] : 0) : (eq < pl.n_early - n_bad ? (int)s_sel[eq] : eq + n_bad));

@@ -70,3 +70,12 @@ def test_early_start_that_does_not_fit():
     wl = CONFIGS["cfg2"].with_(d_model=64, d_ff=400000, n_experts=2, top_k=1, cap=2, n_layers=1)
     rep, _ = run_case(wl, n_tokens=1, plan=3)
     assert rep.plan == 3 and rep.tokens_checked == 1
+
+
+@pytest.mark.parametrize("E,k,f,B", [(2, 1, 400000, 2), (256, 16, 40000, 16)])
+def test_very_wide_experts(E, k, f, B):
+    """More units of the first projection than a 32-bit product with the units of an expert holds, and more tasks per
+    CTA than 1024: both are bounded by the shared memory of the table only."""
+    wl = CONFIGS["cfg2"].with_(d_model=64, d_ff=f, n_experts=E, top_k=k, cap=E, sigma=1.0, n_layers=1)
+    rep, _ = run_case(wl, n_tokens=B, plan=3, tok_list=[0, B - 1])
+    assert rep.plan == 3 and rep.tokens_checked == 2
