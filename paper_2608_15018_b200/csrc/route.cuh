@@ -406,7 +406,7 @@ __device__ __forceinline__ void route_body(const Shape &sh, int B, const Workspa
                                            const float *__restrict__ conf, int32_t *__restrict__ sel_idx,
                                            float *__restrict__ sel_w, int32_t *__restrict__ n_unique, const ZeroList &zl)
 {
-    extern __shared__ double s_dyn[];
+    extern __shared__ __align__(16) double s_dyn[];       // (the gating reads parts of it 16 bytes at a time)
     __shared__ int s_last;
     const int tid = threadIdx.x;
     // Programmatic dependent launch: everything this kernel writes is read by the kernels of the layer in
