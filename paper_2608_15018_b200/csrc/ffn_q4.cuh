@@ -96,7 +96,8 @@ inline Q4Plan q4_make_plan(const Shape &sh, int B, int n_sm, bool early)
     // full share)
     p.early = early && n_sm > 1 ? 1 : 0;
     p.n_cta = n_sm - p.early;
-    p.feasible = p.stages >= 4 && B <= kMaxTokens && sh.weight_dtype == DT_Q4B32 && sh.act_dtype == DT_BF16 && sh.d % 256 == 0 &&
+    // (three stages at the limits: 60 and more tokens of 14 and more of 256 experts beside 4 shared ones; never less)
+    p.feasible = p.stages >= 3 && B <= kMaxTokens && sh.weight_dtype == DT_Q4B32 && sh.act_dtype == DT_BF16 && sh.d % 256 == 0 &&
                  sh.f % 256 == 0 && (sh.n_sh == 0 || sh.f_sh % 256 == 0);
     return p;
 }

@@ -43,3 +43,11 @@ def test_row_blocks_without_tokens(B):
     for _ in range(4):
         rep, _ = run_case(wl, n_tokens=B, plan=3)
         assert rep.plan == 3 and rep.tokens_checked == B
+
+
+def test_largest_tables():
+    """All limits at once: the tables leave three stages of the ring."""
+    wl = CONFIGS["cfg4"].with_(d_model=512, d_ff=256, d_ff_shared=512, n_shared=4, shared_gate=True, n_experts=256, top_k=16,
+                               cap=256, sigma=1.0, n_layers=1)
+    rep, _ = run_case(wl, n_tokens=64, plan=3, tok_list=list(range(0, 64, 7)))
+    assert rep.plan == 3
