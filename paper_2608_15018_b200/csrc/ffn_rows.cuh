@@ -34,7 +34,7 @@
 // and without the bias, at most 0.1 of them is not.  An expert that is not has been read for nothing: it
 // gets no tokens and no second projection.  The first projection of all others follows when the
 // selection is known, the second projection when warps 6..9 have built the tables from the finished
-// gating.  Early results wait in tensor memory (up to 16 accumulators) for the token lists.  Nothing but
+// gating.  Early results wait in tensor memory (two or four tasks) for the token lists.  Nothing but
 // weights is read before the routing kernel says that its own inputs are there, and no weights either in
 // the first layer of a call: what is in front of that in the stream is the caller's and may be writing them.
 // (In a later layer the library's own kernels are in front, and those of the first layer have waited.)
@@ -47,9 +47,13 @@
 // weights), which is why one issuer is enough.
 // Measured, us per layer, split-K kernel before / this one: OLMoE shape 8 tokens 52 / 42, Qwen1.5-MoE
 // shape 16 tokens 54.6 / 42, DeepSeek-V2-Lite shape 16 tokens 60 / 52, 64 tokens 140 / 129.
-// Even and odd k-tiles go to two accumulators that the epilogue adds: the tensor core truncates when
-// it adds to an accumulator, so half the chain is half the error (relative 2-norm against the float64
-// oracle 5.3e-6 with one chain of 128 steps).
+// The tensor core truncates when it adds to an accumulator, so the k-tiles of a task go in turn to several
+// accumulators (chains) that the epilogue adds: eight in the first projection up to 16 tokens, four above, and as
+// many as their columns hold in the second one.  Relative 2-norm of the error against float64, two / four /
+// eight chains in the first projection: OLMoE shape 1 token 3.2e-6 / 2.6e-6 / 2.4e-6, 8 tokens 3.4e-6 / 2.7e-6 /
+// 2.5e-6, 64 tokens 3.8e-6 / 2.8e-6 / -, 128 narrow experts 13 tokens 3.5e-6 / 2.7e-6 / 2.5e-6, 128 wide ones
+// 8 tokens 4.5e-6 / 3.0e-6 / 2.6e-6 (one chain, OLMoE shape 8 tokens: 5.3e-6); the split-K kernel had 2.5e-6,
+// 2.8e-6, 3.1e-6, 2.7e-6 and 4.0e-6.
 #pragma once
 
 #include <cuda.h>
@@ -61,7 +65,7 @@ namespace s2moe {
 
 constexpr int kRwThreads = 352;
 constexpr int kRwMaxStages = 8;
-constexpr int kRwMaxAcc = 16;
+constexpr int kRwMaxAcc = 4;
 constexpr int kRwWBytes = 32768;               // weight bytes of a stage: 8 row pairs x 2 k-tiles, or a 128-row block x 2 k-tiles
 constexpr int kRwStaticSmem = 2048;            // static shared memory at most (barriers, lots, ids)
 constexpr int kRwMaxSmem = 232448 - kRwStaticSmem;
@@ -91,6 +95,7 @@ struct RwPlan {
     int n1;              // N of the first projection's MMAs: tokens padded to 16
     int xr;              // rows of a resident hidden-state tile (8 up to 8 tokens: the MMA's other 8 columns are not read)
     int x_bytes;         // > 0: the hidden states stay resident in shared memory
+    int c1;              // chains of a first-projection task
     int acc_cols, n_acc, tmem_cols;
     int max_tasks;
     int tab_bytes;
@@ -134,6 +139,12 @@ struct RwTask {
 };
 static_assert(sizeof(RwTask) == 32, "layout");
 
+// chains of a second-projection task of `rows` slots: 2 * rows columns each (hi and lo parts)
+__device__ __forceinline__ int rw_chains2(int acc_cols, int rows)
+{
+    return 16 * rows <= acc_cols ? 8 : 8 * rows <= acc_cols ? 4 : 2;
+}
+
 // rows of the activation box that holds T tokens
 __host__ __device__ __forceinline__ int rw_tok_rows(int T) { return T <= 8 ? 8 : (T <= 16 ? 16 : (T <= 32 ? 32 : 64)); }
 
@@ -159,7 +170,8 @@ inline RwPlan rw_make_plan(const Shape &sh, int B, int n_sm, bool early, int rou
     // resident tiles and a routing block).
     p.one_rows = trows >= 32 ? trows : 0;
     const int tok2 = (p.one_rows ? 1 : 2) * 2 * trows * 128, tok1 = 2 * p.n1 * 128;
-    p.acc_cols = 2 * trows > 2 * p.n1 ? 2 * trows : 2 * p.n1;       // (32, 64, 128: a power of two)
+    p.c1 = p.n1 == 16 ? 8 : 4;
+    p.acc_cols = p.c1 * p.n1 > 4 * trows ? p.c1 * p.n1 : 4 * trows;       // (128, 256: a power of two)
     while (p.acc_cols & (p.acc_cols - 1)) p.acc_cols += 32;
     p.n_acc = 512 / p.acc_cols;
     if (p.n_acc > kRwMaxAcc) p.n_acc = kRwMaxAcc;
@@ -268,19 +280,32 @@ __device__ __forceinline__ void rw_mma(uint32_t d_tmem, uint64_t a_desc, uint64_
         "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(acc)
         : "memory");
 }
-// sums of eight columns at t0 and eight at t1
-__device__ __forceinline__ void rw_ld8_sum(uint32_t t0, uint32_t t1, float (&v)[8])
+// sums of eight columns at t, t + step, .. (n pieces, four loaded at a time)
+__device__ __forceinline__ void rw_ld8_sums(uint32_t t, uint32_t step, int n, float (&v)[8])
 {
-    uint32_t r[8], s[8];
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                 : "r"(t0));
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                 : "=r"(s[0]), "=r"(s[1]), "=r"(s[2]), "=r"(s[3]), "=r"(s[4]), "=r"(s[5]), "=r"(s[6]), "=r"(s[7])
-                 : "r"(t1));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]) + __uint_as_float(s[i]);
+    for (int j = 0; j < 8; ++j) v[j] = 0.0f;
+#pragma unroll 1
+    for (; n >= 4; n -= 4, t += 4 * step) {
+        uint32_t r[32];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                         : "=r"(r[8 * i]), "=r"(r[8 * i + 1]), "=r"(r[8 * i + 2]), "=r"(r[8 * i + 3]), "=r"(r[8 * i + 4]),
+                           "=r"(r[8 * i + 5]), "=r"(r[8 * i + 6]), "=r"(r[8 * i + 7])
+                         : "r"(t + step * i));
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            v[j] += (__uint_as_float(r[j]) + __uint_as_float(r[8 + j])) + (__uint_as_float(r[16 + j]) + __uint_as_float(r[24 + j]));
+    }
+#pragma unroll 1
+    for (; n > 0; --n, t += step) {
+        float w[8];
+        tc_ld8(t, w);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v[j] += w[j];
+    }
 }
 
 // A lot: units in groups of g.d, dealt to the CTAs in contiguous shares.  Of this CTA's share: first
@@ -572,7 +597,7 @@ ffn_rows_kernel(const __grid_constant__ RwMaps maps, const __grid_constant__ RwA
                 }
                 const uint32_t d_tmem = tmem_base + buf * (uint32_t)pl.acc_cols;
                 if (!(flags & 1)) {
-                    const int np = flags >> 8, cps = pl.x_bytes ? 8 / np : 1;
+                    const int np = flags >> 8, cps = pl.x_bytes ? 8 / np : 1, last = pl.c1 - 1;
                     for (int kt = 0; kt < nk; kt += 2 * cps) {
                         if (!mbar_wait(&full_bar[s], par)) { atomicExch(ws.status, ST_MBAR_TIMEOUT); alive = false; break; }
                         tc_fence_after();
@@ -586,8 +611,8 @@ ffn_rows_kernel(const __grid_constant__ RwMaps maps, const __grid_constant__ RwA
                                 if (k + q < ke) {
 #pragma unroll
                                     for (int h = 0; h < 4; ++h)
-                                        rw_mma(d_tmem + (uint32_t)(q * pl.n1), ad + (uint64_t)(64 * q + 2 * h),
-                                               bd + (uint64_t)(x_step * q + 2 * h), idesc1, h > 0 || k > 0 ? 1u : 0u);
+                                        rw_mma(d_tmem + (uint32_t)((q + (k & last)) * pl.n1), ad + (uint64_t)(64 * q + 2 * h),
+                                               bd + (uint64_t)(x_step * q + 2 * h), idesc1, h > 0 || k + q > last ? 1u : 0u);
                                 }
                             }
                             ad += (uint64_t)(np * 256);
@@ -599,8 +624,7 @@ ffn_rows_kernel(const __grid_constant__ RwMaps maps, const __grid_constant__ RwA
                 } else {
                     const int k1 = tk >> 16, k0 = tk & 0xffff, rows = flags >> 8;
                     const uint32_t idesc = tc_idesc(2 * rows);
-                    // (the columns of an accumulator leave room for two chains up to half the batch)
-                    const bool twin = 4 * rows <= pl.acc_cols;
+                    const int last = rw_chains2(pl.acc_cols, rows) - 1;
                     const int step = rows == pl.one_rows ? 1 : 2;
                     for (int kt = k0; kt < k1; kt += step) {
                         if (!mbar_wait(&full_bar[s], par)) { atomicExch(ws.status, ST_MBAR_TIMEOUT); alive = false; break; }
@@ -611,8 +635,8 @@ ffn_rows_kernel(const __grid_constant__ RwMaps maps, const __grid_constant__ RwA
                             if (q < step && kt + q < k1) {
 #pragma unroll
                                 for (int h = 0; h < 4; ++h)
-                                    rw_mma(d_tmem + (q && twin ? 2u * (uint32_t)rows : 0u), ad + (uint64_t)(1024 * q + 2 * h),
-                                           bd + (uint64_t)(rows * 16 * q + 2 * h), idesc, h > 0 || kt > k0 || (q && !twin) ? 1u : 0u);
+                                    rw_mma(d_tmem + (uint32_t)(2 * rows * ((kt + q - k0) & last)), ad + (uint64_t)(1024 * q + 2 * h),
+                                           bd + (uint64_t)(rows * 16 * q + 2 * h), idesc, h > 0 || kt + q - k0 > last ? 1u : 0u);
                             }
                         }
                         tc_commit(&empty_bar[s]);
@@ -998,16 +1022,11 @@ ffn_rows_kernel(const __grid_constant__ RwMaps maps, const __grid_constant__ RwA
                 const int fr = t.pos + pair * 8 + (L & 7);
                 const size_t base = shd ? (size_t)n_routed * sh.f + (size_t)(g.off - n_routed) * sh.f_sh + fr : (size_t)g.off * sh.f + fr;
                 const size_t stride = shd ? (size_t)sh.f_sh : (size_t)sh.f;
-                const uint32_t second = nk > 1 ? (uint32_t)pl.n1 : 0u;
                 for (int c = 0; c < p.B; c += 8) {
                     const unsigned m8 = (unsigned)((g.mask >> c) & 0xffull);
                     if (m8 == 0u) continue;
                     float v[8];
-                    if (second) {
-                        rw_ld8_sum(taddr + c, taddr + second + c, v);
-                    } else {
-                        tc_ld8(taddr + c, v);
-                    }
+                    rw_ld8_sums(taddr + c, (uint32_t)pl.n1, min(pl.c1, nk), v);      // (a chain without a k-tile is not read)
                     int rank = __popcll(g.mask & ((1ull << c) - 1ull));
 #pragma unroll
                     for (int j = 0; j < 8; j += 2) {
@@ -1028,15 +1047,10 @@ ffn_rows_kernel(const __grid_constant__ RwMaps maps, const __grid_constant__ RwA
             } else {
                 const int row = t.pos + q * 32 + lane, rows = t.flags >> 8;
                 const bool row_ok = row < sh.d;
-                const bool twin = 4 * rows <= pl.acc_cols && (t.k >> 16) - (t.k & 0xffff) > 1;
+                const int pieces = 2 * min(rw_chains2(pl.acc_cols, rows), (t.k >> 16) - (t.k & 0xffff));   // hi and lo of every chain
                 for (int c = 0; c < g.T; c += 8) {
-                    float v[8], w[8];
-                    rw_ld8_sum(taddr + c, taddr + rows + c, v);
-                    if (twin) {
-                        rw_ld8_sum(taddr + 2 * rows + c, taddr + 3 * rows + c, w);
-#pragma unroll
-                        for (int j = 0; j < 8; ++j) v[j] += w[j];
-                    }
+                    float v[8];
+                    rw_ld8_sums(taddr + c, (uint32_t)rows, pieces, v);
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
                         if (c + j < g.T && row_ok) {

@@ -79,3 +79,16 @@ def test_very_wide_experts(E, k, f, B):
     wl = CONFIGS["cfg2"].with_(d_model=64, d_ff=f, n_experts=E, top_k=k, cap=E, sigma=1.0, n_layers=1)
     rep, _ = run_case(wl, n_tokens=B, plan=3, tok_list=[0, B - 1])
     assert rep.plan == 3 and rep.tokens_checked == 2
+
+
+# Relative 2-norm of a token's error, the largest over the batch.  The bf16 hi + lo parts of the activations give about
+# 2.4e-6; what the tensor core truncates at every accumulation adds to it in proportion to the length L of a chain:
+# the sum of squares of 2.4e-6 and c * L fits two, four and eight chains with c = 3.7e-8 (OLMoE width, L = 64, 32, 16).
+# The bounds lie half way between the measured errors (2.5, 3.0, 3.1, 3.2, 3.6, 2.7, 2.7 and 3.6e-6) and those of
+# chains of twice and four times the length (3.2, 4.5, 4.8, 4.8, 4.8, 3.7, 4.6 and 5.5e-6).
+@pytest.mark.parametrize("cfg,B,bound", [("cfg2", 1, 2.9e-6), ("cfg2", 8, 3.7e-6), ("cfg2", 20, 3.9e-6), ("cfg2", 48, 4.0e-6),
+                                         ("cfg2", 64, 4.2e-6), ("cfg3", 16, 3.2e-6), ("e128b", 8, 3.6e-6), ("e128b", 64, 4.5e-6)])
+def test_error_against_float64(cfg, B, bound):
+    wl = CONFIGS[cfg].with_(n_experts=16, cap=2 * CONFIGS[cfg].top_k)
+    rep, _ = run_case(wl, n_tokens=B, plan=3)
+    assert rep.plan == 3 and rep.rms_rel_err <= bound
