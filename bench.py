@@ -35,10 +35,9 @@ UNIT = "tokens/s"
 FALLBACK_HBM_GBS = 6650.0
 
 
-# DRAM bytes (read + write) per algorithmic byte, from the ncu captures summarised under profiles/
-# (expert_kernels_plan3.md, ffn_stream_kernel_cfg2_2layers.md); traffic grows with the
-# number of distinct experts exactly as the algorithmic bytes do.
-TRAFFIC_RATIO = {"ffn_tc_kernel": 1.02, "ffn_tc_kernel/int4": 1.02, "ffn_stream_kernel": 1.005}
+# DRAM bytes (read + write) per algorithmic byte, from the ncu captures summarised under profiles/;
+# traffic grows with the number of distinct experts exactly as the algorithmic bytes do.
+TRAFFIC_RATIO = {"ffn_rows_kernel": 1.02, "ffn_q4_kernel": 1.02, "ffn_stream_kernel": 1.005}
 
 
 def parse_args():
@@ -206,7 +205,7 @@ def run_reference(args, wl, B, sigma):
     print(json.dumps(line), flush=True)
 
 
-def roofline_of(kernels, step_bytes, steps, L, q4, peak, peak_kind):
+def roofline_of(kernels, step_bytes, steps, L, peak, peak_kind):
     """Roofline figures of the kernel with the largest summed duration in an event-timed region."""
     if not kernels:
         return None
@@ -218,8 +217,7 @@ def roofline_of(kernels, step_bytes, steps, L, q4, peak, peak_kind):
     share = {"ffn_gateup_simple": 2.0 / 3.0, "ffn_down_simple": 1.0 / 3.0}.get(dom, 1.0)
     bytes_per_launch = share * step_bytes / L / max(launches_per_layer, 1e-9)
     achieved = bytes_per_launch / (per_launch_ms * 1e-3) / 1e9
-    base = dom.split("/")[0]
-    ratio = TRAFFIC_RATIO.get(base + "/int4" if q4 else base, TRAFFIC_RATIO.get(base))
+    ratio = TRAFFIC_RATIO.get(dom)
     return {"bound": "hbm", "kernel": dom, "achieved": achieved, "peak": peak, "unit": "GB/s",
             "frac": achieved / peak, "peak_kind": f"of {peak_kind}",
             "traffic": ratio * bytes_per_launch if ratio else None,
@@ -385,7 +383,7 @@ def measure_stack(wl, B, sigma, L, plan, steps, warmup, dev, rank, world, peak, 
         "repeat_ms_min_median_max": [min(graph_all), statistics.median(graph_all), max(graph_all)] if graph_all else None,
         "stream_ms_per_step_with_kernel_events": stream_ms_total / steps,
         "kernels": kernels,
-        "roofline": roofline_of(kernels, step_bytes, steps, L, wl.weight_dtype == workloads.Q4B32, peak, peak_kind),
+        "roofline": roofline_of(kernels, step_bytes, steps, L, peak, peak_kind),
         "gpu_launches_per_step": launches_per_step,
         "clocks": clocks, "device_status": status,
         "l2": f"inputs larger than L2: {step_bytes / 1e9:.2f} GB of expert weights per step",

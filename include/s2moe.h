@@ -281,7 +281,7 @@ double s2moe_unique_expert_bytes(const s2moe_ctx *ctx, int32_t n_unique);
  * number of timed launches.  s2moe_kernel_class_name gives the kernel's name, or
  * NULL past the last class.  Do not use during stream capture.
  */
-#define S2MOE_KERNEL_CLASSES 6
+#define S2MOE_KERNEL_CLASSES 7
 int s2moe_profile_begin(s2moe_ctx *ctx, int32_t max_records);
 int s2moe_profile_end(s2moe_ctx *ctx, int32_t n_classes, double *ms_out, int64_t *launches_out);
 const char *s2moe_kernel_class_name(int32_t cls);

@@ -70,8 +70,8 @@ constexpr int kRwWBytes = 32768;               // weight bytes of a stage: 8 row
 constexpr int kRwStaticSmem = 2048;            // static shared memory at most (barriers, lots, ids)
 constexpr int kRwMaxSmem = 232448 - kRwStaticSmem;
 constexpr int kRwSets = 2;                     // epilogue sets
-constexpr int kRwMaxWaves = 4;
-constexpr int kRwLots2 = kRwMaxWaves + 1;      // lots of the second projection: wave 0, shared experts, other waves
+constexpr int kRwMaxWaves = 2;
+constexpr int kRwLots2 = kRwMaxWaves + 1;      // lots of the second projection: wave 0, shared experts, wave 1
 constexpr int kRwLevels = 3;                   // task lists: shared experts, early list, all experts, second projection
 
 // Division of 0 <= n < 2^31 by a launch constant d: with L = ceil(log2 d) and m = floor(2^(31 + L) / d) + 1, which
@@ -102,7 +102,7 @@ struct RwPlan {
     int smem_bytes;
     int early, n_early;           // early start; its experts
     int one_rows;                 // second-projection tasks of that many slots take one k-tile per stage (0: none)
-    int split16[kRwMaxWaves - 1];   // where waves 1, 2, 3 begin, in 16ths of the first projection (16: no such wave)
+    int split16;         // where wave 1 begins, in 16ths of the first projection
     int delta;           // second-projection units that weigh as much as one first-projection unit
     RwDiv gf, gs, tf, ts, kr, ks, rb, p;   // row groups and tasks of a routed / shared expert, P2 units of their row blocks, row blocks, CTAs
 };
@@ -135,7 +135,7 @@ struct RwTask {
     int srow;            // P2: row of the activation map
     int a;               // group slot
     int pos;             // P1: first row of the inner dimension; P2: first output row
-    int pad0, pad1;
+    int pad[2];
 };
 static_assert(sizeof(RwTask) == 32, "layout");
 
@@ -184,12 +184,13 @@ inline RwPlan rw_make_plan(const Shape &sh, int B, int n_sm, bool early, int rou
     p.ks = rw_div_make(sh.n_sh ? (sh.f_sh + 127) / 128 : 1);
     p.rb = rw_div_make((sh.d + 127) / 128);
     // tasks of a CTA at most: a share of n units in groups of g, m units per task, meets n / g + 2 groups,
-    // and every group adds at most one ragged task to n / m whole ones
+    // and every group adds at most one ragged task to n / m whole ones (44: four per lot, and room for what
+    // `delta` moves from one CTA to another and for the tables' first pass)
     const long long P = n_sm - 1 > 0 ? n_sm - 1 : 1, U = sh.E < (long long)B * sh.k + p.n_early ? sh.E : (long long)B * sh.k + p.n_early;
     const long long n1r = U * p.gf.d, n1s = sh.n_sh ? (long long)sh.n_sh * p.gs.d : 0;
     const long long n2r = U * p.rb.d * p.kr.d, n2s = sh.n_sh ? (long long)sh.n_sh * p.rb.d * p.ks.d : 0;
     const long long tasks = n1r / P / 8 + n1r / P / p.gf.d + n1s / P / 8 + n1s / P / p.gs.d + n2r / P / p.kr.d + n2s / P / p.ks.d +
-                            4 * (kRwMaxWaves + kRwLots2 + 2);
+                            44;
     // (unit numbers are 31-bit, those of the first projection also 8 times over; k-tiles are kept in 15 bits)
     if (8 * (n1r + n1s) + 64 * P >= 1ll << 31 || n1r + n1s + n2r + n2s + 128 * P + 64 * P * (sh.d / 1024 + 1) >= 1ll << 31 ||
         p.kr.d >= 1u << 14 || p.ks.d >= 1u << 14)
@@ -231,13 +232,11 @@ inline RwPlan rw_make_plan(const Shape &sh, int B, int n_sm, bool early, int rou
         if (p.stages >= (res ? 3 : 2)) { p.feasible = 1; break; }
     }
     if (!p.feasible) return p;
-    // Two waves.  Measured, us per layer, wave 1 from 8/16 / waves 1 and 2 from 8/16 and 13/16: OLMoE shape at 8
+    // Two waves, cut in the middle.  Measured, us per layer, with a third one from 13/16 on: OLMoE shape at 8
     // tokens 40.9 / 41.0, one token 32.1 / 32.4, DeepSeek-V2-Lite shape at 16 tokens 51.7 / 52.4, at 64
     // 126.5 / 127.9, Qwen1.5-MoE shape 42.3 / 43.1, 128 narrow experts at 13 tokens 38.3 / 38.2, 128 wide ones
     // at 8 75.4 / 76.2.
-    p.split16[0] = 8;
-    p.split16[1] = 16;
-    p.split16[2] = 16;
+    p.split16 = 8;
     p.delta = (sh.d + 512) / 1024;
     return p;
 }
@@ -773,11 +772,11 @@ ffn_rows_kernel(const __grid_constant__ RwMaps maps, const __grid_constant__ RwA
                 __syncwarp();
             }
             // lane w: wave w begins at the first routed group whose first projection lies past split16 / 16
-            // of all of it (the early and the shared experts are in wave 0); lane 4: the end
+            // of all of it (the early and the shared experts are in wave 0); lane kRwMaxWaves: the end
             int bnd = 0;
             if (lane > 0 && lane < kRwMaxWaves) {
-                const int s16 = pl.split16[lane - 1], want = ((U * Gf + n_sh_units) * s16 >> 4) - n_sh_units;
-                bnd = s16 >= 16 ? U : min(U, max(rw_div(max(want, 0) + Gf - 1, pl.gf), max(n_early, sh.n_sh ? 0 : 1)));
+                const int want = ((U * Gf + n_sh_units) * pl.split16 >> 4) - n_sh_units;
+                bnd = min(U, max(rw_div(max(want, 0) + Gf - 1, pl.gf), max(n_early, sh.n_sh ? 0 : 1)));
             } else if (lane >= kRwMaxWaves) {
                 bnd = U;
             }

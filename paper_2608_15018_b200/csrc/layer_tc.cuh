@@ -56,12 +56,11 @@ struct TcPlan {
     int tok_off;       // offset of the token tiles inside a stage
     int kg;            // k-tiles per stage (1 for bf16 weights; 1, 2 or 4 for int4)
     int tokb;          // bytes of the token tiles of one k-tile
-    int fused;         // the kernel also routes and gates (one launch per layer)
-    int gate_bytes;    // fused: shared memory of the gating (staged logits and its tables)
-    int ksplit;        // fused: pieces of the contraction a router row is cut into
+    int gate_bytes;    // shared memory of the gating (staged logits and its tables)
+    int ksplit;        // pieces of the contraction a router row is cut into
 };
 
-// what the fused layer kernel needs for its routing stage (unused by the two-launch form)
+// what the kernel needs for its routing stage
 struct TcRoute {
     const void *hidden, *router, *sh_scale;     // [B][d] bf16, [E][d] router dtype, [d] or NULL
     const float *conf;                          // [B] or NULL
@@ -96,7 +95,6 @@ inline TcPlan tc_make_plan(const Shape &sh, int B, int n_sm, int n_slots)
     const int G = sh.E + sh.n_sh;
     p.n_cta = n_sm;
     p.n1 = (B + 15) & ~15;
-    p.fused = 1;
     {
         p.gate_bytes = (int)((8 * ((size_t)B * sh.E + 2 * (size_t)B) + gate_mem_bytes(sh.E, B, sh.k) + 64 + 15) & ~(size_t)15);   // logits, confidences, gate logits, tables
         // a router row is cut into pieces so that the warps of all CTAs share the logit pass

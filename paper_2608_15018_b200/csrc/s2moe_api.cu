@@ -84,7 +84,7 @@ struct s2moe_cache {
     ExpertCache c;
 };
 
-enum KernelClass { KC_ROUTER = 0, KC_GATING = 1, KC_GATEUP = 2, KC_DOWN = 3, KC_STREAM = 4, KC_TC = 5, KC_LAYER = 6, KC_COUNT = 7 };
+enum KernelClass { KC_ROUTER = 0, KC_Q4 = 1, KC_GATEUP = 2, KC_DOWN = 3, KC_STREAM = 4, KC_ROWS = 5, KC_LAYER = 6, KC_COUNT = 7 };
 
 namespace {
 
@@ -660,7 +660,7 @@ int verify_one(s2moe_ctx *ctx, int layer, bool first, int B, const void *hidden,
         a.sh = sh; a.ws = ctx->ws; a.plan = rp; a.y = out; a.act_hi = ctx->act_hi; a.act_lo = ctx->act_lo; a.B = B;
         a.mode = ctx->rw_mode[layer];
         a.first = first ? 1 : 0;
-        LaunchScope scope(ctx, KC_TC, st);
+        LaunchScope scope(ctx, KC_ROWS, st);
         cudaLaunchConfig_t lc = pdl_config(ctx, rp.n_cta, kRwThreads, rp.smem_bytes, st, rp.early != 0);
         cudaLaunchKernelEx(&lc, ffn_rows_kernel, maps, a);
     } else if (plan == 3 || plan == 4) {
@@ -688,7 +688,7 @@ int verify_one(s2moe_ctx *ctx, int layer, bool first, int B, const void *hidden,
             Q4Args a;
             a.sh = sh; a.ws = ctx->ws; a.plan = qp; a.y = out; a.pre = ctx->pre;
             a.act_hi = ctx->act_hi; a.act_lo = ctx->act_lo; a.B = B;
-            LaunchScope scope(ctx, KC_TC, st);
+            LaunchScope scope(ctx, KC_Q4, st);
             cudaLaunchConfig_t lc = pdl_config(ctx, qp.n_cta, kQ4Threads, qp.smem_bytes, st, qp.early != 0);
             cudaLaunchKernelEx(&lc, ffn_q4_kernel, maps, a);
         } else {
@@ -1246,11 +1246,11 @@ const char *s2moe_kernel_class_name(int32_t cls)
 {
     switch (cls) {
         case KC_ROUTER: return "route_kernel";
-        case KC_GATING: return "(unused)";
+        case KC_Q4: return "ffn_q4_kernel";
         case KC_GATEUP: return "ffn_gateup_simple";
         case KC_DOWN: return "ffn_down_simple";
         case KC_STREAM: return "ffn_stream_kernel";
-        case KC_TC: return "ffn_tc_kernel";
+        case KC_ROWS: return "ffn_rows_kernel";
         case KC_LAYER: return "layer_tc_kernel";
         default: return nullptr;
     }
@@ -1275,7 +1275,6 @@ int s2moe_debug_read(s2moe_ctx *ctx, int32_t what, void *host_out, size_t bytes)
         case 5: src = ctx->ws.active; need = 4 * (size_t)hdr[0]; break;
         case 6: src = ctx->ws.header; need = 16; break;
         case 7: src = ctx->ws.header + 8; need = 32; break;
-        case 8: src = ctx->ws.act; need = bytes; break;   // timing build: per-warp cycle counters
         default: return S2MOE_EINVAL;
     }
     if (bytes < need) return S2MOE_EINVAL;
