@@ -29,7 +29,7 @@
 // Early start: see route.cuh.  The kernel is resident while the routing kernel still runs (its blocks
 // are small enough to share the SMs), even before the layer in front has ended.  It streams the weights
 // of the shared experts' first projection at once; as soon as the router's logits are there, and beside
-// the gating, the first projection of the top_k experts of largest aggregated importance g_e (Eq. 4),
+// the gating, the first projection of the top_k experts (RwPlan::n_early) of largest aggregated importance g_e (Eq. 4),
 // which are nearly always selected: over the shapes of the workloads, 1 to 64 tokens, noise 0.1 to 1, with
 // and without the bias, at most 0.1 of them is not.  An expert that is not has been read for nothing: it
 // gets no tokens and no second projection.  The first projection of all others follows when the
@@ -103,7 +103,6 @@ struct RwPlan {
     int early, n_early;           // early start; its experts
     int one_rows;                 // second-projection tasks of that many slots take one k-tile per stage (0: none)
     int split16;         // where wave 1 begins, in 16ths of the first projection
-    int delta;           // second-projection units that weigh as much as one first-projection unit
     RwDiv gf, gs, tf, ts, kr, ks, rb, p;   // row groups and tasks of a routed / shared expert, P2 units of their row blocks, row blocks, CTAs
 };
 
@@ -157,8 +156,10 @@ inline RwPlan rw_make_plan(const Shape &sh, int B, int n_sm, bool early, int rou
     const int G = sh.E + sh.n_sh, n_slots = B * sh.k + sh.n_sh * B;
     p.early = early && n_sm > 1;
     // experts whose first projection starts before the gating (see the header comment)
-    // (one or two tokens select little more than top_k: some are left for a second wave)
-    p.n_early = p.early ? (sh.k < 4 ? (sh.k == 3 ? 2 : 1) : (B <= 2 ? (3 * sh.k + 2) / 4 : sh.k)) : 0;
+    // One or two tokens select little more than top_k, and wave 1 begins behind the early experts: a quarter is
+    // left for it.  Measured, us per layer, three quarters / all of top_k: OLMoE shape (top 8) 1 token 30.4 / 32.9,
+    // 2 tokens 35.3 / 37.1, 128 narrow experts (top 8) 1 token 30.4 / 29.6, Qwen1.5-MoE shape (top 4) 35.7 / 34.9.
+    p.n_early = p.early ? (B <= 2 ? (3 * sh.k + 2) / 4 : sh.k) : 0;
     p.n1 = (B + 15) & ~15;
     const int trows = rw_tok_rows(B);
     // Tasks of the second projection whose token tiles would make every stage larger (32 slots where the batch
@@ -184,15 +185,15 @@ inline RwPlan rw_make_plan(const Shape &sh, int B, int n_sm, bool early, int rou
     p.ks = rw_div_make(sh.n_sh ? (sh.f_sh + 127) / 128 : 1);
     p.rb = rw_div_make((sh.d + 127) / 128);
     // tasks of a CTA at most: a share of n units in groups of g, m units per task, meets n / g + 2 groups,
-    // and every group adds at most one ragged task to n / m whole ones (44: four per lot, and room for what
-    // `delta` moves from one CTA to another and for the tables' first pass)
+    // and every group adds at most one ragged task to n / m whole ones (44: four per lot, and room for
+    // the tables' first pass)
     const long long P = n_sm - 1 > 0 ? n_sm - 1 : 1, U = sh.E < (long long)B * sh.k + p.n_early ? sh.E : (long long)B * sh.k + p.n_early;
     const long long n1r = U * p.gf.d, n1s = sh.n_sh ? (long long)sh.n_sh * p.gs.d : 0;
     const long long n2r = U * p.rb.d * p.kr.d, n2s = sh.n_sh ? (long long)sh.n_sh * p.rb.d * p.ks.d : 0;
     const long long tasks = n1r / P / 8 + n1r / P / p.gf.d + n1s / P / 8 + n1s / P / p.gs.d + n2r / P / p.kr.d + n2s / P / p.ks.d +
                             44;
     // (unit numbers are 31-bit, those of the first projection also 8 times over; k-tiles are kept in 15 bits)
-    if (8 * (n1r + n1s) + 64 * P >= 1ll << 31 || n1r + n1s + n2r + n2s + 128 * P + 64 * P * (sh.d / 1024 + 1) >= 1ll << 31 ||
+    if (8 * (n1r + n1s) + 64 * P >= 1ll << 31 || n1r + n1s + n2r + n2s + 128 * P >= 1ll << 31 ||
         p.kr.d >= 1u << 14 || p.ks.d >= 1u << 14)
         return p;
     // (as many as there are: a table that leaves no room for two stages makes the plan infeasible)
@@ -237,7 +238,6 @@ inline RwPlan rw_make_plan(const Shape &sh, int B, int n_sm, bool early, int rou
     // 126.5 / 127.9, Qwen1.5-MoE shape 42.3 / 43.1, 128 narrow experts at 13 tokens 38.3 / 38.2, 128 wide ones
     // at 8 75.4 / 76.2.
     p.split16 = 8;
-    p.delta = (sh.d + 512) / 1024;
     return p;
 }
 
@@ -900,31 +900,17 @@ ffn_rows_kernel(const __grid_constant__ RwMaps maps, const __grid_constant__ RwA
                     const int w = lane < 2 ? 0 : min(lane - 1, kRwMaxWaves - 1);
                     int n = sx ? sh.n_sh * u2s : (real ? s_bound[w + 1] - s_bound[w] - (w == 0 ? n_bad : 0) : w < 2) * u2r;
                     if (lane >= kRwLots2) n = 0;
-                    // units dealt before this lot, and how many CTAs (0 .. R - 1) have one unit of the first
-                    // projection more than the others: they get that much less of the second one, in its last lot
-                    const int n1 = sh.n_sh * Gs + U * Gf, R = n1 - rw_div(n1, pl.p) * P;
+                    // units dealt before this lot (a CTA that got a unit more of the first projection gets its full share
+                    // of the second one all the same: taking d / 1024 units from it cost 0.9 % at 8 tokens of
+                    // the OLMoE shape and 2.5 % at 64 of the DeepSeek-V2-Lite shape)
                     int before = n;
 #pragma unroll
                     for (int o = 1; o < 8; o <<= 1) {
                         const int t = __shfl_up_sync(0xffffffffu, before, o);
                         if (lane >= o) before += t;
                     }
-                    before += n1 - n;
-                    const unsigned nz = __ballot_sync(0xffffffffu, n > 0);
                     int start, cnt;
-                    const int v = n + pl.delta * R, qv = rw_div(v, pl.p);
-                    if (lane == 31 - __clz(nz) && qv >= pl.delta) {
-                        const int r = v - qv * P, rot = before - rw_div(before, pl.p) * P;
-                        int c = cta - rot;
-                        if (c < 0) c += P;
-                        // CTAs before this one in the order that starts at rot, and those of them below R
-                        const int end = rot + c;
-                        const int ex = end <= P ? max(0, min(end, R) - min(rot, R)) : (R - min(rot, R)) + min(end - P, R);
-                        start = c * qv + min(c, r) - pl.delta * ex;
-                        cnt = qv + (c < r ? 1 : 0) - (cta < R ? pl.delta : 0);
-                    } else {
-                        share(n, before, start, cnt);
-                    }
+                    share(n, before - n + sh.n_sh * Gs + U * Gf, start, cnt);
                     const RwSeg sg = rw_seg(start, n > 0 ? cnt : 0, sx ? pl.ks : pl.kr, 24, 1);
                     int first = sg.n;
 #pragma unroll
