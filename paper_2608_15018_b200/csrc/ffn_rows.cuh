@@ -569,12 +569,13 @@ ffn_rows_kernel(const __grid_constant__ RwMaps maps, const __grid_constant__ RwA
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer
         if (tc_elect()) {
-            bool alive = true, x_there = pl.x_bytes == 0;
+            bool alive = true, x_there = pl.x_bytes == 0, x_copied = false;
             if (pl.x_bytes && (alive = inputs_wait())) {
                 // the hidden states' tiles, eight k-tiles per copy (past the end: zeros)
                 const uint32_t xb = smem_u32(&x_bar), xd = smem_u32(xres);
                 rw_expect(xb, (uint32_t)(((nk + 7) & ~7) * pl.xr * 128));
                 for (int kt = 0; kt < nk; kt += 8) rw_tma_3d(xd + (uint32_t)(kt * pl.xr * 128), &maps.m[10], 0, 0, kt, xb);
+                x_copied = true;
             }
             int s = 0, lim = lim0, level = 0;
             uint32_t par = 0, run = 0;
@@ -646,6 +647,8 @@ ffn_rows_kernel(const __grid_constant__ RwMaps maps, const __grid_constant__ RwA
                 tc_commit(&acc_full[buf]);
                 ++run;
             }
+            // (a CTA without tasks: the copies of the hidden states must have landed before it ends)
+            if (x_copied && !x_there && !mbar_wait(&x_bar, 0)) atomicExch(ws.status, ST_MBAR_TIMEOUT);
         }
     } else if (warp == 10) {
         // ------------------------------------------------------------------ early experts, first projection's tasks; then watcher

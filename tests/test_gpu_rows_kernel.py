@@ -92,3 +92,19 @@ def test_error_against_float64(cfg, B, bound):
     wl = CONFIGS[cfg].with_(n_experts=16, cap=2 * CONFIGS[cfg].top_k)
     rep, _ = run_case(wl, n_tokens=B, plan=3)
     assert rep.plan == 3 and rep.rms_rel_err <= bound
+
+
+def test_ctas_without_tasks():
+    """Narrow experts of a wide model: most CTAs get no task, copy the hidden states into shared memory all the same
+    and make room for the next layer's CTA."""
+    wl = CONFIGS["cfg2"].with_(d_model=2048, d_ff=32, n_experts=2, top_k=1, cap=2, n_layers=6, n_tokens=8)
+    W = [workloads.layer_weights(wl, l, "cuda") for l in range(6)]
+    H = torch.stack([workloads.hidden_states(wl, l, 8, device="cuda") for l in range(6)])
+    with binding.S2MoE(binding.Config.from_workload(wl, n_layers=6, kernel_plan=3), W) as m:
+        o = m.alloc_outputs(8, stack=True)
+        for _ in range(20):
+            m.verify_stack(H, None, o)
+        torch.cuda.synchronize()
+        assert m.device_status() == 0
+    for l in range(6):
+        check_outputs(wl, W[l], H[l], None, binding.LayerOutput(o.out[l], o.sel_idx[l], o.sel_w[l], o.n_unique[l:l + 1]))
