@@ -9,7 +9,7 @@ Metric: verified draft tokens/s per MoE layer = B / (step time / n_layers).
                   [--sigma S] [--plan P] [--impl reference] [--no-cpu-baseline] [--headline-only]
 
 The default run times the headline workload (cfg 2) and then, in the same JSON line under
-"per_workload", the other workloads of the benchmark spec (cfg 3; cfg 4 at 8 and 32 tokens; cfg 5 at
+"per_workload", the other workloads (cfg 3; cfg 4 at 8 and 32 tokens; cfg 5 at
 16 and 64 tokens), each with its unique-expert bandwidth as a fraction of 8 TB/s and of the
 measured copy bandwidth.  Every figure is the median of at least 15 repeats of a K-step graph
 replay, at least half a second of timed GPU work.
@@ -420,7 +420,7 @@ def run_own(args, wl, B, sigma):
     head = measure_stack(wl, B, sigma, L, args.plan, args.steps, args.warmup, dev, rank, world, peak, peak_kind, local)
     per = []
     if world == 1 and not args.headline_only and args.workload == "cfg2" and args.tokens is None and args.layers is None:
-        # every other workload of the benchmark spec in the same line (weights generated and freed one
+        # every other workload in the same line (weights generated and freed one
         # stack at a time); cfg 5 carries the fit of the cost model over a sweep of tree sizes
         for name, nb, sg, k in PER_WORKLOAD:
             w2 = workloads.CONFIGS[name]
@@ -459,7 +459,7 @@ def run_own(args, wl, B, sigma):
             "per_workload": per,
             "worst_workload": {"workload": worst["workload"], "n_tokens": worst["n_tokens"],
                                "frac_of_measured": worst["frac_of_measured"], "frac_of_8tbs": worst["frac_of_8tbs"]},
-            "target": "north star: >= 0.70 of ~8 TB/s on unique-expert bytes at 8 or more tokens; not met (see frac_of_8tbs)",
+            "target": ">= 0.70 of ~8 TB/s on unique-expert bytes at 8 or more tokens; not met (see frac_of_8tbs)",
         }
         if world == 1 and not args.no_cpu_baseline:
             line["cpu_baseline"] = cpu_baseline(wl, B, sigma, args.cpu_seconds, range(L))

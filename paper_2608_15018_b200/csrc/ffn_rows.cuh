@@ -45,8 +45,9 @@
 // in a thread chosen by elect.sync: measured on B200, an MMA of 128 x 16 x 16 then issues every 39 cycles
 // against 55 from a `lane == 0` branch (the tensor core itself needs 32 to read the 4 KiB of
 // weights), which is why one issuer is enough.
-// Measured, us per layer, split-K kernel before / this one: OLMoE shape 8 tokens 52 / 42, Qwen1.5-MoE
-// shape 16 tokens 54.6 / 42, DeepSeek-V2-Lite shape 16 tokens 60 / 52, 64 tokens 140 / 129.
+// Measured on one GPU, us per layer, split-K kernel / this one when it replaced it: OLMoE shape 1 token 41.1 / 35.5,
+// 8 tokens 50.9 / 46.7, Qwen1.5-MoE shape 16 tokens 54.9 / 46.7, DeepSeek-V2-Lite shape 16 tokens 59.5 / 54.5,
+// 64 tokens 131.5 / 130.5, 128 wide experts 8 tokens 89.7 / 75.4.
 // The tensor core truncates when it adds to an accumulator, so the k-tiles of a task go in turn to several
 // accumulators (chains) that the epilogue adds: eight in the first projection up to 16 tokens, four above, and as
 // many as their columns hold in the second one.  Relative 2-norm of the error against float64, two / four /
