@@ -30,9 +30,12 @@ def _write(how, kernel, dst, src):
 
 
 @pytest.mark.parametrize("how", ["copy", "early trigger"])
-@pytest.mark.parametrize("call", ["layer", "stack"])
+@pytest.mark.parametrize("call", ["layer", "stack", "graph"])
 @pytest.mark.parametrize("cfg,B", [("cfg3", 8), ("cfg3", 16), ("cfg5", 4), ("cfg5", 33)])
-def test_weights_written_just_before_the_call(cfg, B, call, how):
+@pytest.mark.parametrize("early", [True, False])
+def test_weights_written_just_before_the_call(cfg, B, early, call, how, monkeypatch):
+    if not early:
+        monkeypatch.setenv("S2MOE_NO_EARLY", "1")
     wl = CONFIGS[cfg].with_(d_model=512, d_ff=256, n_experts=16, cap=8, d_ff_shared=1024, n_layers=2)
     kernel = torch.cuda._compile_kernel(WRITER, "late_copy") if how != "copy" else None
     names = ("sh_gate", "sh_up", "sh_down", "w_gate", "w_up", "w_down", "router")
@@ -48,19 +51,28 @@ def test_weights_written_just_before_the_call(cfg, B, call, how):
             for l in range(2):
                 old[l]["sh_scale"].copy_(new[l]["sh_scale"])
         # the shared experts' weights last: the writer directly in front of the call
-        for name in reversed(names):
-            for l in (1, 0):
-                if call == "layer" and name.startswith("sh_") and l == 1:
-                    continue
-                _write(how, kernel, old[l][name], new[l][name])
-        if call == "stack":
+        def refresh():
+            for name in reversed(names):
+                for l in (1, 0):
+                    if call != "layer" or l == 0 or not name.startswith("sh_"):
+                        _write(how, kernel, old[l][name], new[l][name])
+
+        if call == "graph":
+            side = torch.cuda.Stream()
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph, stream=side):
+                refresh()
+                m.verify_stack(H, None, o, stream=side)
+            graph.replay()
+        elif call == "stack":
+            refresh()
             m.verify_stack(H, None, o)
         else:
-            for l in range(2):
-                if l == 1:
-                    for name in ("sh_down", "sh_up", "sh_gate"):
-                        _write(how, kernel, old[l][name], new[l][name])
-                m.verify_layer(l, H[l], None, views[l])
+            refresh()
+            m.verify_layer(0, H[0], None, views[0])
+            for name in ("sh_down", "sh_up", "sh_gate"):
+                _write(how, kernel, old[1][name], new[1][name])
+            m.verify_layer(1, H[1], None, views[1])
         torch.cuda.synchronize()
         assert m.device_status() == 0
     for l in range(2):
