@@ -423,10 +423,8 @@ def expert_masks(sel_idx: torch.Tensor, n_experts: int, out: Optional[torch.Tens
     if out is None:
         out = torch.zeros((n, 1, words), dtype=torch.int64, device=sel_idx.device)
     n_layers = out.shape[1]
-    if not 0 <= layer < n_layers:
-        raise ValueError(f"layer {layer} of {n_layers}")
-    if out.element_size() != 8 or out.numel() < n * n_layers * words:
-        raise ValueError(f"out: expected int64 [{n}][{n_layers}][{words}], got {out.dtype} {list(out.shape)}")
+    if not 0 <= layer < n_layers or out.nbytes < 8 * n * n_layers * words:      # (the C call gets addresses only)
+        raise ValueError(f"layer {layer} of out {list(out.shape)} {out.dtype}: int64 [{n}][n_layers][{words}] expected")
     rc = lib.s2moe_expert_masks(_dptr(sel_idx), n, k, n_experts, _dptr(out) + 8 * layer * words, n_layers * words, _stream_handle(stream))
     if rc != OK:
         raise S2MoEError(rc, "s2moe_expert_masks")
