@@ -13,41 +13,52 @@
 // per SM; of each of the four segments (phase 1 / 2 of wave 0 / 1) a CTA takes one contiguous run of
 // units, so that consecutive k-pieces of a row block are summed up in registers and reduced to memory once.
 //
-// What a unit passes through: TMA brings its packed rows and scales into a stage of the ring; the
-// dequantising warps turn it into binary16 values q * scale in tensor memory, the A operand of the MMAs,
+// What a unit passes through: TMA brings its packed rows and scales into a stage of the ring; a group of
+// dequantising warps turns it into binary16 values q * scale in tensor memory, the A operand of the MMAs,
 // whose accumulators stay there over a run of units.  The token tiles of a unit are fetched into a buffer
 // that belongs to the A operand's slot, so a stage is free as soon as it has been dequantised.
 //
 // What bounds it: instruction issue and latency.  At 6.5 TB/s an SM gets 42 weights per cycle; a weight
-// costs 13 / 8 thread instructions to dequantise and as much again for everything around it, and the
-// MMAs of a unit (N = 16: each covers 16 columns of 128 rows) are issued at 40 to 70 cycles each.  So what
-// the issuers and the producer execute per unit counts: they run in a thread chosen by elect.sync, a
-// unit's entry in shared memory is 16 bytes (44 before), what only some units need is a function of
-// its own (inlined everywhere it pushes the loops out of the instruction cache), two issuers instead of four.
-// Measured at the Mixtral shape, us per layer, before / now: 1 token 82 / 67, 8 tokens 147 / 122, 32 tokens
-// 183 / 138, 64 tokens 251 / 163 (the weights alone: 31 and 62 at the measured copy rate).
+// costs 13 / 8 thread instructions to dequantise and nearly as much again for everything around it.  The MMAs
+// themselves are cheap (A in tensor memory, N = 16: 22 cycles each from one thread, 16 a unit; N = 32: 26, N = 64: 37),
+// but every instruction of a single thread's role waits for its turn behind the busy warps of its scheduler.  So
+//   - the groups (three, each with a slot of its own, where the accumulators leave room for three, that is up to 32
+//     tokens; else two) take the units in turn: a unit is some 800 cycles of issue, then its group waits 700 to 750 for the
+//     issuer to notice, the MMAs and their completion, and the other groups work meanwhile.  With one group the schedulers
+//     idled that long in every unit, with two the groups fell into step and idled together;
+//   - weights and token tiles have a producer each: one thread for both needed 600 cycles per copy under that load, so
+//     weights arrived just as they were asked for although the ring has ten stages;
+//   - a unit's entry in shared memory holds what the roles need (16 bytes and the row of the map), and what only some
+//     units need is a function of its own (inlined everywhere it pushes the loops out of the instruction cache).
+// A slot, and a stage of the ring (whose length is a multiple of the groups), belong to one group, so that whoever waits for
+// their barriers sees every phase: a barrier tells only odd phases from even ones.
+// Measured at the Mixtral shape, us per layer, with one group and one producer / now: 1 token 66.8 / 59.2, 8 tokens
+// 119.8 / 96.5, 16 130.3 / 104.7, 32 136.9 / 120, 64 158.9 / 155.2 (the weights alone: 31 at 1 token, 62 at 8 at the
+// measured copy rate).
 //
 // Tried instead: the nibbles as binary16 subnormals n - 8 (9 instructions per 8 weights, exact), one
 // accumulator per block of 32 columns and the scales applied in fp32 behind the MMAs: eight accumulators a unit
-// instead of one a run have to be read back, 163 us at 8 tokens and 376 at 32.  16 dequantising warps:
-// 125 and 141.  The A operand's slots handed over in halves: 134 and 147.  Three such slots: 125 and 141.
+// instead of one a run have to be read back, 163 us at 8 tokens and 376 at 32 (147 and 183 for the kernel of the time).
+// Units ordered so that a set of token tiles serves eight row blocks: eight times the reductions at the ends of
+// runs, 128 at 8 tokens against 121.  Two issuers, unit by unit, with two groups: 111 and 133 at 8 and 32 tokens.
 //
 // Early start: the grid does not wait for the routing kernel as a whole.  The selected experts, known
 // before the mixing weights and the buckets, are enough for every unit but the epilogue's targets, so
 // the first projection streams while the gating ends.
 //
-// Warp roles (608 threads): 0 TMA producer; 1 and 6 MMA issuers (one where the accumulators leave no room for
-// two); 2..5 epilogue; 7..9 converters; 10 watcher (polls the waves' second counters and publishes them
-// in shared memory); 11..18 dequantising.  Warps 7..10 build the tables first.
+// Warp roles (Q4Plan::threads): 0 weight producer; 1 MMA issuer; 2..5 epilogue; 7..9 converters; 10 watcher (polls
+// the waves' second counters and publishes them in shared memory); 11 token producer; from 12 on dequantising.  Warps
+// 7..10 build the tables first.
 #pragma once
 
 #include "tc_common.cuh"
 
 namespace s2moe {
 
-constexpr int kQ4Threads = 608;
-constexpr int kQ4DeqWarps = 8;                 // 4 chunks of a row per thread
-constexpr int kQ4MaxUnits = 416;               // units of one CTA decoded once into shared memory
+constexpr int kQ4FirstDeq = 12;                // first dequantising warp (a multiple of 4)
+constexpr int kQ4MaxThreads = 32 * (kQ4FirstDeq + 16);
+constexpr int kQ4MaxGroups = 3;                // dequantising groups, unit by unit in turn
+constexpr int kQ4MaxUnits = 384;               // units of one CTA decoded once into shared memory
 constexpr int kQ4MaxWaves = 2, kQ4Segs = 2 * kQ4MaxWaves;
 
 struct Q4Plan {
@@ -58,7 +69,10 @@ struct Q4Plan {
     int tab_bytes;
     int smem_bytes;
     int tokb;          // bytes of the token tiles of one k-tile
-    int n_iss;         // MMA issuer warps (2 where the accumulators fit)
+    int groups;        // dequantising groups; each has a slot of the A operand, 128 columns at the end of tensor memory
+    int deq_warps;     // warps of a group: 4 (a row per thread) or 8 (half a row)
+    int threads;
+    int acc_cols;      // columns of an accumulator
     int early;         // the first projection starts when the selection is known
 };
 
@@ -82,39 +96,45 @@ inline Q4Plan q4_make_plan(const Shape &sh, int B, int n_sm, bool early)
     p.n1 = (B + 15) & ~15;
     p.tokb = 2048 * ((B + 7) / 8);             // phase 2: per 8 slots their hi and lo rows; phase 1: n1 rows
     p.tab_bytes = ((int)sizeof(TcGroup) * G + 8 * n_slots + 1023) & ~1023;
-    // Tensor memory: columns 256..511 hold two slots of a whole unit (4 k-tiles x 32 columns of binary16 pairs),
-    // columns 0..255 the accumulators: 2 buffers x issuers x 2 * n1 columns.  Measured at the Mixtral shape,
-    // us per layer with 1 / 2 / 4 issuers: 8 tokens 148.7 / 126.0 / 134.0, 1 token 80.5 / 69.0 / 72.8, 32 tokens
-    // 161 / 140 (four do not fit).
-    p.n_iss = 8 * p.n1 <= kTcQ4ACol ? 2 : 1;
+    // Tensor memory: two accumulators of 64 columns (of 128 above 32 tokens) and the slots of the A operand.  Where two of a
+    // unit's N columns fit an accumulator its K-steps go to two chains in turn: the tensor core truncates when it adds.
+    // Three groups of four warps up to 32 tokens, two of eight above (three slots do not fit).  Measured, us per layer at the
+    // Mixtral shape, three / two: 8 tokens 96 / 111, 16 tokens 105 / 120, 32 tokens 117 / 133; four-warp groups with a
+    // row's eight chunks loaded together 99 / - at 8, and two of them 172 against 164 at 64.
+    p.acc_cols = B <= 32 ? 64 : 128;
+    p.groups = (512 - 2 * p.acc_cols) / 128;
+    p.deq_warps = p.groups == 3 ? 4 : 8;
+    p.threads = 32 * (kQ4FirstDeq + p.groups * p.deq_warps);
     // The token tiles lie beside the ring, one set per slot of the A operand: a stage is free as soon as its
     // weights and scales have been read, and not only when the MMAs have completed.
-    p.stages = (kTcMaxSmem - p.tab_bytes - 1024 - 2 * kTcQ4KG * p.tokb) / kQ4StageBytes;
+    p.stages = (kTcMaxSmem - p.tab_bytes - 1024 - p.groups * kTcQ4KG * p.tokb) / kQ4StageBytes;
     if (p.stages > kTcMaxStages) p.stages = kTcMaxStages;
-    p.smem_bytes = p.tab_bytes + p.stages * kQ4StageBytes + 2 * kTcQ4KG * p.tokb + 1024;
+    p.stages -= p.stages % p.groups;           // (a stage is always the same group's)
+    p.smem_bytes = p.tab_bytes + p.stages * kQ4StageBytes + p.groups * kTcQ4KG * p.tokb + 1024;
     // (the SM that runs the gating is taken until the routing kernel ends: its CTA would start last with a
     // full share)
     p.early = early && n_sm > 1 ? 1 : 0;
     p.n_cta = n_sm - p.early;
-    // (three stages at the limits: 60 and more tokens of 14 and more of 256 experts beside 4 shared ones; never less)
-    p.feasible = p.stages >= 3 && B <= kMaxTokens && sh.weight_dtype == DT_Q4B32 && sh.act_dtype == DT_BF16 && sh.d % 256 == 0 &&
+    // (two stages at the limits: 60 and more tokens of 14 and more of 256 experts beside 4 shared ones; never less)
+    p.feasible = p.stages >= p.groups && B <= kMaxTokens && sh.weight_dtype == DT_Q4B32 && sh.act_dtype == DT_BF16 && sh.d % 256 == 0 &&
                  sh.f % 256 == 0 && (sh.n_sh == 0 || sh.f_sh % 256 == 0);
     return p;
 }
 
 // What a unit needs, in one 16-byte entry: meta = first | last << 1 | (phase 2) << 2 | N << 8 (N of a phase-2
-// unit is filled in with the buckets), group entry | matrix << 16 | segment << 20, row block, first k-tile
+// unit is filled in with the buckets), group entry | map << 16 | segment << 20, first row of the matrix, first k-tile;
+// beside it the first row of the map
 struct Q4Segments {
     int start[kQ4Segs], cnt[kQ4Segs];  // this CTA's run of units of every segment
     int total1, U;                     // units of the first projection, routed experts
 };
 // unit i of this CTA (out of line: it runs once per unit while the tables are built, and only for units
 // past the table afterwards; inlined at every use it pushes the roles' loops out of the instruction cache)
-__device__ __noinline__ uint4 q4_unit_make(const Q4Segments &sg, const TcGroup *groups, const Shape &sh, int n1, int i)
+__device__ __noinline__ uint4 q4_unit_make(const Q4Segments &sg, const TcGroup *groups, const Shape &sh, const Q4Plan &pl, int i)
 {
     int seg = 0, j = i;
     while (seg < kQ4Segs - 1 && j >= sg.cnt[seg]) { j -= sg.cnt[seg]; ++seg; }
-    const int total1 = sg.total1, U = sg.U, u = sg.start[seg] + j, last = sg.cnt[seg] - 1;
+    const int total1 = sg.total1, U = sg.U, u = sg.start[seg] + j, left = sg.cnt[seg] - 1 - j;
     const int kp1 = sh.d >> 8, rb2 = sh.d >> 7;
     int a, mat, rb, piece, kp;
     if (u < total1) {
@@ -137,23 +157,29 @@ __device__ __noinline__ uint4 q4_unit_make(const Q4Segments &sg, const TcGroup *
         piece = local - rb * kp;
         mat = 2;
     }
-    const uint32_t first = j == 0 || piece == 0, end = j == last || piece == kp - 1;
     // (N of a phase-2 unit: 0 before the buckets are known)
-    const uint32_t n = mat < 2 ? (uint32_t)n1 : 16u * (((uint32_t)groups[a].T + 7u) >> 3);
-    return make_uint4(first | (end << 1) | (mat == 2 ? 4u : 0u) | (n << 8), (uint32_t)a | ((uint32_t)mat << 16) | ((uint32_t)seg << 20),
-                      (uint32_t)rb, (uint32_t)(4 * piece));
+    const uint32_t n = mat < 2 ? (uint32_t)pl.n1 : 16u * (((uint32_t)groups[a].T + 7u) >> 3);
+    // Where up to 32 tokens leave no room for a second chain (17 and more slots) a run ends after 12 pieces, so that no sum has
+    // more terms than with two chains over a whole share (error against float64 at 32 tokens, Mixtral shape:
+    // one chain 3.1496e-4, cut 3.1478e-4, two chains 3.1482e-4).
+    const bool cut = mat == 2 && pl.acc_cols == 64 && 2u * n > 64u;
+    const uint32_t flags = (j == 0 || piece == 0 || (cut && piece % 12 == 0) ? 1u : 0u) |
+                           (left == 0 || piece == kp - 1 || (cut && piece % 12 == 11) ? 2u : 0u) | (mat == 2 ? 4u : 0u);
+    return make_uint4(flags | (n << 8), (uint32_t)a | ((uint32_t)(a >= U ? mat + 3 : mat) << 16) | ((uint32_t)seg << 20),
+                      (uint32_t)rb * 128u, (uint32_t)(4 * piece));
 }
 
-__global__ void __launch_bounds__(kQ4Threads, 1)
+__global__ void __launch_bounds__(kQ4MaxThreads, 1)
 ffn_q4_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ Q4Args p)
 {
     extern __shared__ __align__(1024) uint8_t q4_smem[];
-    __shared__ __align__(8) uint64_t full_bar[kTcMaxStages], empty_bar[kTcMaxStages], a_full[2], a_empty[2];
+    __shared__ __align__(8) uint64_t full_bar[kTcMaxStages], empty_bar[kTcMaxStages], a_full[kQ4MaxGroups], a_empty[kQ4MaxGroups];
     __shared__ __align__(8) uint64_t acc_full[2], acc_empty[2], conv_go[kQ4MaxWaves], tab_bar[2], cv_bar;
     __shared__ uint32_t s_tmem;
     __shared__ int s_flag, s_n_units, s_split, s_n_active;
     __shared__ Q4Segments s_seg;
     __shared__ uint4 s_units[kQ4MaxUnits];
+    __shared__ int s_row[kQ4MaxUnits];
     __shared__ uint16_t s_id[kMaxExperts];
     __shared__ volatile int s_ready[kQ4MaxWaves];  // wave w's activations are written (set by the watcher warp)
 
@@ -161,7 +187,8 @@ ffn_q4_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ Q4Arg
     const Workspace &ws = p.ws;
     const Q4Plan &pl = p.plan;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int S = pl.stages, P = (int)gridDim.x, NI = pl.n_iss;
+    const int S = pl.stages, P = (int)gridDim.x, NG = pl.groups, ACC = pl.acc_cols;
+    const uint32_t a_col = 512u - 128u * (uint32_t)NG;      // first column of the A operand's slots
     const bool EARLY = pl.early != 0;
     const int n_routed = p.B * sh.k, n_slots = n_routed + sh.n_sh * p.B;
     const int kp1 = sh.d >> 8, rb2 = sh.d >> 7;
@@ -178,15 +205,17 @@ ffn_q4_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ Q4Arg
     if (warp == 2) {
         if (lane < S) {
             mbar_init(&full_bar[lane], 1);
-            mbar_init(&empty_bar[lane], kQ4DeqWarps);
+            mbar_init(&empty_bar[lane], pl.deq_warps);
         }
         if (lane < 2) {
-            mbar_init(&acc_full[lane], NI);
+            mbar_init(&acc_full[lane], 1);
             mbar_init(&acc_empty[lane], 4);
-            mbar_init(&a_full[lane], kQ4DeqWarps + 1);             // the dequantising warps and the producer's arrival with the token bytes
-            mbar_init(&a_empty[lane], NI);
-            mbar_init(&tab_bar[lane], 1);
         }
+        if (lane < kQ4MaxGroups) {
+            mbar_init(&a_full[lane], pl.deq_warps + 1);             // the dequantising warps and the token producer's arrival with the token bytes
+            mbar_init(&a_empty[lane], 1);
+        }
+        if (lane < 2) mbar_init(&tab_bar[lane], 1);
         if (lane < kQ4MaxWaves) {
             mbar_init(&conv_go[lane], 4);
             s_ready[lane] = 0;
@@ -202,8 +231,13 @@ ffn_q4_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ Q4Arg
     tc_fence_after();
     const uint32_t tmem_base = s_tmem;
 
-    auto unit_at = [&](int i) -> uint4 { return i < kQ4MaxUnits ? s_units[i] : q4_unit_make(s_seg, groups, sh, pl.n1, i); };
-    auto umeta_at = [&](int i) -> uint32_t { return i < kQ4MaxUnits ? s_units[i].x : q4_unit_make(s_seg, groups, sh, pl.n1, i).x; };
+    auto unit_at = [&](int i) -> uint4 { return i < kQ4MaxUnits ? s_units[i] : q4_unit_make(s_seg, groups, sh, pl, i); };
+    auto umeta_at = [&](int i) -> uint32_t { return i < kQ4MaxUnits ? s_units[i].x : q4_unit_make(s_seg, groups, sh, pl, i).x; };
+    auto map_row = [&](const uint4 &un) -> int {
+        const TcGroup &g = groups[un.y & 0xffffu];
+        const int mi = (int)(un.y >> 16) & 15;
+        return (mi >= 3 ? g.group - sh.E : g.group) * (mi == 2 || mi == 5 ? sh.d : g.f) + (int)un.z;
+    };
     // level 0: every unit; level 1: tokens and slots of the routed experts (and everything the routing
     // kernel clears is clear)
     auto tab_wait = [&](int level) -> bool {
@@ -305,7 +339,11 @@ ffn_q4_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ Q4Arg
             s_n_active = n_active;
         }
         asm volatile("bar.sync 1, 128;" ::: "memory");
-        for (int i = tt; i < n_units && i < kQ4MaxUnits; i += 128) s_units[i] = q4_unit_make(s_seg, groups, sh, pl.n1, i);
+        for (int i = tt; i < n_units && i < kQ4MaxUnits; i += 128) {
+            const uint4 un = q4_unit_make(s_seg, groups, sh, pl, i);
+            s_units[i] = un;
+            s_row[i] = map_row(un);
+        }
         asm volatile("bar.sync 1, 128;" ::: "memory");
         if (tt == 0) mbar_arrive(&tab_bar[0]);                     // (release: the tables are written)
         // The next kernel in the stream may come up once this CTA has read the words of the early start: the next
@@ -327,152 +365,134 @@ ffn_q4_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ Q4Arg
         asm volatile("bar.sync 1, 128;" ::: "memory");
         const int n_p1 = s_seg.cnt[0] + s_seg.cnt[1];
         for (int i = n_p1 + tt; i < n_units && i < kQ4MaxUnits; i += 128)
-            s_units[i].x = (s_units[i].x & 0xffu) | ((16u * (((uint32_t)groups[s_units[i].y & 0xffffu].T + 7u) >> 3)) << 8);
+            s_units[i].x = q4_unit_make(s_seg, groups, sh, pl, i).x;
         asm volatile("bar.sync 1, 128;" ::: "memory");
         if (tt == 0) mbar_arrive(&tab_bar[1]);
     }
 
     if (warp == 0) {
-        // ------------------------------------------------------------------ TMA producer
-        // Two cursors over the same sequence of units.  The packed tiles and scales go into the stage ring (a
-        // slot is free once the dequantising warps have read it); the token tiles go into the
-        // set of the A operand's slot they are used with (free once the MMAs that read it have completed; their
-        // bytes are counted by the barrier the dequantising warps arrive on, so that an MMA issuer waits
-        // once), and in the second projection only when their wave's activations are written.  One thread
-        // serves both, so it polls.
+        // ------------------------------------------------------------------ weight producer
+        // packed k-tiles (128 bytes of every row) and the 8 scales per row of these 256 columns into the ring
         if (tc_elect() && tab_wait(0)) {
             const uint64_t wpolicy = l2_evict_first_policy();
+            const int n_units = s_n_units;
+            int s = 0;
+            uint32_t ring_par = 1;
+            for (int i = 0; i < n_units; ++i) {
+                uint4 un;
+                int row;
+                if (i < kQ4MaxUnits) {
+                    un = s_units[i];
+                    row = s_row[i];
+                } else {
+                    un = q4_unit_make(s_seg, groups, sh, pl, i);
+                    row = map_row(un);
+                }
+                const CUtensorMap *map = &maps.m[(un.y >> 16) & 15u];
+                uint8_t *stage = ring + (size_t)s * kQ4StageBytes;
+                if (!mbar_wait(&empty_bar[s], ring_par)) { atomicExch(ws.status, ST_MBAR_TIMEOUT); break; }
+                mbar_expect_tx(&full_bar[s], kQ4StageBytes);
+                tma_load_2d_stream(stage, map, (int)un.w * 32, row, &full_bar[s], wpolicy);
+                tma_load_2d(stage + kTcQ4KG * kTcQ4Packed, map + 9, (int)un.w * 2, row, &full_bar[s]);
+                tc_ring_next(s, ring_par, S);
+            }
+        }
+    } else if (warp == 11) {
+        // ------------------------------------------------------------------ token producer
+        // The token tiles go into the set of the A operand's slot they are used with (free once the MMAs that read
+        // it have completed; their bytes are counted by the barrier the dequantising warps arrive on, so that an MMA
+        // issuer waits once), in the second projection only when their wave's activations are written.
+        if (tc_elect() && tab_wait(0)) {
             const int n_units = s_n_units, split = s_split;
-            int pi = 0, ti = 0;                          // unit of each cursor
-            int s = 0, ta = 0;
-            uint32_t ring_par = 1, t_par = 1;
-            int ready_w = 0;
-            unsigned idle = 0;
-            bool alive = true;
+            int ta = 0, ready_w = 0;
+            uint32_t t_par = 1;
             // (the permuted hidden states are written by the routing kernel with generic stores)
             asm volatile("fence.proxy.async.global;" ::: "memory");
-            while (alive && (pi < n_units || ti < n_units)) {
-                bool progress = false;
-                if (pi < n_units && mbar_test(&empty_bar[s], ring_par)) {
-                    const uint4 un = unit_at(pi);
-                    const TcGroup &g = groups[un.y & 0xffffu];
-                    const int mat = (int)(un.y >> 16) & 15;
-                    const bool shared = g.group >= sh.E;
-                    const int row0 = (shared ? g.group - sh.E : g.group) * (mat == 2 ? sh.d : g.f) + (int)un.z * 128;
-                    const int mi = (shared ? 3 : 0) + mat;
-                    // packed k-tiles (128 bytes of every row) and the 8 scales per row of these 256 columns
-                    uint8_t *stage = ring + (size_t)s * kQ4StageBytes;
-                    mbar_expect_tx(&full_bar[s], kQ4StageBytes);
-                    tma_load_2d_stream(stage, &maps.m[mi], (int)un.w * 32, row0, &full_bar[s], wpolicy);
-                    tma_load_2d(stage + kTcQ4KG * kTcQ4Packed, &maps.m[9 + mi], (int)un.w * 2, row0, &full_bar[s]);
-                    tc_ring_next(s, ring_par, S);
-                    ++pi;
-                    progress = true;
-                }
-                if (ti < n_units) {
-                    uint4 un = unit_at(ti);
-                    const bool p2 = (un.x & 4u) != 0;
+            for (int i = 0; i < n_units; ++i) {
+                uint4 un = unit_at(i);
+                const bool p2 = (un.x & 4u) != 0;
+                if (p2) {
                     const int wv = (int)(un.y & 0xffffu) >= split ? 1 : 0;
-                    bool ready = !p2 || wv < ready_w;
-                    if (!ready && s_ready[wv]) {
+                    if (wv >= ready_w) {
+                        bool ok = false;
+                        for (unsigned t = 0; t < kTcSpinLimit && !ok; ++t) {
+                            ok = s_ready[wv] != 0;
+                            if (!ok) __nanosleep(100);
+                        }
                         // the activations of this wave are written: order them before the copies below
                         __threadfence_block();
                         asm volatile("fence.proxy.async.global;" ::: "memory");
-                        if (!tab_wait(1)) break;
-                        un = unit_at(ti);
+                        if (!ok || !tab_wait(1)) { atomicExch(ws.status, ST_MBAR_TIMEOUT); break; }
+                        un = unit_at(i);
                         ready_w = wv + 1;
-                        ready = true;
-                    }
-                    if (ready && mbar_test(&a_empty[ta], t_par)) {
-                        uint8_t *op = tokring + (size_t)ta * kTcQ4KG * pl.tokb;
-                        if (!p2) {
-                            // the hidden-state tiles of all four k-tiles in one copy: [k-tile][tokb / 128 rows]
-                            mbar_expect_tx(&a_full[ta], (uint32_t)(kTcQ4KG * pl.tokb));
-                            tma_load_3d(op, &maps.m[6], 0, 0, (int)un.w, &a_full[ta]);
-                        } else {
-                            // one copy per 8 slots for all four k-tiles: [hi | lo][k-tile][8 rows]
-                            const TcGroup &g = groups[un.y & 0xffffu];
-                            const bool shared = g.group >= sh.E;
-                            const int srow = shared ? g.off - n_routed : g.off, n = (int)(un.x >> 8);
-                            mbar_expect_tx(&a_full[ta], (uint32_t)(kTcQ4KG * n * 128));
-                            for (int r = 0; r < n / 2; r += 8)
-                                tma_load_4d(op + r * 256 * kTcQ4KG, &maps.m[shared ? 8 : 7], 0, srow + r, (int)un.w, 0, &a_full[ta]);
-                        }
-                        tc_ring_next(ta, t_par, 2);
-                        ++ti;
-                        progress = true;
                     }
                 }
-                if (progress) {
-                    idle = 0;
+                uint8_t *op = tokring + (size_t)ta * kTcQ4KG * pl.tokb;
+                if (!mbar_wait(&a_empty[ta], t_par)) { atomicExch(ws.status, ST_MBAR_TIMEOUT); break; }
+                if (!p2) {
+                    // the hidden-state tiles of all four k-tiles in one copy: [k-tile][tokb / 128 rows]
+                    mbar_expect_tx(&a_full[ta], (uint32_t)(kTcQ4KG * pl.tokb));
+                    tma_load_3d(op, &maps.m[6], 0, 0, (int)un.w, &a_full[ta]);
                 } else {
-                    // nothing to issue: leave the scheduler to the dequantising warps for a while
-                    __nanosleep(100);
-                    if (++idle > kTcSpinLimit) {
-                        atomicExch(ws.status, ST_MBAR_TIMEOUT);
-                        alive = false;
-                    }
+                    // one copy per 8 slots for all four k-tiles: [hi | lo][k-tile][8 rows]
+                    const TcGroup &g = groups[un.y & 0xffffu];
+                    const bool shared = g.group >= sh.E;
+                    const int srow = shared ? g.off - n_routed : g.off, n = (int)(un.x >> 8);
+                    mbar_expect_tx(&a_full[ta], (uint32_t)(kTcQ4KG * n * 128));
+                    for (int r = 0; r < n / 2; r += 8)
+                        tma_load_4d(op + r * 256 * kTcQ4KG, &maps.m[shared ? 8 : 7], 0, srow + r, (int)un.w, 0, &a_full[ta]);
                 }
+                tc_ring_next(ta, t_par, NG);
             }
         }
-    } else if (warp == 1 || warp == 6) {
-        // ------------------------------------------------------------------ MMA issuers
-        // With N = 16 every MMA covers only 4 KiB of bf16-sized weights, so two warps share the work: issuer h
-        // takes K-steps 2h and 2h + 1 of every k-tile; each accumulates into its own columns of tensor memory
-        // and the epilogue adds the partial accumulators.
-        const int half = warp == 1 ? 0 : 1;
-        if (half < NI && tc_elect() && tab_wait(0)) {
+    } else if (warp == 1) {
+        // ------------------------------------------------------------------ MMA issuer
+        if (tc_elect() && tab_wait(0)) {
             const int n_units = s_n_units;
-            const uint32_t ks = 4u / (uint32_t)NI, koff = 2u * ks * (uint32_t)half;
             const uint32_t hi1 = (uint32_t)(tc_smem_desc(tokring) >> 32), hi2 = (uint32_t)(tc_smem_desc_sbo(tokring, (uint32_t)kTcQ4KG * 1024u) >> 32);
-            const uint32_t tok_lo = (uint32_t)tc_smem_desc(tokring) + koff;
-            const uint32_t a_tmem0 = tmem_base + (uint32_t)kTcQ4ACol + 4u * koff;     // 8 columns per K-step
+            const uint32_t tok_lo = (uint32_t)tc_smem_desc(tokring), a_tmem0 = tmem_base + a_col;
             const uint32_t tok_slot = (uint32_t)kTcQ4KG * ((uint32_t)pl.tokb >> 4), step1 = (uint32_t)pl.tokb >> 4;
-            // (an instruction between two MMAs costs as much as the MMA: the K-steps are straight-line code for either
-            // number of issuers, and a unit's entry is read before the wait for the unit in front of it)
-            auto issue = [&](auto steps) {
-                constexpr uint32_t KS = decltype(steps)::value;
-                uint32_t d_tmem = tmem_base + (uint32_t)(half * 2 * pl.n1), buf = 0, run_par = 1, a_par = 0;
-                uint32_t ta = 0, um = n_units > 0 ? umeta_at(0) : 0u;
-                bool tabs = false;
-                for (int ui = 0; ui < n_units; ++ui) {
-                    if ((um & 4u) && !tabs) {
-                        tabs = true;
-                        if (!tab_wait(1)) break;
-                        um = umeta_at(ui);
-                    }
-                    const bool p2 = (um & 4u) != 0, first = (um & 1u) != 0, last = (um & 2u) != 0;
-                    // slot ta's k-tiles (32 columns each) and their token tiles: phase 1 [k-tile][rows], phase 2
-                    // [8 slots][hi | lo][k-tile][8 rows] (8-row groups 4 KiB apart)
-                    const uint32_t idesc = tc_idesc_f16((int)(um >> 8));
-                    const uint32_t a_tm = a_tmem0 + ta * (kTcQ4KG * 32u), b_lo = tok_lo + ta * tok_slot;
-                    const uint32_t b_step = p2 ? 64u : step1, b_hi = p2 ? hi2 : hi1;
-                    if (first && !mbar_wait(&acc_empty[buf], run_par)) { atomicExch(ws.status, ST_MBAR_TIMEOUT); break; }
-                    if (ui + 1 < n_units) um = umeta_at(ui + 1);
-                    // the unit in tensor memory, written by the dequantising warps, and its token tiles
-                    if (!mbar_wait(&a_full[ta], a_par)) { atomicExch(ws.status, ST_MBAR_TIMEOUT); break; }
-                    tc_fence_after();
-#pragma unroll
-                    for (uint32_t g = 0; g < kTcQ4KG; ++g)
-#pragma unroll
-                        for (uint32_t k = 0; k < KS; ++k)
-                            tc_mma_bf16_tmem_a(d_tmem, a_tm + 32u * g + 8u * k, b_lo + g * b_step + 2u * k, b_hi, idesc, g + k > 0 || !first ? 1u : 0u);
-                    tc_commit(&a_empty[ta]);           // frees the A operand and the token tiles
-                    ta ^= 1u;
-                    if (ta == 0) a_par ^= 1u;
-                    if (last) {
-                        tc_commit(&acc_full[buf]);
-                        buf ^= 1u;
-                        if (buf == 0) run_par ^= 1u;
-                        d_tmem = tmem_base + (uint32_t)(buf * 2 * NI * pl.n1 + half * 2 * pl.n1);
-                    }
+            uint32_t buf = 0, run_par = 1, a_par = 0, um = n_units > 0 ? umeta_at(0) : 0u;
+            int ta = 0;
+            bool tabs = false;
+            // (an instruction between two MMAs costs as much as the MMA: the K-steps are straight-line code, and a
+            // unit's entry is read before the wait for the unit in front of it)
+            for (int ui = 0; ui < n_units; ++ui) {
+                if ((um & 4u) && !tabs) {
+                    tabs = true;
+                    if (!tab_wait(1)) break;
+                    um = umeta_at(ui);
                 }
-            };
-            if (NI == 2) issue(std::integral_constant<uint32_t, 2>{});
-            else issue(std::integral_constant<uint32_t, 4>{});
+                const uint32_t m = um;
+                const bool p2 = (m & 4u) != 0, first = (m & 1u) != 0;
+                // slot ta's k-tiles (32 columns each) and their token tiles: phase 1 [k-tile][rows], phase 2
+                // [8 slots][hi | lo][k-tile][8 rows] (8-row groups 4 KiB apart)
+                const uint32_t N = m >> 8, idesc = tc_idesc_f16((int)N), d_tmem = tmem_base + buf * (uint32_t)ACC;
+                const uint32_t odd = 2u * N <= (uint32_t)ACC ? N : 0u;     // where the odd K-steps add up
+                const uint32_t a_tm = a_tmem0 + (uint32_t)ta * (kTcQ4KG * 32u), b_lo = tok_lo + (uint32_t)ta * tok_slot;
+                const uint32_t b_step = p2 ? 64u : step1, b_hi = p2 ? hi2 : hi1;
+                if (first && !mbar_wait(&acc_empty[buf], run_par)) { atomicExch(ws.status, ST_MBAR_TIMEOUT); break; }
+                if (ui + 1 < n_units) um = umeta_at(ui + 1);
+                // the unit in tensor memory, written by the dequantising warps, and its token tiles
+                if (!mbar_wait(&a_full[ta], a_par)) { atomicExch(ws.status, ST_MBAR_TIMEOUT); break; }
+                tc_fence_after();
+#pragma unroll
+                for (uint32_t g = 0; g < kTcQ4KG; ++g)
+#pragma unroll
+                    for (uint32_t k = 0; k < 4; ++k)
+                        tc_mma_bf16_tmem_a(d_tmem + (k & 1u ? odd : 0u), a_tm + 32u * g + 8u * k, b_lo + g * b_step + 2u * k, b_hi, idesc,
+                                           g > 0 || k > 1 || (k == 1 && odd == 0u) || !first ? 1u : 0u);
+                tc_commit(&a_empty[ta]);               // frees the A operand and the token tiles
+                if (m & 2u) {
+                    tc_commit(&acc_full[buf]);
+                    buf ^= 1u;
+                    if (buf == 0) run_par ^= 1u;
+                }
+                tc_ring_next(ta, a_par, NG);
+            }
         }
         __syncwarp();
-    } else if (warp >= 11 && warp < 11 + kQ4DeqWarps) {
+    } else if (warp >= kQ4FirstDeq) {
         // ------------------------------------------------------------------ dequantising warps
         // Every row of a packed k-tile (64 nibbles, stored q + 8) becomes 64 binary16 values q * scale (row =
         // lane, two values per 32-bit column): per 32-bit word eight nibbles -> 1024 + n or 1024 + 16 n as
@@ -480,73 +500,81 @@ ffn_q4_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ Q4Arg
         // so the product is the only rounding: 2^-12 relative).
         // A stage holds 256 columns: per row eight chunks of 16 packed bytes (32 weights, one scale each).  A warp
         // reaches the 32 lanes of its quarter (warp index mod 4) only, so thread (r, h) takes row
-        // r = 32 * (warp mod 4) + lane and chunks 4 h .. 4 h + 3, h = 0 for the first four warps, 1 for the others.
-        const int r = 32 * (warp & 3) + lane, h = (warp - 11) >> 2;
-        int s = 0, ta = 0;
+        // r = 32 * (warp mod 4) + lane and, in a group of four warps, all its chunks, in a group of eight chunks 4 h ..
+        // 4 h + 3, h = 0 for the first four warps, 1 for the others.
+        // While a group waits for the MMAs of its unit before, the others have the schedulers: groups that take
+        // their units in step (two of them, measured) leave them idle for a third of the time.
+        const int r = 32 * (warp & 3) + lane, dw = warp - kQ4FirstDeq, grp = dw / pl.deq_warps;
+        const int h0 = (dw - grp * pl.deq_warps) >> 2, h1 = pl.deq_warps == 4 ? 2 : h0 + 1;
+        int s = grp;
         uint32_t ring_par = 0, a_par = 1;
-        const uint32_t a_lane = tmem_base + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)kTcQ4ACol;
+        const uint32_t a_slot = tmem_base + ((uint32_t)(32 * (warp & 3)) << 16) + a_col + (uint32_t)grp * 128u;
         const __half2 minus1032 = __floats2half2_rn(-1032.0f, -1032.0f), sixteenth = __floats2half2_rn(0.0625f, 0.0625f),
                       minus72 = __floats2half2_rn(-72.0f, -72.0f);
         const int n_units = tab_wait(0) ? s_n_units : 0;
-        for (int ui = 0; ui < n_units; ++ui, tc_ring_next(s, ring_par, S), tc_ring_next(ta, a_par, 2)) {
+        for (int ui = grp; ui < n_units; ui += NG) {
             const bool ok_full = mbar_wait(&full_bar[s], ring_par);
-            if (!ok_full || !mbar_wait(&a_empty[ta], a_par)) { if (lane == 0) atomicExch(ws.status, ST_MBAR_TIMEOUT); break; }
+            if (!ok_full || !mbar_wait(&a_empty[grp], a_par)) { if (lane == 0) atomicExch(ws.status, ST_MBAR_TIMEOUT); break; }
             tc_fence_after();                                      // the MMAs that read this slot have completed
             const uint8_t *stage = ring + (size_t)s * kQ4StageBytes, *prow = stage + (size_t)r * 128;
-            const uint2 sc2w = *reinterpret_cast<const uint2 *>(stage + kTcQ4KG * kTcQ4Packed + r * 16 + h * 8);   // this thread's four scales
-            const uint32_t sc[2] = {sc2w.x, sc2w.y};
-            const uint32_t a_slot = a_lane + (uint32_t)ta * 128u;
-            // all packed chunks of this thread first: the stores to tensor memory below order
-            // memory accesses, so a load behind one of them would wait for it
-            uint4 pks[4];
+#pragma unroll 1
+            for (int h = h0; h < h1; ++h) {
+                const uint2 sc2w = *reinterpret_cast<const uint2 *>(stage + kTcQ4KG * kTcQ4Packed + r * 16 + h * 8);   // four scales
+                const uint32_t sc[2] = {sc2w.x, sc2w.y};
+                // all packed chunks first: the stores to tensor memory below order
+                // memory accesses, so a load behind one of them would wait for it
+                uint4 pks[4];
 #pragma unroll
-            for (int qi = 0; qi < 4; ++qi) {
-                // (the packed rows are swizzled over their 128 bytes by the TMA copy)
-                pks[qi] = *reinterpret_cast<const uint4 *>(prow + (((h * 4 + qi) ^ (r & 7)) * 16));
-            }
-#pragma unroll
-            for (int qi = 0; qi < 4; ++qi) {
-                const int q = h * 4 + qi;                         // chunk of 32 weights inside the stage
-                const uint4 pk = pks[qi];
-                // the block's scale is binary16 already: both halves of a register
-                const uint32_t sc2u = __byte_perm(sc[qi >> 1], 0u, (qi & 1) ? 0x3232u : 0x1010u);
-                const __half2 sc2 = *reinterpret_cast<const __half2 *>(&sc2u);
-                const uint32_t w[4] = {pk.x, pk.y, pk.z, pk.w};
-                uint32_t o[16];
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    // A nibble n OR-ed into the mantissa of binary16 1024 is 1024 + n exactly; one
-                    // that sits four bits higher gives 1024 + 16 n, which one fused multiply-add
-                    // (x / 16 - 72) turns into the same n - 8 without a shift.  So a 32-bit word
-                    // costs one shift and four logic instructions, and the pairs come out as
-                    // (n0, n4), (n1, n5), (n2, n6), (n3, n7): the token tiles carry the same
-                    // permutation of every 8 columns, so no instruction is spent on reordering.
-                    // n - 8 is exact; the product with the scale rounds once (2^-12 relative).
-                    const uint32_t mlo = 0x000F000Fu, mhi = 0x00F000F0u, k1024 = 0x64006400u;
-                    const uint32_t w8 = w[c] >> 8;
-                    uint32_t e[4];
-                    tc_nibble_pair(e[0], w[c], mlo, k1024);
-                    tc_nibble_pair(e[1], w[c], mhi, k1024);
-                    tc_nibble_pair(e[2], w8, mlo, k1024);
-                    tc_nibble_pair(e[3], w8, mhi, k1024);
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const __half2 x = *reinterpret_cast<const __half2 *>(&e[j]);
-                        const __half2 qv = (j & 1) ? __hfma2(x, sixteenth, minus72) : __hadd2(x, minus1032);
-                        const __half2 v = __hmul2(qv, sc2);
-                        o[4 * c + j] = *reinterpret_cast<const uint32_t *>(&v);
-                    }
+                for (int qi = 0; qi < 4; ++qi) {
+                    // (the packed rows are swizzled over their 128 bytes by the TMA copy)
+                    pks[qi] = *reinterpret_cast<const uint4 *>(prow + (((h * 4 + qi) ^ (r & 7)) * 16));
                 }
-                tc_st16(a_slot + (uint32_t)q * 16u, o);          // k-tile q / 2, its columns 16 * (q % 2) ..
+#pragma unroll
+                for (int qi = 0; qi < 4; ++qi) {
+                    const int q = h * 4 + qi;                     // chunk of 32 weights inside the stage
+                    const uint4 pk = pks[qi];
+                    // the block's scale is binary16 already: both halves of a register
+                    const uint32_t sc2u = __byte_perm(sc[qi >> 1], 0u, (qi & 1) ? 0x3232u : 0x1010u);
+                    const __half2 sc2 = *reinterpret_cast<const __half2 *>(&sc2u);
+                    const uint32_t w[4] = {pk.x, pk.y, pk.z, pk.w};
+                    uint32_t o[16];
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        // A nibble n OR-ed into the mantissa of binary16 1024 is 1024 + n exactly; one
+                        // that sits four bits higher gives 1024 + 16 n, which one fused multiply-add
+                        // (x / 16 - 72) turns into the same n - 8 without a shift.  So a 32-bit word
+                        // costs one shift and four logic instructions, and the pairs come out as
+                        // (n0, n4), (n1, n5), (n2, n6), (n3, n7): the token tiles carry the same
+                        // permutation of every 8 columns, so no instruction is spent on reordering.
+                        // n - 8 is exact; the product with the scale rounds once (2^-12 relative).
+                        const uint32_t mlo = 0x000F000Fu, mhi = 0x00F000F0u, k1024 = 0x64006400u;
+                        const uint32_t w8 = w[c] >> 8;
+                        uint32_t e[4];
+                        tc_nibble_pair(e[0], w[c], mlo, k1024);
+                        tc_nibble_pair(e[1], w[c], mhi, k1024);
+                        tc_nibble_pair(e[2], w8, mlo, k1024);
+                        tc_nibble_pair(e[3], w8, mhi, k1024);
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            const __half2 x = *reinterpret_cast<const __half2 *>(&e[j]);
+                            const __half2 qv = (j & 1) ? __hfma2(x, sixteenth, minus72) : __hadd2(x, minus1032);
+                            const __half2 v = __hmul2(qv, sc2);
+                            o[4 * c + j] = *reinterpret_cast<const uint32_t *>(&v);
+                        }
+                    }
+                    tc_st16(a_slot + (uint32_t)q * 16u, o);      // k-tile q / 2, its columns 16 * (q % 2) ..
+                }
             }
-
             asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
             tc_fence_before();
             __syncwarp();
             if (lane == 0) {
-                mbar_arrive(&a_full[ta]);
+                mbar_arrive(&a_full[grp]);
                 mbar_arrive(&empty_bar[s]);                        // the packed tiles have been read
             }
+            s += NG;                                               // (the ring's length is a multiple of the groups)
+            if (s >= S) { s -= S; ring_par ^= 1u; }
+            a_par ^= 1u;
         }
     } else if (warp == 10) {
         // ------------------------------------------------------------------ watcher
@@ -634,11 +662,10 @@ ffn_q4_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ Q4Arg
             if (!tc_bar(&cv_bar, cv_phase, lane)) break;
             if (et == 0) tc_red_release(&ws.sync[kTcReady - 4 + w]);
         }
-    } else {
+    } else if (warp >= 2 && warp <= 5) {
         // ------------------------------------------------------------------ epilogue warps
         const int q = warp & 3;                        // TMEM lane quarter this warp may read
         const long long n_el = (long long)n_routed * sh.f + (long long)sh.n_sh * p.B * sh.f_sh;
-        const uint32_t other = (uint32_t)(2 * pl.n1);  // the next issuer's partial accumulator
         uint32_t run = 0;
         int handed = 0, n_units = 0, W = 0;
         bool alive = tab_wait(0), tabs = false;
@@ -657,31 +684,34 @@ ffn_q4_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ Q4Arg
         for (int ui = 0; ui < n_units && alive; ++ui) {
             uint4 un = unit_at(ui);
             service((int)(un.y >> 20));
-            if (!(un.x & 2u)) continue;                // the run's accumulator is read after its last unit
+            if (!(un.x & 6u)) continue;                // the run's accumulator is read after its last unit
             if (!tabs) {
                 tabs = true;
                 if (!tab_wait(1)) break;
                 un = unit_at(ui);
             }
+            if (!(un.x & 2u)) continue;
             const TcGroup &g = groups[un.y & 0xffffu];
+            const int n = (int)(un.x >> 8), row = (int)un.z + q * 32 + lane;
             const uint32_t buf = run & 1u;
-            const int n = (int)(un.x >> 8), row = (int)un.z * 128 + q * 32 + lane;
             if (!mbar_wait(&acc_full[buf], (run >> 1) & 1u)) {
                 if (lane == 0) atomicExch(ws.status, ST_MBAR_TIMEOUT);
                 alive = false;
                 break;
             }
             tc_fence_after();
-            const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * 2 * NI * pl.n1);
+            const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + buf * (uint32_t)ACC;
             const bool p2 = (un.x & 4u) != 0;
             // slot of the expert's i-th token = g.off + i; walk its tokens in ascending order
-            float *dst = p.pre + (size_t)((un.y >> 16) & 15u) * n_el + act_offset(g.off, n_routed, sh.f, sh.f_sh) + row;
+            const int mi = (int)(un.y >> 16) & 15;
+            float *dst = p.pre + (size_t)(mi >= 3 ? mi - 3 : mi) * n_el + act_offset(g.off, n_routed, sh.f, sh.f_sh) + row;
             const size_t f = (size_t)g.f;
             for (int c = 0; c < n; c += 16) {
-                float v[16], v2[16];                   // phase 2: 8 hi, 8 lo of slots c / 2 .. c / 2 + 7
+                float v[16];                           // phase 2: 8 hi, 8 lo of slots c / 2 .. c / 2 + 7
                 tc_ld16(taddr + c, v);
-                for (int h = 1; h < NI; ++h) {
-                    tc_ld16(taddr + h * other + c, v2);
+                if (2 * n <= ACC) {                    // the odd K-steps' chain
+                    float v2[16];
+                    tc_ld16(taddr + n + c, v2);
 #pragma unroll
                     for (int i = 0; i < 16; ++i) v[i] += v2[i];
                 }

@@ -689,7 +689,7 @@ int verify_one(s2moe_ctx *ctx, int layer, bool first, int B, const void *hidden,
             a.sh = sh; a.ws = ctx->ws; a.plan = qp; a.y = out; a.pre = ctx->pre;
             a.act_hi = ctx->act_hi; a.act_lo = ctx->act_lo; a.B = B;
             LaunchScope scope(ctx, KC_Q4, st);
-            cudaLaunchConfig_t lc = pdl_config(ctx, qp.n_cta, kQ4Threads, qp.smem_bytes, st, qp.early != 0);
+            cudaLaunchConfig_t lc = pdl_config(ctx, qp.n_cta, qp.threads, qp.smem_bytes, st, qp.early != 0);
             cudaLaunchKernelEx(&lc, ffn_q4_kernel, maps, a);
         } else {
             fused::TcArgs a;
