@@ -181,6 +181,8 @@ def _dptr(t: Optional[torch.Tensor]) -> Optional[int]:
 
 # The current stream's handle without a Stream object around it: 0.1 us instead of 3.5 us per call
 _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+# (the device without the check that CUDA is initialised, which whoever has a CUDA tensor has behind him)
+_device = getattr(torch._C, "_cuda_getDevice", torch.cuda.current_device)
 
 
 def _stream_handle(stream: Optional[torch.cuda.Stream]) -> int:
@@ -188,7 +190,7 @@ def _stream_handle(stream: Optional[torch.cuda.Stream]) -> int:
         return stream.cuda_stream
     if _raw_stream is None:
         return torch.cuda.current_stream().cuda_stream
-    return _raw_stream(torch.cuda.current_device())
+    return _raw_stream(_device())
 
 
 @dataclass
@@ -417,7 +419,7 @@ def expert_masks(sel_idx: torch.Tensor, n_experts: int, out: Optional[torch.Tens
     """Predicted expert sets as bit masks through ``s2moe_expert_masks``.  ``sel_idx`` is
     [n_tokens][top_k] int32 on the device; the result is int64 [n_tokens][n_layers][words]
     (bit e % 64 of word e / 64); with ``out`` given, layer ``layer`` of it is written."""
-    lib = load_library()
+    lib = _lib or load_library()
     n, k = sel_idx.shape
     words = (n_experts + 63) // 64
     if out is None:
@@ -436,13 +438,12 @@ def adaptive_expand(parent: torch.Tensor, p_tok: torch.Tensor, masks: torch.Tens
                     stream: Optional[torch.cuda.Stream] = None):
     """Greedy routing-aware admission through ``s2moe_adaptive_expand``.  ``masks`` is int64
     [n_cand][n_layers][words].  Returns (admitted, order, n_admitted, union) on the device."""
-    lib = load_library()
+    lib = _lib or load_library()
     n, n_layers, words = masks.shape
-    dev = masks.device
-    admitted = torch.empty((n,), dtype=torch.int32, device=dev)
-    order = torch.empty((n,), dtype=torch.int32, device=dev)
-    n_adm = torch.empty((1,), dtype=torch.int32, device=dev)
-    union = torch.empty((n_layers, words), dtype=torch.int64, device=dev)
+    admitted = masks.new_empty(n, dtype=torch.int32)
+    order = torch.empty_like(admitted)
+    n_adm = masks.new_empty(1, dtype=torch.int32)
+    union = masks.new_empty((n_layers, words), dtype=torch.int64)
     rc = lib.s2moe_adaptive_expand(n, n_layers, n_experts, _dptr(parent), _dptr(p_tok), _dptr(masks), _dptr(c_draft),
                                    float(t_ar), float(t_exp), _dptr(admitted), _dptr(order), _dptr(n_adm),
                                    _dptr(union), _stream_handle(stream))
