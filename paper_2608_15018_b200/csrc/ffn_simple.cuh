@@ -5,6 +5,11 @@
 //
 //   ffn_gateup_simple : a[slot][j] = silu(W_g[e][j] . x) * (W_u[e][j] . x)
 //   ffn_down_simple   : y[token][r] += p * (W_d[e][r] . a[slot])
+//
+// Small layers are bound by the latency of what depends on what, so every load is issued as soon as its address is
+// known: the first weights of a row before the operands are staged (they need the group only), the tokens from the
+// group's mask instead of the slots' list (one dependent load less), and the second kernel reads the group, its slots
+// and its first weights before it waits for the first one.
 #pragma once
 
 #include "common.cuh"
@@ -62,8 +67,8 @@ __device__ __forceinline__ GroupView group_view(const Shape &sh, const LayerPtrs
         g.sup = (const uint8_t *)lp.sh_s_up + gu * (sh.d / 32) * 2;
         g.sdown = (const uint8_t *)lp.sh_s_down + dn * (sh.f_sh / 32) * 2;
     }
-    g.count = ws.counts[group];
-    g.offset = ws.offsets[group];
+    g.count = __ldcg(&ws.counts[group]);
+    g.offset = __ldcg(&ws.offsets[group]);
     return g;
 }
 
@@ -74,13 +79,14 @@ ffn_gateup_simple(Shape sh, LayerPtrs lp, Workspace ws, const void *__restrict__
 {
     extern __shared__ float s_x[];  // [tok chunk][k chunk]
     simple_dependency();
-    if ((int)blockIdx.y >= ws.header[0]) return;
-    const int group = ws.active[blockIdx.y];
+    const int n_active = __ldcg(&ws.header[0]), group = __ldcg(&ws.active[blockIdx.y]), n_routed = __ldcg(&ws.header[3]) * sh.k;
+    if ((int)blockIdx.y >= n_active) return;
     const GroupView g = group_view(sh, lp, ws, group);
+    unsigned long long mask = __ldcg(&ws.tokmask[group]);      // its tokens that are left
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int j = blockIdx.x * kSimpleWarps + warp;
     if (blockIdx.x * kSimpleWarps >= g.f) return;
-    const int d = sh.d, n_routed = ws.header[3] * sh.k;
+    const int d = sh.d;
     const size_t ab = ACT == DT_F32 ? 4 : 2;
     const bool row_ok = j < g.f;
     const uint8_t *grow = g.gate + (size_t)j * row_bytes(WT, d);
@@ -95,10 +101,17 @@ ffn_gateup_simple(Shape sh, LayerPtrs lp, Workspace ws, const void *__restrict__
         for (int t = 0; t < kSimpleTokChunk; ++t) ag[t] = au[t] = 0.f;
         for (int k0 = 0; k0 < d; k0 += kSimpleKChunk) {
             const int kc = min(kSimpleKChunk, d - k0);
+            float wg[8], wu[8];
+            if (row_ok && lane * 8 < kc) {
+                load8_weight<WT>(grow, gs, k0 + lane * 8, wg);
+                load8_weight<WT>(urow, us, k0 + lane * 8, wu);
+            }
             __syncthreads();
             for (int i = threadIdx.x * 8; i < nt * kc; i += blockDim.x * 8) {
                 const int t = i / kc, c = i - t * kc;
-                const int tok = ws.slot_token[g.offset + t0 + t];
+                unsigned long long m = mask;
+                for (int s = 0; s < t; ++s) m &= m - 1ull;
+                const int tok = __ffsll((long long)m) - 1;
                 float v[8];
                 load8_plain<ACT>((const uint8_t *)hidden + (size_t)tok * d * ab, k0 + c, v);
 #pragma unroll
@@ -107,9 +120,10 @@ ffn_gateup_simple(Shape sh, LayerPtrs lp, Workspace ws, const void *__restrict__
             __syncthreads();
             if (row_ok) {
                 for (int c = lane * 8; c < kc; c += 256) {
-                    float wg[8], wu[8];
-                    load8_weight<WT>(grow, gs, k0 + c, wg);
-                    load8_weight<WT>(urow, us, k0 + c, wu);
+                    if (c >= 256) {
+                        load8_weight<WT>(grow, gs, k0 + c, wg);
+                        load8_weight<WT>(urow, us, k0 + c, wu);
+                    }
 #pragma unroll
                     for (int t = 0; t < kSimpleTokChunk; ++t) {
                         if (t < nt) {
@@ -134,6 +148,7 @@ ffn_gateup_simple(Shape sh, LayerPtrs lp, Workspace ws, const void *__restrict__
                 }
             }
         }
+        for (int t = 0; t < nt; ++t) mask &= mask - 1ull;
     }
 }
 
@@ -143,37 +158,53 @@ __global__ void __launch_bounds__(kSimpleWarps * 32)
 ffn_down_simple(Shape sh, LayerPtrs lp, Workspace ws, float *__restrict__ y)
 {
     extern __shared__ float s_x[];
-    simple_dependency();
-    if ((int)blockIdx.y >= ws.header[0]) return;
-    const int group = ws.active[blockIdx.y];
+    // The kernel in front lets this one start when it has seen the routing kernel's end, so what that one wrote is
+    // there; the activations are not before the dependency.
+    const int n_active = __ldcg(&ws.header[0]), group = __ldcg(&ws.active[blockIdx.y]), n_routed = __ldcg(&ws.header[3]) * sh.k;
+    if ((int)blockIdx.y >= n_active) return;
     const GroupView g = group_view(sh, lp, ws, group);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int r = blockIdx.x * kSimpleWarps + warp;
-    const int d = sh.d, f = g.f, n_routed = ws.header[3] * sh.k;
+    const int d = sh.d, f = g.f;
     const bool row_ok = r < d;
     const uint8_t *drow = g.down + (size_t)r * row_bytes(WT, f);
     const uint8_t *ds = g.sdown + (size_t)r * (f / 32) * 2;
+    bool waited = false;
 
     for (int t0 = 0; t0 < g.count; t0 += kSimpleTokChunk) {
         const int nt = min(kSimpleTokChunk, g.count - t0);
+        // lane t: token and mixing weight of slot t
+        const int slot_l = g.offset + t0 + min(lane, nt - 1), tok_l = __ldcg(&ws.slot_token[slot_l]);
+        const float p_l = __ldcg(&ws.slot_w[slot_l]);
         float acc[kSimpleTokChunk];
 #pragma unroll
         for (int t = 0; t < kSimpleTokChunk; ++t) acc[t] = 0.f;
         for (int k0 = 0; k0 < f; k0 += kSimpleKChunk) {
             const int kc = min(kSimpleKChunk, f - k0);
+            float w[8], w2[8];                          // the first two pieces of the row
+            if (row_ok && lane * 8 < kc) load8_weight<WT>(drow, ds, k0 + lane * 8, w);
+            if (row_ok && 256 + lane * 8 < kc) load8_weight<WT>(drow, ds, k0 + 256 + lane * 8, w2);
+            if (!waited) {
+                waited = true;
+                simple_dependency();
+            }
             __syncthreads();
             for (int i = threadIdx.x * 4; i < nt * kc; i += blockDim.x * 4) {
                 const int t = i / kc, c = i - t * kc;
                 const int slot = g.offset + t0 + t;
-                const float4 v = *reinterpret_cast<const float4 *>(
-                    &ws.act[act_offset(slot, n_routed, sh.f, sh.f_sh) + k0 + c]);
+                const float4 v = __ldcg(reinterpret_cast<const float4 *>(
+                    &ws.act[act_offset(slot, n_routed, sh.f, sh.f_sh) + k0 + c]));
                 *reinterpret_cast<float4 *>(&s_x[t * kSimpleKChunk + c]) = v;
             }
             __syncthreads();
             if (row_ok) {
                 for (int c = lane * 8; c < kc; c += 256) {
-                    float w[8];
-                    load8_weight<WT>(drow, ds, k0 + c, w);
+                    if (c >= 512) {
+                        load8_weight<WT>(drow, ds, k0 + c, w);
+                    } else if (c >= 256) {
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) w[q] = w2[q];
+                    }
 #pragma unroll
                     for (int t = 0; t < kSimpleTokChunk; ++t) {
                         if (t < nt) {
@@ -190,10 +221,7 @@ ffn_down_simple(Shape sh, LayerPtrs lp, Workspace ws, float *__restrict__ y)
         for (int t = 0; t < kSimpleTokChunk; ++t) {
             if (t < nt) {
                 const float s = warp_sum_f(acc[t]);
-                if (lane == 0 && row_ok) {
-                    const int slot = g.offset + t0 + t;
-                    atomicAdd(&y[(size_t)ws.slot_token[slot] * d + r], ws.slot_w[slot] * s);
-                }
+                if (lane == t && row_ok) atomicAdd(&y[(size_t)tok_l * d + r], p_l * s);
             }
         }
     }
