@@ -419,7 +419,7 @@ def expert_masks(sel_idx: torch.Tensor, n_experts: int, out: Optional[torch.Tens
     """Predicted expert sets as bit masks through ``s2moe_expert_masks``.  ``sel_idx`` is
     [n_tokens][top_k] int32 on the device; the result is int64 [n_tokens][n_layers][words]
     (bit e % 64 of word e / 64); with ``out`` given, layer ``layer`` of it is written."""
-    lib = _lib or load_library()
+    lib = load_library()
     n, k = sel_idx.shape
     words = (n_experts + 63) // 64
     if out is None:
@@ -438,7 +438,7 @@ def adaptive_expand(parent: torch.Tensor, p_tok: torch.Tensor, masks: torch.Tens
                     stream: Optional[torch.cuda.Stream] = None):
     """Greedy routing-aware admission through ``s2moe_adaptive_expand``.  ``masks`` is int64
     [n_cand][n_layers][words].  Returns (admitted, order, n_admitted, union) on the device."""
-    lib = _lib or load_library()
+    lib = load_library()
     n, n_layers, words = masks.shape
     admitted = masks.new_empty(n, dtype=torch.int32)
     order = torch.empty_like(admitted)
