@@ -96,8 +96,14 @@ inline Q4Plan q4_make_plan(const Shape &sh, int B, int n_sm, bool early)
     p.n1 = (B + 15) & ~15;
     p.tokb = 2048 * ((B + 7) / 8);             // phase 2: per 8 slots their hi and lo rows; phase 1: n1 rows
     p.tab_bytes = ((int)sizeof(TcGroup) * G + 8 * n_slots + 1023) & ~1023;
-    // Tensor memory: two accumulators of 64 columns (of 128 above 32 tokens) and the slots of the A operand.  Where two of a
-    // unit's N columns fit an accumulator its K-steps go to two chains in turn: the tensor core truncates when it adds.
+    // Tensor memory: two accumulators of 64 columns (of 128 above 32 tokens) and the slots of the A operand.  The K-steps of a
+    // run go to two chains in turn, since the tensor core truncates when it adds: both in one accumulator where twice a
+    // unit's N columns fit it, else, up to 32 tokens, one in each of the two (an expert with 17 and more tokens; the next run
+    // waits for the epilogue then).  Measured for those experts, all tokens on four of them, relative error of the second
+    // projection's sums at d_ff 1536 / 3072 / 6144: two chains 1.9 / 3.1 / 6.5e-7, one chain cut after 12 k-pieces 3.5 /
+    // 6.6 / 12.5e-7.  Time against that, us per layer: Mixtral shape 24 tokens 113.9 / 112.9, 32 tokens 121.0 / 119.2, d_ff
+    // 4096 32 tokens 41.9 / 40.8.  Chains cut after half of every run, so that the accumulators stay two: 44.5 there.
+    // Above 32 tokens an accumulator of 128 columns holds two chains of up to 64, or one of more (33 and more tokens).
     // Three groups of four warps up to 32 tokens, two of eight above (three slots do not fit).  Measured, us per layer at the
     // Mixtral shape, three / two: 8 tokens 96 / 111, 16 tokens 105 / 120, 32 tokens 117 / 133; four-warp groups with a
     // row's eight chunks loaded together 99 / - at 8, and two of them 172 against 164 at 64.
@@ -130,11 +136,11 @@ struct Q4Segments {
 };
 // unit i of this CTA (out of line: it runs once per unit while the tables are built, and only for units
 // past the table afterwards; inlined at every use it pushes the roles' loops out of the instruction cache)
-__device__ __noinline__ uint4 q4_unit_make(const Q4Segments &sg, const TcGroup *groups, const Shape &sh, const Q4Plan &pl, int i)
+__device__ __noinline__ uint4 q4_unit_make(const Q4Segments &sg, const TcGroup *groups, const Shape &sh, int n1, int i)
 {
     int seg = 0, j = i;
     while (seg < kQ4Segs - 1 && j >= sg.cnt[seg]) { j -= sg.cnt[seg]; ++seg; }
-    const int total1 = sg.total1, U = sg.U, u = sg.start[seg] + j, left = sg.cnt[seg] - 1 - j;
+    const int total1 = sg.total1, U = sg.U, u = sg.start[seg] + j, last = sg.cnt[seg] - 1;
     const int kp1 = sh.d >> 8, rb2 = sh.d >> 7;
     int a, mat, rb, piece, kp;
     if (u < total1) {
@@ -157,15 +163,10 @@ __device__ __noinline__ uint4 q4_unit_make(const Q4Segments &sg, const TcGroup *
         piece = local - rb * kp;
         mat = 2;
     }
+    const uint32_t first = j == 0 || piece == 0, end = j == last || piece == kp - 1;
     // (N of a phase-2 unit: 0 before the buckets are known)
-    const uint32_t n = mat < 2 ? (uint32_t)pl.n1 : 16u * (((uint32_t)groups[a].T + 7u) >> 3);
-    // Where up to 32 tokens leave no room for a second chain (17 and more slots) a run ends after 12 pieces, so that no sum has
-    // more terms than with two chains over a whole share (error against float64 at 32 tokens, Mixtral shape:
-    // one chain 3.1496e-4, cut 3.1478e-4, two chains 3.1482e-4).
-    const bool cut = mat == 2 && pl.acc_cols == 64 && 2u * n > 64u;
-    const uint32_t flags = (j == 0 || piece == 0 || (cut && piece % 12 == 0) ? 1u : 0u) |
-                           (left == 0 || piece == kp - 1 || (cut && piece % 12 == 11) ? 2u : 0u) | (mat == 2 ? 4u : 0u);
-    return make_uint4(flags | (n << 8), (uint32_t)a | ((uint32_t)(a >= U ? mat + 3 : mat) << 16) | ((uint32_t)seg << 20),
+    const uint32_t n = mat < 2 ? (uint32_t)n1 : 16u * (((uint32_t)groups[a].T + 7u) >> 3);
+    return make_uint4(first | (end << 1) | (mat == 2 ? 4u : 0u) | (n << 8), (uint32_t)a | ((uint32_t)(a >= U ? mat + 3 : mat) << 16) | ((uint32_t)seg << 20),
                       (uint32_t)rb * 128u, (uint32_t)(4 * piece));
 }
 
@@ -231,8 +232,8 @@ ffn_q4_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ Q4Arg
     tc_fence_after();
     const uint32_t tmem_base = s_tmem;
 
-    auto unit_at = [&](int i) -> uint4 { return i < kQ4MaxUnits ? s_units[i] : q4_unit_make(s_seg, groups, sh, pl, i); };
-    auto umeta_at = [&](int i) -> uint32_t { return i < kQ4MaxUnits ? s_units[i].x : q4_unit_make(s_seg, groups, sh, pl, i).x; };
+    auto unit_at = [&](int i) -> uint4 { return i < kQ4MaxUnits ? s_units[i] : q4_unit_make(s_seg, groups, sh, pl.n1, i); };
+    auto umeta_at = [&](int i) -> uint32_t { return i < kQ4MaxUnits ? s_units[i].x : q4_unit_make(s_seg, groups, sh, pl.n1, i).x; };
     auto map_row = [&](const uint4 &un) -> int {
         const TcGroup &g = groups[un.y & 0xffffu];
         const int mi = (int)(un.y >> 16) & 15;
@@ -340,7 +341,7 @@ ffn_q4_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ Q4Arg
         }
         asm volatile("bar.sync 1, 128;" ::: "memory");
         for (int i = tt; i < n_units && i < kQ4MaxUnits; i += 128) {
-            const uint4 un = q4_unit_make(s_seg, groups, sh, pl, i);
+            const uint4 un = q4_unit_make(s_seg, groups, sh, pl.n1, i);
             s_units[i] = un;
             s_row[i] = map_row(un);
         }
@@ -365,7 +366,7 @@ ffn_q4_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ Q4Arg
         asm volatile("bar.sync 1, 128;" ::: "memory");
         const int n_p1 = s_seg.cnt[0] + s_seg.cnt[1];
         for (int i = n_p1 + tt; i < n_units && i < kQ4MaxUnits; i += 128)
-            s_units[i].x = q4_unit_make(s_seg, groups, sh, pl, i).x;
+            s_units[i].x = (s_units[i].x & 0xffu) | ((16u * (((uint32_t)groups[s_units[i].y & 0xffffu].T + 7u) >> 3)) << 8);
         asm volatile("bar.sync 1, 128;" ::: "memory");
         if (tt == 0) mbar_arrive(&tab_bar[1]);
     }
@@ -385,7 +386,7 @@ ffn_q4_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ Q4Arg
                     un = s_units[i];
                     row = s_row[i];
                 } else {
-                    un = q4_unit_make(s_seg, groups, sh, pl, i);
+                    un = q4_unit_make(s_seg, groups, sh, pl.n1, i);
                     row = map_row(un);
                 }
                 const CUtensorMap *map = &maps.m[(un.y >> 16) & 15u];
@@ -468,10 +469,15 @@ ffn_q4_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ Q4Arg
                 // slot ta's k-tiles (32 columns each) and their token tiles: phase 1 [k-tile][rows], phase 2
                 // [8 slots][hi | lo][k-tile][8 rows] (8-row groups 4 KiB apart)
                 const uint32_t N = m >> 8, idesc = tc_idesc_f16((int)N), d_tmem = tmem_base + buf * (uint32_t)ACC;
-                const uint32_t odd = 2u * N <= (uint32_t)ACC ? N : 0u;     // where the odd K-steps add up
+                // where the odd K-steps add up: behind the even ones, in the other accumulator, or with them
+                const bool both = ACC == 64 && 2u * N > 64u;
+                const uint32_t odd = 2u * N <= (uint32_t)ACC ? N : !both ? 0u : buf ? 0u - 64u : 64u;
                 const uint32_t a_tm = a_tmem0 + (uint32_t)ta * (kTcQ4KG * 32u), b_lo = tok_lo + (uint32_t)ta * tok_slot;
                 const uint32_t b_step = p2 ? 64u : step1, b_hi = p2 ? hi2 : hi1;
-                if (first && !mbar_wait(&acc_empty[buf], run_par)) { atomicExch(ws.status, ST_MBAR_TIMEOUT); break; }
+                if (first && (!mbar_wait(&acc_empty[buf], run_par) || (both && !mbar_wait(&acc_empty[buf ^ 1u], run_par ^ buf)))) {
+                    atomicExch(ws.status, ST_MBAR_TIMEOUT);
+                    break;
+                }
                 if (ui + 1 < n_units) um = umeta_at(ui + 1);
                 // the unit in tensor memory, written by the dequantising warps, and its token tiles
                 if (!mbar_wait(&a_full[ta], a_par)) { atomicExch(ws.status, ST_MBAR_TIMEOUT); break; }
@@ -485,8 +491,9 @@ ffn_q4_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ Q4Arg
                 tc_commit(&a_empty[ta]);               // frees the A operand and the token tiles
                 if (m & 2u) {
                     tc_commit(&acc_full[buf]);
-                    buf ^= 1u;
-                    if (buf == 0) run_par ^= 1u;
+                    if (both) tc_commit(&acc_full[buf ^ 1u]);      // (and the accumulator in turn is the same one)
+                    else buf ^= 1u;
+                    if (both || buf == 0) run_par ^= 1u;
                 }
                 tc_ring_next(ta, a_par, NG);
             }
@@ -694,7 +701,8 @@ ffn_q4_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ Q4Arg
             const TcGroup &g = groups[un.y & 0xffffu];
             const int n = (int)(un.x >> 8), row = (int)un.z + q * 32 + lane;
             const uint32_t buf = run & 1u;
-            if (!mbar_wait(&acc_full[buf], (run >> 1) & 1u)) {
+            const bool both = ACC == 64 && 2 * n > 64;                  // the run's two chains took both accumulators
+            if (!mbar_wait(&acc_full[buf], (run >> 1) & 1u) || (both && !mbar_wait(&acc_full[buf ^ 1u], ((run + 1u) >> 1) & 1u))) {
                 if (lane == 0) atomicExch(ws.status, ST_MBAR_TIMEOUT);
                 alive = false;
                 break;
@@ -706,14 +714,18 @@ ffn_q4_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ Q4Arg
             const int mi = (int)(un.y >> 16) & 15;
             float *dst = p.pre + (size_t)(mi >= 3 ? mi - 3 : mi) * n_el + act_offset(g.off, n_routed, sh.f, sh.f_sh) + row;
             const size_t f = (size_t)g.f;
+            const uint32_t odd = both ? (buf ? 0u - 64u : 64u) : (uint32_t)n;   // columns from a chain to the odd K-steps' one
             for (int c = 0; c < n; c += 16) {
                 float v[16];                           // phase 2: 8 hi, 8 lo of slots c / 2 .. c / 2 + 7
-                tc_ld16(taddr + c, v);
-                if (2 * n <= ACC) {                    // the odd K-steps' chain
-                    float v2[16];
-                    tc_ld16(taddr + n + c, v2);
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) v[i] += v2[i];
+                if (both || 2 * n <= ACC) tc_ld16_sum(taddr + c, taddr + odd + c, v);
+                else tc_ld16(taddr + c, v);
+                if (c + 16 >= n) {                     // the accumulator may be overwritten
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) {
+                        mbar_arrive(&acc_empty[buf]);
+                        if (both) mbar_arrive(&acc_empty[buf ^ 1u]);
+                    }
                 }
                 if (!p2) {
                     const unsigned m16 = (unsigned)((g.mask >> c) & 0xffffull);
@@ -732,11 +744,7 @@ ffn_q4_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ Q4Arg
                     }
                 }
             }
-            // the accumulator may be overwritten
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&acc_empty[buf]);
-            ++run;
+            run += both ? 2u : 1u;
         }
         service(kQ4Segs);
     }
