@@ -6,10 +6,18 @@
 //   ffn_gateup_simple : a[slot][j] = silu(W_g[e][j] . x) * (W_u[e][j] . x)
 //   ffn_down_simple   : y[token][r] += p * (W_d[e][r] . a[slot])
 //
-// Small layers are bound by the latency of what depends on what, so every load is issued as soon as its address is
-// known: the first weights of a row before the operands are staged (they need the group only), the tokens from the
-// group's mask instead of the slots' list (one dependent load less), and the second kernel reads the group, its slots
-// and its first weights before it waits for the first one.
+// Small layers are bound by the latency of what depends on what, so loads are issued as soon as their address is
+// known: fp32 weights of a row's first pieces before the operands are staged (they need the group only), the tokens of a
+// group of one chunk from its mask instead of the slots' list (one dependent load less), and the first blocks of the
+// second kernel read the group, its slots and its first weights before they wait for the first kernel.
+// Large ones are bound by how long a block occupies its SM (64 KiB of shared memory: three at a time), and most blocks of a
+// layer with many experts belong to a group without tokens: those leave after loads that hit L1 (after loads from L2 half of
+// such a layer's time went into them), and rows of many pieces in 16 bits and less take their weights in the loop.
+// Measured in a captured stack, us per layer, everything read behind the dependency / now: fp32, 8 experts of 256 x 512,
+// 1, 4, 16 tokens 14.3, 16.5, 27.2 / 13.8, 15.9, 26.8; fp32, 64 experts of 2048 x 1024, 1, 8, 64 tokens 76.1, 180, 1023 / 74.8,
+// 176, 1007; bf16 the same 68.5, 163, 932 / 69.5, 163, 919; int4, 8 experts of 4096 x 14336, 1, 8, 64 tokens 284, 835, 5432 /
+// 285, 836, 5442.  With the early reads by every block and every weight format: 64 experts, 1 token 123 (fp32) and 120
+// (bf16), int4 332, 899 and 5562.
 #pragma once
 
 #include "common.cuh"
@@ -39,11 +47,9 @@ struct GroupView {
     const uint8_t *gate, *up, *down;        // first row of this group's matrices
     const uint8_t *sgate, *sup, *sdown;     // first scale
     int f;                                  // inner dim of this group
-    int count, offset;                      // tokens, first slot
 };
 
-__device__ __forceinline__ GroupView group_view(const Shape &sh, const LayerPtrs &lp, const Workspace &ws,
-                                                int group)
+__device__ __forceinline__ GroupView group_view(const Shape &sh, const LayerPtrs &lp, int group)
 {
     GroupView g;
     const int wt = sh.weight_dtype;
@@ -67,8 +73,6 @@ __device__ __forceinline__ GroupView group_view(const Shape &sh, const LayerPtrs
         g.sup = (const uint8_t *)lp.sh_s_up + gu * (sh.d / 32) * 2;
         g.sdown = (const uint8_t *)lp.sh_s_down + dn * (sh.f_sh / 32) * 2;
     }
-    g.count = __ldcg(&ws.counts[group]);
-    g.offset = __ldcg(&ws.offsets[group]);
     return g;
 }
 
@@ -79,10 +83,11 @@ ffn_gateup_simple(Shape sh, LayerPtrs lp, Workspace ws, const void *__restrict__
 {
     extern __shared__ float s_x[];  // [tok chunk][k chunk]
     simple_dependency();
-    const int n_active = __ldcg(&ws.header[0]), group = __ldcg(&ws.active[blockIdx.y]), n_routed = __ldcg(&ws.header[3]) * sh.k;
+    const int n_active = ws.header[0], group = ws.active[blockIdx.y], n_routed = ws.header[3] * sh.k;
     if ((int)blockIdx.y >= n_active) return;
-    const GroupView g = group_view(sh, lp, ws, group);
-    unsigned long long mask = __ldcg(&ws.tokmask[group]);      // its tokens that are left
+    const GroupView g = group_view(sh, lp, group);
+    const int count = ws.counts[group], offset = ws.offsets[group];
+    const unsigned long long mask = ws.tokmask[group];         // its tokens
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int j = blockIdx.x * kSimpleWarps + warp;
     if (blockIdx.x * kSimpleWarps >= g.f) return;
@@ -94,24 +99,29 @@ ffn_gateup_simple(Shape sh, LayerPtrs lp, Workspace ws, const void *__restrict__
     const uint8_t *gs = g.sgate + (size_t)j * (d / 32) * 2;
     const uint8_t *us = g.sup + (size_t)j * (d / 32) * 2;
 
-    for (int t0 = 0; t0 < g.count; t0 += kSimpleTokChunk) {
-        const int nt = min(kSimpleTokChunk, g.count - t0);
+    for (int t0 = 0; t0 < count; t0 += kSimpleTokChunk) {
+        const int nt = min(kSimpleTokChunk, count - t0);
         float ag[kSimpleTokChunk], au[kSimpleTokChunk];
 #pragma unroll
         for (int t = 0; t < kSimpleTokChunk; ++t) ag[t] = au[t] = 0.f;
         for (int k0 = 0; k0 < d; k0 += kSimpleKChunk) {
             const int kc = min(kSimpleKChunk, d - k0);
             float wg[8], wu[8];
-            if (row_ok && lane * 8 < kc) {
+            if (WT == DT_F32 && row_ok && lane * 8 < kc) {
                 load8_weight<WT>(grow, gs, k0 + lane * 8, wg);
                 load8_weight<WT>(urow, us, k0 + lane * 8, wu);
             }
             __syncthreads();
             for (int i = threadIdx.x * 8; i < nt * kc; i += blockDim.x * 8) {
                 const int t = i / kc, c = i - t * kc;
-                unsigned long long m = mask;
-                for (int s = 0; s < t; ++s) m &= m - 1ull;
-                const int tok = __ffsll((long long)m) - 1;
+                int tok;
+                if (count <= kSimpleTokChunk) {
+                    unsigned long long m = mask;
+                    for (int s = 0; s < t; ++s) m &= m - 1ull;
+                    tok = __ffsll((long long)m) - 1;
+                } else {
+                    tok = ws.slot_token[offset + t0 + t];
+                }
                 float v[8];
                 load8_plain<ACT>((const uint8_t *)hidden + (size_t)tok * d * ab, k0 + c, v);
 #pragma unroll
@@ -120,7 +130,7 @@ ffn_gateup_simple(Shape sh, LayerPtrs lp, Workspace ws, const void *__restrict__
             __syncthreads();
             if (row_ok) {
                 for (int c = lane * 8; c < kc; c += 256) {
-                    if (c >= 256) {
+                    if (WT != DT_F32 || c >= 256) {
                         load8_weight<WT>(grow, gs, k0 + c, wg);
                         load8_weight<WT>(urow, us, k0 + c, wu);
                     }
@@ -143,47 +153,52 @@ ffn_gateup_simple(Shape sh, LayerPtrs lp, Workspace ws, const void *__restrict__
             if (t < nt) {
                 const float sg = warp_sum_f(ag[t]), su = warp_sum_f(au[t]);
                 if (lane == 0 && row_ok) {
-                    const int slot = g.offset + t0 + t;
+                    const int slot = offset + t0 + t;
                     ws.act[act_offset(slot, n_routed, sh.f, sh.f_sh) + j] = silu_mul(sg, su);
                 }
             }
         }
-        for (int t = 0; t < nt; ++t) mask &= mask - 1ull;
     }
 }
 
-// grid (ceil(d / kSimpleWarps), E + n_sh); same dynamic smem
+// grid (ceil(d / kSimpleWarps), E + n_sh); same dynamic smem.  Only ever launched directly behind ffn_gateup_simple of the same
+// layer (launch_simple), whose blocks let it start when they have seen the routing kernel's end: so what that one wrote is
+// there for the blocks that read it before their dependency, while the activations are not.  Those are the blocks that come
+// up first (early_blocks, as many as run at a time; the later ones find the first kernel ended) of groups that
+// every batch has (a token selects k different experts); the others wait first and read through L1.
 template <int WT>
 __global__ void __launch_bounds__(kSimpleWarps * 32)
-ffn_down_simple(Shape sh, LayerPtrs lp, Workspace ws, float *__restrict__ y)
+ffn_down_simple(Shape sh, LayerPtrs lp, Workspace ws, float *__restrict__ y, int early_blocks)
 {
     extern __shared__ float s_x[];
-    // The kernel in front lets this one start when it has seen the routing kernel's end, so what that one wrote is
-    // there; the activations are not before the dependency.
-    const int n_active = __ldcg(&ws.header[0]), group = __ldcg(&ws.active[blockIdx.y]), n_routed = __ldcg(&ws.header[3]) * sh.k;
+    const bool early = (int)(blockIdx.y * gridDim.x + blockIdx.x) < early_blocks && (int)blockIdx.y < sh.k + sh.n_sh;
+    bool waited = !early;
+    if (waited) simple_dependency();
+    auto word = [&](const int32_t *p) { return early ? __ldcg(p) : *p; };
+    const int n_active = word(&ws.header[0]), group = word(&ws.active[blockIdx.y]), n_routed = word(&ws.header[3]) * sh.k;
     if ((int)blockIdx.y >= n_active) return;
-    const GroupView g = group_view(sh, lp, ws, group);
+    const GroupView g = group_view(sh, lp, group);
+    const int count = word(&ws.counts[group]), offset = word(&ws.offsets[group]);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int r = blockIdx.x * kSimpleWarps + warp;
     const int d = sh.d, f = g.f;
     const bool row_ok = r < d;
     const uint8_t *drow = g.down + (size_t)r * row_bytes(WT, f);
     const uint8_t *ds = g.sdown + (size_t)r * (f / 32) * 2;
-    bool waited = false;
 
-    for (int t0 = 0; t0 < g.count; t0 += kSimpleTokChunk) {
-        const int nt = min(kSimpleTokChunk, g.count - t0);
+    for (int t0 = 0; t0 < count; t0 += kSimpleTokChunk) {
+        const int nt = min(kSimpleTokChunk, count - t0);
         // lane t: token and mixing weight of slot t
-        const int slot_l = g.offset + t0 + min(lane, nt - 1), tok_l = __ldcg(&ws.slot_token[slot_l]);
-        const float p_l = __ldcg(&ws.slot_w[slot_l]);
+        const int slot_l = offset + t0 + min(lane, nt - 1), tok_l = word(&ws.slot_token[slot_l]);
+        const float p_l = early ? __ldcg(&ws.slot_w[slot_l]) : ws.slot_w[slot_l];
         float acc[kSimpleTokChunk];
 #pragma unroll
         for (int t = 0; t < kSimpleTokChunk; ++t) acc[t] = 0.f;
         for (int k0 = 0; k0 < f; k0 += kSimpleKChunk) {
             const int kc = min(kSimpleKChunk, f - k0);
             float w[8], w2[8];                          // the first two pieces of the row
-            if (row_ok && lane * 8 < kc) load8_weight<WT>(drow, ds, k0 + lane * 8, w);
-            if (row_ok && 256 + lane * 8 < kc) load8_weight<WT>(drow, ds, k0 + 256 + lane * 8, w2);
+            if (WT == DT_F32 && row_ok && lane * 8 < kc) load8_weight<WT>(drow, ds, k0 + lane * 8, w);
+            if (WT == DT_F32 && row_ok && 256 + lane * 8 < kc) load8_weight<WT>(drow, ds, k0 + 256 + lane * 8, w2);
             if (!waited) {
                 waited = true;
                 simple_dependency();
@@ -191,15 +206,15 @@ ffn_down_simple(Shape sh, LayerPtrs lp, Workspace ws, float *__restrict__ y)
             __syncthreads();
             for (int i = threadIdx.x * 4; i < nt * kc; i += blockDim.x * 4) {
                 const int t = i / kc, c = i - t * kc;
-                const int slot = g.offset + t0 + t;
-                const float4 v = __ldcg(reinterpret_cast<const float4 *>(
-                    &ws.act[act_offset(slot, n_routed, sh.f, sh.f_sh) + k0 + c]));
+                const int slot = offset + t0 + t;
+                const float4 v = *reinterpret_cast<const float4 *>(
+                    &ws.act[act_offset(slot, n_routed, sh.f, sh.f_sh) + k0 + c]);
                 *reinterpret_cast<float4 *>(&s_x[t * kSimpleKChunk + c]) = v;
             }
             __syncthreads();
             if (row_ok) {
                 for (int c = lane * 8; c < kc; c += 256) {
-                    if (c >= 512) {
+                    if (WT != DT_F32 || c >= 512) {
                         load8_weight<WT>(drow, ds, k0 + c, w);
                     } else if (c >= 256) {
 #pragma unroll

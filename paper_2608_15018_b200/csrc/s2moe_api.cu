@@ -327,6 +327,7 @@ cudaError_t prepare_route()
 }
 
 constexpr size_t kSimpleSmem = (size_t)kSimpleTokChunk * kSimpleKChunk * sizeof(float);
+constexpr int kSimplePerSm = 3;       // blocks of that much shared memory on an SM
 
 template <int WT, int ACT>
 void launch_simple(s2moe_ctx *ctx, const LayerPtrs &lp, const void *hidden, float *out, cudaStream_t st)
@@ -343,10 +344,12 @@ void launch_simple(s2moe_ctx *ctx, const LayerPtrs &lp, const void *hidden, floa
         cudaLaunchKernelEx(&lc, ffn_gateup_simple<WT, ACT>, sh, lp, ctx->ws, hidden);
     }
     {
+        // (nothing may come between the two launches: the second kernel reads the routing kernel's tables before its own
+        // dependency, on the word of the first one's blocks)
         LaunchScope scope(ctx, KC_DOWN, st);
         cudaLaunchConfig_t lc = pdl_config(ctx, 1, kSimpleWarps * 32, kSimpleSmem, st);
         lc.gridDim = g2;
-        cudaLaunchKernelEx(&lc, ffn_down_simple<WT>, sh, lp, ctx->ws, out);
+        cudaLaunchKernelEx(&lc, ffn_down_simple<WT>, sh, lp, ctx->ws, out, kSimplePerSm * ctx->n_sm);
     }
 }
 

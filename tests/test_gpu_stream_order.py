@@ -77,3 +77,52 @@ def test_weights_written_just_before_the_call(cfg, B, early, call, how, monkeypa
         assert m.device_status() == 0
     for l in range(2):
         check_outputs(wl, new[l], H[l], None, views[l])
+
+
+@pytest.mark.parametrize("how", ["copy", "early trigger"])
+@pytest.mark.parametrize("call", ["layer", "stack", "graph"])
+@pytest.mark.parametrize("cfg,B", [("cfg1", 1), ("cfg1", 9), ("cfg2", 4), ("cfg4", 4)])
+def test_weights_written_just_before_the_call_of_the_cuda_core_kernels(cfg, B, call, how):
+    """The second kernel of kernel plan 1 reads the routing kernel's tables and weights before it waits for the first: both
+    layers' weights written in front of the call, the second layer's again between the two calls of single layers."""
+    wl = CONFIGS[cfg].with_(d_model=256, d_ff=512, n_experts=12, top_k=3, cap=6, n_layers=2, n_shared=1, d_ff_shared=256,
+                            shared_gate=True)
+    kernel = torch.cuda._compile_kernel(WRITER, "late_copy") if how != "copy" else None
+    old = [workloads.layer_weights(wl.with_(seed=91), l, "cuda") for l in range(2)]
+    new = [workloads.layer_weights(wl, l, "cuda") for l in range(2)]
+    H = torch.stack([workloads.hidden_states(wl, l, B, device="cuda") for l in range(2)])
+    with binding.S2MoE(binding.Config.from_workload(wl, n_layers=2, kernel_plan=1), old) as m:
+        o = m.alloc_outputs(B, stack=True)
+        views = [binding.LayerOutput(o.out[l], o.sel_idx[l], o.sel_w[l], o.n_unique[l:l + 1]) for l in range(2)]
+        m.verify_stack(H, None, o)
+        torch.cuda.synchronize()
+        side = torch.cuda.Stream()
+
+        def refresh(l):
+            for name in sorted(new[l], key=lambda n: "down" in n):       # W_down last
+                if new[l][name].numel() * new[l][name].element_size() % 16:
+                    old[l][name].copy_(new[l][name])
+                else:
+                    _write(how, kernel, old[l][name], new[l][name])
+
+        def calls(stream=None):
+            if call == "layer":
+                for l in range(2):
+                    refresh(l)
+                    m.verify_layer(l, H[l], None, views[l], stream=stream)
+            else:
+                for l in (1, 0):
+                    refresh(l)
+                m.verify_stack(H, None, o, stream=stream)
+
+        if call == "graph":
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph, stream=side):
+                calls(side)
+            graph.replay()
+        else:
+            calls()
+        torch.cuda.synchronize()
+        assert m.device_status() == 0
+    for l in range(2):
+        check_outputs(wl, new[l], H[l], None, views[l])
