@@ -319,12 +319,16 @@ adaptive_expand_regs_kernel(int n, int lw, int lp, const int32_t *__restrict__ p
     if (i == 0) *n_admitted = bad ? -1 : count;          // -1: parent[] was malformed
     if (union_out) {
         __syncthreads();
-        for (int w = warp; w < lw; w += n_warps) {
+        // as many threads of a warp per word as there are for all words
+        int lg = 0;
+        while (lg < 5 && (lw << (lg + 1)) <= (int)blockDim.x) ++lg;
+        for (int base = 0; base < lw; base += (int)blockDim.x >> lg) {
+            const int w = base + (i >> lg);
             unsigned long long u = 0ull;
-            for (int e = lane; e < n; e += 32)
-                if (s_adm[e]) u |= s_rows[e * pitch + w];
-            u = ((unsigned long long)__reduce_or_sync(0xffffffffu, (unsigned)(u >> 32)) << 32) | __reduce_or_sync(0xffffffffu, (unsigned)u);
-            if (lane == 0) union_out[w] = u;
+            if (w < lw)
+                for (int e = i & ((1 << lg) - 1); e < n; e += 1 << lg) u |= s_rows[e * pitch + w] & (0ull - (unsigned long long)s_adm[e]);
+            for (int o = 1 << lg >> 1; o > 0; o >>= 1) u |= __shfl_xor_sync(0xffffffffu, u, o);
+            if (w < lw && (i & ((1 << lg) - 1)) == 0) union_out[w] = u;
         }
     }
 }

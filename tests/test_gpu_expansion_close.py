@@ -1,6 +1,7 @@
 """The admission kernel where an approximate utility cannot decide: utilities that differ in the last places of float32
 or float64, that are equal, that lie at 1, and operands outside the ranges of the approximation (zero, negative, tiny,
-huge), in every layout of the words in registers.  Decisions exactly those of the oracle."""
+huge, not a number), in every layout of the words in registers (1 to 32 threads a candidate, two and four pairs of words each,
+blocks on both sides of 512 threads) and beyond them.  Decisions exactly those of the oracle."""
 import random
 
 import numpy as np
@@ -35,14 +36,25 @@ def _operands(kind, n, rng):
                 2.0, 0.125)
     if kind == "tiny":
         return [x * 2.0 ** -80 for x in near], [2.0 ** -82] * n, 1.0, 2.0 ** -84
+    if kind == "equal":
+        return [1.0] * n, [0.5] * n, 64.0, 0.125
+    if kind == "no draft cost":   # c_draft NULL: a candidate that brings nothing new costs nothing, whatever its confidence
+        return [rng.choice([0.0, 1e-30, 0.5, 0.75, 0.75]) for _ in range(n)], None, 16.0, 0.125
+    if kind == "not a number":
+        return [rng.choice([float("nan"), 0.5, 0.75, 0.875]) for _ in range(n)], [0.25] * n, 16.0, 0.125
+    if kind == "huge benefit":
+        return [rng.choice([2.0 ** 90, 0.5]) for _ in range(n)], [0.25] * n, 4.0, 0.125
     if kind == "huge":
         return near, [2.0 ** 100] * n, 2.0 ** 102, 2.0 ** 98
     return near, [rng.choice([0.5, float("inf")]) for _ in range(n)], 16.0, 0.125
 
 
-@pytest.mark.parametrize("kind", ["last places", "at one", "products", "zero costs", "signs", "tiny", "huge", "infinite"])
+@pytest.mark.parametrize("kind", ["last places", "at one", "products", "zero costs", "signs", "tiny", "huge", "infinite", "equal",
+                                  "no draft cost", "not a number", "huge benefit"])
 @pytest.mark.parametrize("n,n_layers,n_experts", [(5, 1, 64), (64, 16, 64), (33, 9, 128), (64, 48, 128), (65, 3, 64),
-                                                  (96, 24, 128), (160, 48, 128), (256, 20, 128)])
+                                                  (96, 24, 128), (160, 48, 128), (256, 20, 128), (1, 48, 128), (32, 48, 128),
+                                                  (32, 128, 128), (8, 128, 128), (64, 32, 64), (33, 16, 64), (128, 16, 64),
+                                                  (129, 16, 64), (256, 8, 64)])
 def test_close_and_extreme_utilities(n, n_layers, n_experts, kind):
     from paper_2608_15018_b200 import binding
 
@@ -56,11 +68,12 @@ def test_close_and_extreme_utilities(n, n_layers, n_experts, kind):
         for _ in range(4):
             s[rng.randrange(n_layers)] |= 1 << rng.randrange(n_experts)
     masks = [list(rng.choice(sets)) for _ in range(n)]
-    want_adm, want_order, want_union = ox.adaptive_expand(parent, p_tok, masks, c_draft, t_ar, t_exp)
+    want_adm, want_order, want_union = ox.adaptive_expand(parent, p_tok, masks, c_draft or [0.0] * n, t_ar, t_exp)
     words = (n_experts + 63) // 64
     adm, order, n_adm, union = binding.adaptive_expand(
         torch.tensor(parent, dtype=torch.int32, device=dev), torch.tensor(p_tok, dtype=torch.float32, device=dev),
-        _masks_tensor(masks, words, dev), n_experts, torch.tensor(c_draft, dtype=torch.float32, device=dev), t_ar, t_exp)
+        _masks_tensor(masks, words, dev), n_experts, None if c_draft is None else torch.tensor(c_draft, dtype=torch.float32, device=dev),
+        t_ar, t_exp)
     torch.cuda.synchronize()
     assert order.cpu().tolist() == want_order + [-1] * (n - len(want_order))
     assert adm.cpu().tolist() == want_adm and n_adm.item() == len(want_order)

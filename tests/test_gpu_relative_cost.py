@@ -44,3 +44,21 @@ def test_experts_that_nobody_selected(cfg):
             o = m.alloc_outputs(1, stack=True)
             us.append(_us(lambda stream: m.verify_stack(H, None, o, stream=stream)))
     assert us[1] < 1.5 * us[0]
+
+
+def _expand_us(n, n_layers, p_last=0.9, parent_last=-1, p=0.9, c_draft=False):
+    """A call of adaptive_expand: n roots (the last one as given), each with experts of its own."""
+    gen = torch.Generator().manual_seed(n)
+    masks = torch.randint(0, 2 ** 62, (n, n_layers, 1), generator=gen).cuda()
+    p_tok = torch.full((n,), p) + torch.rand((n,), generator=gen) * 0.05
+    p_tok[n - 1] = p_last
+    parent = torch.full((n,), -1, dtype=torch.int32)
+    parent[n - 1] = parent_last
+    parent, p_tok, c = parent.cuda(), p_tok.cuda(), torch.full((n,), 0.5).cuda() if c_draft else None
+    return _us(lambda stream: binding.adaptive_expand(parent, p_tok, masks, 64, c, 1e6, 0.125, stream=stream))
+
+
+def test_few_candidates_with_many_words():
+    """One candidate of 96 words against 32 of them (measured a ninth; two thirds where its one warp formed the union word
+    by word)."""
+    assert _expand_us(1, 96) < 0.33 * _expand_us(32, 96)
