@@ -1432,18 +1432,18 @@ int s2moe_adaptive_expand(int32_t n_cand, int32_t n_layers, int32_t n_experts, c
     if (!parent || !p_tok || !masks || !admitted || !order || !n_admitted) return S2MOE_EINVAL;
     const int lw = n_layers * ((n_experts + 63) / 64);
     if (n_cand > kExpandMaxCand || lw > kExpandMaxWords) return S2MOE_ERANGE;
-    // Words in registers where two or four pairs per thread of at most 1024 hold them: measured, us per call, this kernel /
-    // the one below: 8 candidates x 2 words 6.9 / 10.8, 32 x 24 19.0 / 37.9, 64 x 16 32.8 / 72.4, 64 x 96 88.3 / 101.6,
-    // 128 x 8 78.9 / 133.6; with twelve pairs per thread 160 x 96 322 / 261.
+    // Words in registers where two or four pairs per thread of at most 1024 hold them, above 64 candidates two per thread of
+    // at most 512 (all warps look through all keys): measured, us per call, in registers / by the kernel below, 96
+    // candidates x 16 words 76.7 / 109, 128 x 16 118 / 142, 256 x 8 224 / 259; beyond the line 160 x 16 169 / 175, 96 x 24 121 / 109,
+    // 128 x 24 204 / 147, 256 x 16 396 / 277, with four pairs 96 x 48 147 / 127, 128 x 64 249 / 175, 160 x 24 204 / 185.
     const int pairs = (lw + 1) / 2;
     for (const int wp : {2, 4}) {
         int lp = 0;
         while ((wp << lp) < pairs) ++lp;
-        if (lp > 5 || n_cand << lp > 1024) continue;
+        if (lp > 5 || n_cand << lp > (n_cand <= 64 ? 1024 : 512) || (n_cand > 64 && wp > 2)) continue;
         const int threads = ((n_cand << lp) + 31) / 32 * 32;
         const size_t rows = sizeof(uint64_t) * (size_t)n_cand * (2 * wp << lp);
-        auto *kernel = n_cand <= 64 ? (wp == 2 ? adaptive_expand_regs_kernel<2, 2> : adaptive_expand_regs_kernel<2, 4>)
-                                    : (wp == 2 ? adaptive_expand_regs_kernel<8, 2> : adaptive_expand_regs_kernel<8, 4>);
+        auto *kernel = n_cand > 64 ? adaptive_expand_regs_kernel<8, 2> : wp == 2 ? adaptive_expand_regs_kernel<2, 2> : adaptive_expand_regs_kernel<2, 4>;
         if (rows > 32 * 1024 &&
             cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kExpandMaxSmem) != cudaSuccess)
             return S2MOE_ECUDA;
