@@ -181,19 +181,19 @@ adaptive_expand_kernel(int n, int lw, const int32_t *__restrict__ parent, const 
         for (int w = i; w < lw; w += blockDim.x) union_out[w] = s_union[w];
 }
 
-// The candidate of largest utility among those whose key is at least `near`, or -1 if that utility is below 1; by a
-// whole warp (every warp of the block does it for itself).
+// The candidate of largest utility among those whose key is at least `near`, or -1 if that utility is below 1; by the whole
+// block, all of whose warps are here: a thread divides for each candidate, every warp finds the largest for itself.
 __device__ __noinline__ int expand_resolve(const unsigned *keys, const int *fresh, const double *benefit, const double *c_draft,
-                                           double t_exp, int nw, unsigned near)
+                                           unsigned long long *s_exact, double t_exp, int nw, unsigned near)
 {
-    const int lane = threadIdx.x & 31;
+    const int i = threadIdx.x, lane = i & 31;
+    if (i < 32 * nw) s_exact[i] = keys[i] >= near ? expand_key(benefit[i], fresh[i], t_exp, c_draft[i]) : 0ull;
+    __syncthreads();
     unsigned long long best = 0ull;
     int at = 0;
     for (int q = 0; q < nw; ++q) {
-        const int e = 32 * q + lane;
-        if (keys[e] < near) continue;
-        const unsigned long long key = expand_key(benefit[e], fresh[e], t_exp, c_draft[e]);
-        if (key > best) { best = key; at = e; }
+        const unsigned long long key = s_exact[32 * q + lane];
+        if (key > best) { best = key; at = 32 * q + lane; }
     }
     const unsigned long long bk = warp_max_key(best);
     if (bk == 0ull || !(dkey_value(bk) >= 1.0)) return -1;
@@ -207,10 +207,15 @@ __device__ __noinline__ int expand_resolve(const unsigned *keys, const int *fres
 // cycles.  So the threads find the largest utility by an approximate one in float32 (a dozen instructions for the
 // division's hundred, no conversion), every warp for itself, from keys that alternate between two buffers: one barrier
 // per admission.  Only where another key lies within 2^-19 of the largest, or that one so close to 1, are utilities divided
-// out in float64 (expand_resolve), so the decisions are those of the definition.  The approximation is within 5 units of
-// its last place (three roundings, a reciprocal of 1 unit) for operands in the ranges that `plain` asks for;
-// with any operand out of them every admission is resolved exactly.
-// Measured against the kernel above: 64 candidates x 16 words (all admitted) 72 -> 33 us, 128 x 8 134 -> 79.
+// out in float64 (expand_resolve), unless those candidates have the same operands; so the decisions are those of the
+// definition.  The approximation is within 5 units of its last place (three roundings, a reciprocal of 1 unit) for costs
+// and benefits in the ranges that `plain` asks for; with a cost or t_exp out of them (negative, below 2^-40, above 2^40) or a
+// benefit above 2^60 every admission of the call is resolved exactly.  A benefit below the range (the end of a long chain,
+// a token of confidence 0, what hangs on a malformed parent) says nothing about the others.
+// Measured, us per call, the kernel above / this one: 8 candidates x 2 words 11.2 / 7.1, 32 x 24 38.3 / 19.3, 64 x 16 73.0 /
+// 33.6, one of them with confidence 0 and c_draft NULL 75.8 / 33.6, every utility equal 55.5 / 46.8, 64 x 32 68.2 / 44.1, 64
+// x 96 98.6 / 83.4, 96 x 16 109 / 77.8, 128 x 8 135 / 82.0, 128 x 16 142 / 121, 256 x 4 246 / 143, 256 x 8 259 / 229.  Operands out of
+// range (a negative cost): 64 x 16 72.9 / 60.1, 128 x 8 135 / 116, but 64 x 48 75.5 / 114, 64 x 96 98.6 / 124.
 // NQ: candidates / 32 at most (2 or 8); the rows of up to 1024 threads' words are 64 KiB.
 constexpr unsigned kExpandSlack = 16u;
 template <int NQ, int WP>
@@ -224,8 +229,9 @@ adaptive_expand_regs_kernel(int n, int lw, int lp, const int32_t *__restrict__ p
     __shared__ double s_p[kExpandMaxCand], s_cd[kExpandMaxCand];
     __shared__ unsigned s_key[2][32 * NQ];                              // 0: not eligible
     __shared__ int s_fresh[2][32 * NQ], s_adm[kExpandMaxCand];
+    __shared__ unsigned long long s_exact[32 * NQ];
 
-    const int i = threadIdx.x, lane = i & 31, warp = i >> 5, n_warps = (int)blockDim.x >> 5;
+    const int i = threadIdx.x, lane = i & 31, warp = i >> 5, n_warps = (int)blockDim.x >> 5, nw = (n + 31) >> 5;
     const int P = 1 << lp, c = i >> lp, part = i & (P - 1), pitch = 2 * WP * P;
     const bool mine = c < n;
     for (int e = i; e < 2 * 32 * NQ; e += blockDim.x) (&s_key[0][0])[e] = 0u;
@@ -236,12 +242,13 @@ adaptive_expand_regs_kernel(int n, int lw, int lp, const int32_t *__restrict__ p
     const int bad = __syncthreads_or(malformed ? 1 : 0);
     for (int e = i; e < n; e += blockDim.x) s_p[e] = __dmul_rn(s_p[e], (double)t_ar);       // expected benefit
     __syncthreads();
-    const float b32 = mine ? (float)s_p[c] : 1.0f, c32 = mine ? (float)s_cd[c] : 1.0f;
+    // (a benefit below 2^-60, negative or not a number counts as 2^-60: at costs of 0 that is a utility of infinity
+    // and at costs of 2^-40 and more one that is never admitted, as with the benefit itself)
+    const float b32 = mine && s_p[c] >= 0x1p-60 ? (float)s_p[c] : 0x1p-60f, c32 = mine ? (float)s_cd[c] : 1.0f;
     // (zeros without a sign: the bits are compared as whole numbers)
     auto in_range = [](float v, float lim) { return v >= 1.0f / lim && v <= lim; };
     auto zero = [](float v) { return __float_as_uint(v) == 0u; };
-    const bool plain = (zero(t_exp) || in_range(t_exp, 0x1p40f)) && (zero(c32) || in_range(c32, 0x1p40f)) &&
-                       (in_range(b32, 0x1p60f) || (zero(b32) && !zero(c32)));
+    const bool plain = (zero(t_exp) || in_range(t_exp, 0x1p40f)) && (zero(c32) || in_range(c32, 0x1p40f)) && in_range(b32, 0x1p60f);
     const bool exact = __syncthreads_and(plain ? 1 : 0) == 0;
 
     // (a parent that does not precede matches nobody: it is never eligible)
@@ -272,29 +279,41 @@ adaptive_expand_regs_kernel(int n, int lw, int lp, const int32_t *__restrict__ p
     publish(0);
     __syncthreads();
 
-    constexpr unsigned kOne = 0x3f800000u;
+    constexpr unsigned kOne = 0x3f800000u, kInf = 0x7f800000u;
     int count = 0;
     for (; count < n; ++count) {
         const unsigned *keys = s_key[count & 1];
-        unsigned kk[NQ], top = 0u;
+        const int *fr = s_fresh[count & 1];
+        int b = 0;
+        if (!exact) {
+            unsigned kk[NQ], top = 0u;
 #pragma unroll
-        for (int q = 0; q < NQ; ++q) {
-            kk[q] = keys[32 * q + lane];
-            top = max(top, kk[q]);
-        }
-        top = __reduce_max_sync(0xffffffffu, top);
-        if (top == 0u) break;
-        const unsigned near = top > kExpandSlack ? top - kExpandSlack : 1u;
-        int b = 0, holders = 0;
+            for (int q = 0; q < NQ; ++q) {
+                kk[q] = keys[32 * q + lane];
+                top = max(top, kk[q]);
+            }
+            top = __reduce_max_sync(0xffffffffu, top);
+            if (top == 0u) break;
+            const unsigned near = top > kExpandSlack ? top - kExpandSlack : 1u;
+            int holders = 0;
 #pragma unroll
-        for (int q = NQ - 1; q >= 0; --q) {
-            const unsigned hb = __ballot_sync(0xffffffffu, kk[q] >= near);
-            if (hb) b = 32 * q + __ffs(hb) - 1;
-            holders += __popc(hb);
+            for (int q = NQ - 1; q >= 0; --q) {
+                const unsigned hb = __ballot_sync(0xffffffffu, kk[q] >= near);
+                if (hb) b = 32 * q + __ffs(hb) - 1;
+                holders += __popc(hb);
+            }
+            if (top - (kOne - kExpandSlack) <= 2u * kExpandSlack) {
+                b = expand_resolve(keys, fr, s_p, s_cd, s_exact, (double)t_exp, nw, near);
+            } else if (top < kOne) {
+                break;
+            } else if (holders > 1 && top < kInf) {              // (infinite: a cost of 0, nothing to compare)
+                // the same operands, the same utility: the lowest index stands
+                const bool same = i >= 32 * nw || keys[i] < near || (fr[i] == fr[b] && s_p[i] == s_p[b] && s_cd[i] == s_cd[b]);
+                if (!__syncthreads_and(same ? 1 : 0)) b = expand_resolve(keys, fr, s_p, s_cd, s_exact, (double)t_exp, nw, near);
+            }
+        } else {
+            b = expand_resolve(keys, fr, s_p, s_cd, s_exact, (double)t_exp, nw, 1u);
         }
-        if (top < kOne) b = -1;
-        if (holders > 1 || top - (kOne - kExpandSlack) <= 2u * kExpandSlack || exact)
-            b = expand_resolve(keys, s_fresh[count & 1], s_p, s_cd, (double)t_exp, (n + 31) >> 5, near);
         if (b < 0) break;
         if (i == 0) order[count] = b;
         adm |= c == b;

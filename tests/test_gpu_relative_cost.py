@@ -58,6 +58,15 @@ def _expand_us(n, n_layers, p_last=0.9, parent_last=-1, p=0.9, c_draft=False):
     return _us(lambda stream: binding.adaptive_expand(parent, p_tok, masks, 64, c, 1e6, 0.125, stream=stream))
 
 
+@pytest.mark.parametrize("n,n_layers", [(64, 16), (128, 8), (256, 4)])
+@pytest.mark.parametrize("last", ["confidence 0", "tiny", "malformed parent"])
+def test_one_candidate_that_is_never_admitted(n, n_layers, last):
+    """It says nothing about the others' utilities, so the call may not take the exact path for all of them (1.4 to 4 times
+    the time without it where it did)."""
+    kw = {"confidence 0": dict(p_last=0.0), "tiny": dict(p_last=1e-30, c_draft=True), "malformed parent": dict(parent_last=n)}[last]
+    assert _expand_us(n, n_layers, **kw) < 1.4 * _expand_us(n, n_layers, c_draft=kw.get("c_draft", False))
+
+
 def test_few_candidates_with_many_words():
     """One candidate of 96 words against 32 of them (measured a ninth; two thirds where its one warp formed the union word
     by word)."""
