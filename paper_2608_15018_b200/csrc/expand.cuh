@@ -213,12 +213,16 @@ __device__ __noinline__ int expand_resolve(const unsigned *keys, const int *fres
 // benefit above 2^60 every admission of the call is resolved exactly.  A benefit below the range (the end of a long chain,
 // a token of confidence 0, what hangs on a malformed parent) says nothing about the others.
 // Measured, us per call, the kernel above / this one: 8 candidates x 2 words 11.2 / 7.1, 32 x 24 38.3 / 19.3, 64 x 16 73.0 /
-// 33.6, one of them with confidence 0 and c_draft NULL 75.8 / 33.6, every utility equal 55.5 / 46.8, 64 x 32 68.2 / 44.1, 64
-// x 96 98.6 / 83.4, 96 x 16 109 / 77.8, 128 x 8 135 / 82.0, 128 x 16 142 / 121, 256 x 4 246 / 143, 256 x 8 259 / 229.  Operands out of
-// range (a negative cost): 64 x 16 72.9 / 60.1, 128 x 8 135 / 116, but 64 x 48 75.5 / 114, 64 x 96 98.6 / 124.
+// 33.6, one of them with confidence 0 and c_draft NULL 75.8 / 33.6, every utility equal 55.5 / 46.8, 64 x 32 68.2 / 43.0, 64
+// x 96 98.6 / 86.2, 96 x 16 109 / 79.9, 128 x 8 135 / 83.5, 128 x 16 142 / 121, 256 x 4 246 / 138, 256 x 8 259 / 215.  Operands out of
+// range (a negative cost): 64 x 16 72.9 / 60.1, 128 x 8 135 / 112, but 64 x 48 75.5 / 116, 64 x 96 98.6 / 129.
 // NQ: candidates / 32 at most (2 or 8); the rows of up to 1024 threads' words are 64 KiB.
+// SKIP: a candidate that brings nothing new changes nobody's remainder.  The branch holds back the loads behind it, so
+// it is for blocks of 512 threads and more and for more than 64 candidates, where the loads of all warps take longer than
+// their latency: 64 x 96, union full after a few admissions, 83.0 without / 46.6 with it (86.2 against 83.4 where
+// everything is new), 64 x 48 69.1 / 46.3; 64 x 16 33.7 / 26.6, but 33.6 / 37.6 where everything is new.
 constexpr unsigned kExpandSlack = 16u;
-template <int NQ, int WP>
+template <int NQ, int WP, bool SKIP>
 __global__ void __launch_bounds__(1024)
 adaptive_expand_regs_kernel(int n, int lw, int lp, const int32_t *__restrict__ parent, const float *__restrict__ p_tok,
                             const unsigned long long *__restrict__ masks, const float *__restrict__ c_draft, float t_ar,
@@ -318,16 +322,18 @@ adaptive_expand_regs_kernel(int n, int lw, int lp, const int32_t *__restrict__ p
         if (i == 0) order[count] = b;
         adm |= c == b;
         eligible |= my_par == b;
-        const ulonglong2 *rb = rows + b * (pitch >> 1) + part;
-        int gone = 0;
+        if (!SKIP || fr[b] != 0) {
+            const ulonglong2 *rb = rows + b * (pitch >> 1) + part;
+            int gone = 0;
 #pragma unroll
-        for (int j = 0; j < WP; ++j) {
-            const ulonglong2 nb = rb[j * P];
-            gone += __popcll(rem[j].x & nb.x) + __popcll(rem[j].y & nb.y);
-            rem[j].x &= ~nb.x;
-            rem[j].y &= ~nb.y;
+            for (int j = 0; j < WP; ++j) {
+                const ulonglong2 nb = rb[j * P];
+                gone += __popcll(rem[j].x & nb.x) + __popcll(rem[j].y & nb.y);
+                rem[j].x &= ~nb.x;
+                rem[j].y &= ~nb.y;
+            }
+            fresh -= over_parts(gone);
         }
-        fresh -= over_parts(gone);
         publish((count + 1) & 1);
         __syncthreads();
     }

@@ -1434,8 +1434,8 @@ int s2moe_adaptive_expand(int32_t n_cand, int32_t n_layers, int32_t n_experts, c
     if (n_cand > kExpandMaxCand || lw > kExpandMaxWords) return S2MOE_ERANGE;
     // Words in registers where two or four pairs per thread of at most 1024 hold them, above 64 candidates two per thread of
     // at most 512 (all warps look through all keys): measured, us per call, in registers / by the kernel below, 96
-    // candidates x 16 words 76.7 / 109, 128 x 16 118 / 142, 256 x 8 224 / 259; beyond the line 160 x 16 169 / 175, 96 x 24 121 / 109,
-    // 128 x 24 204 / 147, 256 x 16 396 / 277, with four pairs 96 x 48 147 / 127, 128 x 64 249 / 175, 160 x 24 204 / 185.
+    // candidates x 16 words 79.9 / 109, 128 x 16 121 / 142, 256 x 8 215 / 259; beyond the line 160 x 16 175 / 175, 96 x 24 125 / 109,
+    // 128 x 24 210 / 147, 256 x 16 408 / 277, with four pairs 96 x 48 147 / 127, 128 x 64 246 / 175, 160 x 24 203 / 185.
     const int pairs = (lw + 1) / 2;
     for (const int wp : {2, 4}) {
         int lp = 0;
@@ -1443,7 +1443,10 @@ int s2moe_adaptive_expand(int32_t n_cand, int32_t n_layers, int32_t n_experts, c
         if (lp > 5 || n_cand << lp > (n_cand <= 64 ? 1024 : 512) || (n_cand > 64 && wp > 2)) continue;
         const int threads = ((n_cand << lp) + 31) / 32 * 32;
         const size_t rows = sizeof(uint64_t) * (size_t)n_cand * (2 * wp << lp);
-        auto *kernel = n_cand > 64 ? adaptive_expand_regs_kernel<8, 2> : wp == 2 ? adaptive_expand_regs_kernel<2, 2> : adaptive_expand_regs_kernel<2, 4>;
+        const bool skip = threads >= 512;
+        auto *kernel = n_cand > 64 ? adaptive_expand_regs_kernel<8, 2, true>
+                       : wp == 2 ? (skip ? adaptive_expand_regs_kernel<2, 2, true> : adaptive_expand_regs_kernel<2, 2, false>)
+                                 : (skip ? adaptive_expand_regs_kernel<2, 4, true> : adaptive_expand_regs_kernel<2, 4, false>);
         if (rows > 32 * 1024 &&
             cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kExpandMaxSmem) != cudaSuccess)
             return S2MOE_ECUDA;
