@@ -181,7 +181,7 @@ def _dptr(t: Optional[torch.Tensor]) -> Optional[int]:
 
 # The current stream's handle without a Stream object around it: 0.1 us instead of 3.5 us per call
 _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
-# (the device without the check that CUDA is initialised, which whoever has a CUDA tensor has behind him)
+# (the device without the check that CUDA is initialised: the tensors of a call are on it already)
 _device = getattr(torch._C, "_cuda_getDevice", torch.cuda.current_device)
 
 

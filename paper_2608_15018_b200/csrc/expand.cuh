@@ -78,8 +78,8 @@ __device__ __forceinline__ unsigned long long expand_key(double benefit, int fre
 // that decides an admission is float64 with every operation rounded on its own (no fused
 // multiply-add), so that the decisions are those of the plain definition.
 // Bound by latency: three block barriers and one float64 division (some 400 cycles) per admission.
-// Measured against every candidate counting all its words again for every admission: 64 candidates x
-// 16 words (all admitted) 98 -> 74 us, 160 x 96 770 -> 262 us.
+// Measured, us per call, where s2moe_adaptive_expand uses it: 96 candidates x 24 words 109, 128 x 64 175, 256 x 16 277, 160 x 96
+// 262 (770 with every candidate counting all its words again for every admission).
 // SMEM: the rows fit shared memory; else they are read from global memory.
 template <bool SMEM>
 __global__ void __launch_bounds__(kExpandThreads)

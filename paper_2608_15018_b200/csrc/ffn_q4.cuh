@@ -27,14 +27,15 @@
 //     issuer to notice, the MMAs and their completion, and the other groups work meanwhile.  With one group the schedulers
 //     idled that long in every unit, with two the groups fell into step and idled together;
 //   - weights and token tiles have a producer each: one thread for both needed 600 cycles per copy under that load, so
-//     weights arrived just as they were asked for although the ring has ten stages;
+//     weights arrived just as they were asked for although the ring had stages to spare;
 //   - a unit's entry in shared memory holds what the roles need (16 bytes and the row of the map), and what only some
 //     units need is a function of its own (inlined everywhere it pushes the loops out of the instruction cache).
 // A slot, and a stage of the ring (whose length is a multiple of the groups), belong to one group, so that whoever waits for
 // their barriers sees every phase: a barrier tells only odd phases from even ones.
-// Measured at the Mixtral shape, us per layer, with one group and one producer / now: 1 token 66.8 / 59.2, 8 tokens
-// 119.8 / 96.5, 16 130.3 / 104.7, 32 136.9 / 120, 64 158.9 / 155.2 (the weights alone: 31 at 1 token, 62 at 8 at the
-// measured copy rate).
+// Measured at the Mixtral shape, us per layer, with one group and one producer / now: 1 token 66.4 / 58.8, 8 tokens
+// 120.7 / 97.3, 16 132.6 / 107.0, 32 138.7 / 119.1, 64 159.4 / 151.7 (the weights alone: 31 at 1 token, 62 at 8 at the
+// measured copy rate).  Layers of a few units per CTA pay some 1 us for it (more warps to start, a unit takes its group of
+// four longer): 8 experts of 2048 x 1536, 8 tokens 28.4 / 29.6, 48 tokens 34.6 / 35.9; 128 of 2048 x 768, 8 tokens 37.7 / 38.2.
 //
 // Tried instead: the nibbles as binary16 subnormals n - 8 (9 instructions per 8 weights, exact), one
 // accumulator per block of 32 columns and the scales applied in fp32 behind the MMAs: eight accumulators a unit
@@ -46,7 +47,7 @@
 // before the mixing weights and the buckets, are enough for every unit but the epilogue's targets, so
 // the first projection streams while the gating ends.
 //
-// Warp roles (Q4Plan::threads): 0 weight producer; 1 MMA issuer; 2..5 epilogue; 7..9 converters; 10 watcher (polls
+// Warp roles (Q4Plan::threads): 0 weight producer; 1 MMA issuer; 2..5 epilogue; 6 none; 7..9 converters; 10 watcher (polls
 // the waves' second counters and publishes them in shared memory); 11 token producer; from 12 on dequantising.  Warps
 // 7..10 build the tables first.
 #pragma once
@@ -105,8 +106,8 @@ inline Q4Plan q4_make_plan(const Shape &sh, int B, int n_sm, bool early)
     // 4096 32 tokens 41.9 / 40.8.  Chains cut after half of every run, so that the accumulators stay two: 44.5 there.
     // Above 32 tokens an accumulator of 128 columns holds two chains of up to 64, or one of more (33 and more tokens).
     // Three groups of four warps up to 32 tokens, two of eight above (three slots do not fit).  Measured, us per layer at the
-    // Mixtral shape, three / two: 8 tokens 96 / 111, 16 tokens 105 / 120, 32 tokens 117 / 133; four-warp groups with a
-    // row's eight chunks loaded together 99 / - at 8, and two of them 172 against 164 at 64.
+    // Mixtral shape, three / two (with the chains cut, on one box): 8 tokens 96 / 111, 16 tokens 105 / 120, 32 tokens 117 /
+    // 133; four-warp groups with a row's eight chunks loaded together 99 / - at 8, and two of them 172 against 164 at 64.
     p.acc_cols = B <= 32 ? 64 : 128;
     p.groups = (512 - 2 * p.acc_cols) / 128;
     p.deq_warps = p.groups == 3 ? 4 : 8;
@@ -115,7 +116,10 @@ inline Q4Plan q4_make_plan(const Shape &sh, int B, int n_sm, bool early)
     // weights and scales have been read, and not only when the MMAs have completed.
     p.stages = (kTcMaxSmem - p.tab_bytes - 1024 - p.groups * kTcQ4KG * p.tokb) / kQ4StageBytes;
     if (p.stages > kTcMaxStages) p.stages = kTcMaxStages;
-    p.stages -= p.stages % p.groups;           // (a stage is always the same group's)
+    // (a stage is always the same group's: nine stages at most for three groups; where 8 or 7 become 6, at 17 to 32 tokens, the
+    // groups gain more, and with the largest tables, where 7 become 3, 256 experts of 1024 x 512, top 16, beside 4 shared ones
+    // take 77 us at 32 tokens as with one group and seven stages; at 64 tokens two stages for three cost 2 %, 117.2 / 115.0)
+    p.stages -= p.stages % p.groups;
     p.smem_bytes = p.tab_bytes + p.stages * kQ4StageBytes + p.groups * kTcQ4KG * p.tokb + 1024;
     // (the SM that runs the gating is taken until the routing kernel ends: its CTA would start last with a
     // full share)

@@ -1,5 +1,5 @@
-"""The admission kernel at the edges of its layout (one lane per candidate up to 32 and several words
-per lane, several passes over the candidates, rows in shared memory and rows too large for it):
+"""The admission kernels at the edges of their layouts (words in registers, rows in shared memory, rows too large for
+it; test_gpu_expansion_close has the layouts in registers one by one):
 bit-exact against the oracle, through the check of test_gpu_expansion."""
 import pytest
 

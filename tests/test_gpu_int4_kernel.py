@@ -1,6 +1,6 @@
 """The block-int4 expert kernel (kernel plan 3) at the sizes where it can go wrong: the smallest widths (one
-stage per row block, one unit per run), token counts around the padding steps and where two MMA issuers
-give way to one, shared experts, few and many experts, more units per CTA than its table holds, with the
+stage per row block, one unit per run), token counts around the padding steps and where three groups of
+dequantising warps give way to two, shared experts, few and many experts, more units per CTA than its table holds, with the
 early start and without.  Tolerance: the library's own for block-int4 weights."""
 import pytest
 
@@ -46,7 +46,7 @@ def test_row_blocks_without_tokens(B):
 
 
 def test_largest_tables():
-    """All limits at once: the tables leave three stages of the ring."""
+    """All limits at once: the tables leave two stages of the ring, one per group of dequantising warps."""
     wl = CONFIGS["cfg4"].with_(d_model=512, d_ff=256, d_ff_shared=512, n_shared=4, shared_gate=True, n_experts=256, top_k=16,
                                cap=256, sigma=1.0, n_layers=1)
     rep, _ = run_case(wl, n_tokens=64, plan=3, tok_list=list(range(0, 64, 7)))
