@@ -34,8 +34,8 @@
 // their barriers sees every phase: a barrier tells only odd phases from even ones.
 // Measured at the Mixtral shape, us per layer, with one group and one producer / now: 1 token 66.4 / 58.8, 8 tokens
 // 120.7 / 97.3, 16 132.6 / 107.0, 32 138.7 / 119.1, 64 159.4 / 151.7 (the weights alone: 31 at 1 token, 62 at 8 at the
-// measured copy rate).  Layers of a few units per CTA pay some 1 us for it (more warps to start, a unit takes its group of
-// four longer): 8 experts of 2048 x 1536, 8 tokens 28.4 / 29.6, 48 tokens 34.6 / 35.9; 128 of 2048 x 768, 8 tokens 37.7 / 38.2.
+// measured copy rate).  Layers of a few units per CTA pay 0.5 to 1.3 us for it (more warps to start, a unit takes its group of
+// four longer): 8 experts of 2048 x 1536, 8 tokens 28.5 / 29.0, 48 tokens 34.6 / 35.9; 128 of 2048 x 768, 8 tokens 38.7 / 38.5.
 //
 // Tried instead: the nibbles as binary16 subnormals n - 8 (9 instructions per 8 weights, exact), one
 // accumulator per block of 32 columns and the scales applied in fp32 behind the MMAs: eight accumulators a unit
@@ -179,7 +179,7 @@ ffn_q4_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ Q4Arg
 {
     extern __shared__ __align__(1024) uint8_t q4_smem[];
     __shared__ __align__(8) uint64_t full_bar[kTcMaxStages], empty_bar[kTcMaxStages], a_full[kQ4MaxGroups], a_empty[kQ4MaxGroups];
-    __shared__ __align__(8) uint64_t acc_full[2], acc_empty[2], conv_go[kQ4MaxWaves], tab_bar[2], cv_bar;
+    __shared__ __align__(8) uint64_t acc_full[2], acc_empty[2], conv_go[kQ4MaxWaves], tab_bar[2], cv_bar, tok_go;
     __shared__ uint32_t s_tmem;
     __shared__ int s_flag, s_n_units, s_split, s_n_active;
     __shared__ Q4Segments s_seg;
@@ -225,7 +225,10 @@ ffn_q4_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ Q4Arg
             mbar_init(&conv_go[lane], 4);
             s_ready[lane] = 0;
         }
-        if (lane == 0) mbar_init(&cv_bar, 3);
+        if (lane == 0) {
+            mbar_init(&cv_bar, 3);
+            mbar_init(&tok_go, 1);
+        }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     } else if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)), "r"(512u) : "memory");
@@ -399,15 +402,19 @@ ffn_q4_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ Q4Arg
                 mbar_expect_tx(&full_bar[s], kQ4StageBytes);
                 tma_load_2d_stream(stage, map, (int)un.w * 32, row, &full_bar[s], wpolicy);
                 tma_load_2d(stage + kTcQ4KG * kTcQ4Packed, map + 9, (int)un.w * 2, row, &full_bar[s]);
+                if (i == 0) mbar_arrive(&tok_go);
                 tc_ring_next(s, ring_par, S);
             }
+            if (n_units == 0) mbar_arrive(&tok_go);
         }
     } else if (warp == 11) {
         // ------------------------------------------------------------------ token producer
         // The token tiles go into the set of the A operand's slot they are used with (free once the MMAs that read
         // it have completed; their bytes are counted by the barrier the dequantising warps arrive on, so that an MMA
-        // issuer waits once), in the second projection only when their wave's activations are written.
-        if (tc_elect() && tab_wait(0)) {
+        // issuer waits once), in the second projection only when their wave's activations are written.  The first ones go out
+        // behind the first weights, which take longer to be of use (0.3 to 0.5 us of a layer of a few units per CTA: 8 experts of
+        // 4096 x 1024, 8 tokens 30.9 -> 30.7 us, of 2048 x 768 27.4 -> 26.9; Mixtral shape +-0.1 %).
+        if (tc_elect() && mbar_wait(&tok_go, 0)) {             // (the tables are written: the weight producer has waited for them)
             const int n_units = s_n_units, split = s_split;
             int ta = 0, ready_w = 0;
             uint32_t t_par = 1;
